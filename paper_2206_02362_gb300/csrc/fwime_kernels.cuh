@@ -19,12 +19,8 @@ namespace fwk {
 
 constexpr int STRIP = 128;      // x-points per warp in the stencil kernel (32 lanes x float4)
 constexpr int PROP_WARPS = 4;   // warps per CTA in the stencil kernel
-constexpr int EXT_TX = 128;     // x-points per CTA in the scatter / imaging kernels
+constexpr int EXT_TX = 128;     // x-points per CTA in the generic scatter kernel
 constexpr int MAX_NH = 201;     // largest supported number of subsurface offsets
-#ifndef FWIME_EXT_STAGES
-#define FWIME_EXT_STAGES 6
-#endif
-constexpr int EXT_STAGES = FWIME_EXT_STAGES;   // cp.async pipeline depth of the imaging kernels (even, >= 4)
 
 // status bits latched by kernels
 constexpr int ST_CFL = 1;
@@ -150,7 +146,7 @@ struct ExtArgs {
     int accumulate;
 };
 
-enum { IMG_EXT = 0, IMG_CONTRACT = 1, IMG_LOCAL = 2 };
+enum { IMG_EXT = 0, IMG_LOCAL = 2 };
 
 struct ImgArgs {
     int NXP, nh, hm, S, npair, n0;
@@ -158,11 +154,10 @@ struct ImgArgs {
     int z_lo, z_hi, x_lo, x_hi;
     RingRef D;                     // source-side field  D(x - h)
     RingRef L;                     // receiver-side field L(x + h)
-    RingRef M2;                    // IMG_LOCAL: second adjoint field (may be null base)
-    RingRef Ds;                    // IMG_LOCAL: scattered D2t field (may be null base)
-    float alpha;                   // IMG_LOCAL: weight of D * L
-    const float *pt;               // IMG_CONTRACT: p~ padded [nh][P]
-    float *img;                    // IMG_EXT: [nh][P]; others: [P]
+    RingRef M2;                    // local terms: second adjoint field (null base together with Ds, or both set)
+    RingRef Ds;                    // local terms: scattered D2t field
+    float alpha;                   // local terms: weight of D * L
+    float *img;                    // IMG_EXT: [nh][P]; IMG_LOCAL: [P]
     float *img_local;              // IMG_EXT, optional: [P] += the IMG_LOCAL terms (alpha D L + D M2 + Ds L)
 };
 

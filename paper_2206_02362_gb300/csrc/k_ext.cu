@@ -527,564 +527,4 @@ cudaError_t launch_scatter(const ExtArgs &a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ imaging
-
-// ---------------------------------------------------------- imaging, parity-split blocks (default path)
-//
-// I(x, h) += D(x - h) L(x + h).  With u = x - h and w = x + h (same parity) the products of one
-// (step, shot) pair are D(u) L(w) over the band |w - u| <= 2 HM; in the index of one parity,
-// u = ub + par + 2 ut and w = ub + par + 2 wt, the band is |wt - ut| <= HM.  A lane owns 8
-// consecutive ut and a window of 4 nl consecutive wt starting lo after its first ut (a task may
-// have two windows): 8 + 4 nl loaded samples serve up to 32 nl multiply-adds, products outside the
-// band being dropped at compile time.  The windows of the NT tasks (one warp each) tile the band
-// exactly, so every (x, h) is accumulated by exactly one lane of one CTA (a CTA covers 256
-// consecutive u and every offset).  Rows are copied de-interleaved by parity (4-byte cp.async);
-// the 16-byte chunks of a parity array are stored alternately in two halves so that the lanes'
-// vector loads, 8 floats apart, hit distinct banks, and so do the copies.
-struct ImgTask {
-    int lo1, nl1, lo2, nl2;        // windows [lo, lo + 4 nl) of wt - (the lane's first ut); nl2 = 0: none
-};
-
-__host__ __device__ constexpr int img_ntask(int nh)
-{
-    return nh <= 5 ? 1 : nh == 11 ? 2 : nh == 21 ? 3 : nh == 31 ? 4 : 5;
-}
-__host__ __device__ constexpr ImgTask img_task(int nh, int k)
-{
-    return nh == 1 ? ImgTask{0, 2, 0, 0}
-         : nh <= 5 ? ImgTask{-4, 4, 0, 0}
-         : nh == 11 ? (k == 0 ? ImgTask{0, 2, 0, 0} : ImgTask{-8, 2, 8, 2})
-         : nh == 21 ? (k == 0 ? ImgTask{-16, 4, 0, 0} : k == 1 ? ImgTask{0, 2, 0, 0} : ImgTask{8, 4, 0, 0})
-         : nh == 31 ? (k == 0 ? ImgTask{-8, 2, 0, 0} : k == 1 ? ImgTask{0, 2, 0, 0}
-                       : k == 2 ? ImgTask{8, 2, 0, 0} : ImgTask{-16, 2, 16, 2})
-         : (k == 0 ? ImgTask{-24, 4, 0, 0} : k == 1 ? ImgTask{-8, 2, 0, 0} : k == 2 ? ImgTask{0, 2, 0, 0}
-            : k == 3 ? ImgTask{8, 2, 0, 0} : ImgTask{16, 4, 0, 0});
-}
-// every wt - ut offset the band needs, -HM .. 7 + HM, lies in exactly one window; none overlap
-__host__ __device__ constexpr bool img_tasks_tile(int nh)
-{
-    const int hm = (nh - 1) / 2;
-    for (int o = -64; o < 72; ++o) {
-        int n = 0;
-        for (int k = 0; k < img_ntask(nh); ++k) {
-            const ImgTask t = img_task(nh, k);
-            n += (o >= t.lo1 && o < t.lo1 + 4 * t.nl1) + (t.nl2 > 0 && o >= t.lo2 && o < t.lo2 + 4 * t.nl2);
-        }
-        if (n > 1 || (o >= -hm && o <= 7 + hm && n != 1)) return false;
-    }
-    return true;
-}
-static_assert(img_tasks_tile(1) && img_tasks_tile(3) && img_tasks_tile(5) && img_tasks_tile(11) &&
-              img_tasks_tile(21) && img_tasks_tile(31) && img_tasks_tile(41), "imaging tasks must tile the band");
-
-// the task whose first window holds offset 0 for all 8 of a lane's ut (wt - ut = 0): it owns h = 0
-__host__ __device__ constexpr int img_h0_task(int nh)
-{
-    for (int k = 0; k < img_ntask(nh); ++k) {
-        const ImgTask t = img_task(nh, k);
-        if (t.lo1 <= 0 && t.lo1 + 4 * t.nl1 > 7) return k;
-    }
-    return -1;
-}
-static_assert(img_h0_task(1) >= 0 && img_h0_task(3) >= 0 && img_h0_task(5) >= 0 && img_h0_task(11) >= 0 &&
-              img_h0_task(21) >= 0 && img_h0_task(31) >= 0 && img_h0_task(41) >= 0, "h = 0 in one first window");
-
-__host__ __device__ constexpr int img_hc(int len)     // chunk pairs of a parity array (== 2 mod 8: no conflicts)
-{
-    int h = 2 * ((len + 15) / 16);
-    while (h % 8 != 2) ++h;
-    return h;
-}
-
-template <int NH>
-struct ImgShape {
-    static constexpr int HM = (NH - 1) / 2;
-    static constexpr int NT = img_ntask(NH);
-    static constexpr int TX = 32 * NT;
-    static constexpr int lo_min()
-    {
-        int m = 1 << 20;
-        for (int k = 0; k < NT; ++k) {
-            const ImgTask t = img_task(NH, k);
-            m = t.lo1 < m ? t.lo1 : m;
-            if (t.nl2 > 0) m = t.lo2 < m ? t.lo2 : m;
-        }
-        return m;
-    }
-    static constexpr int hi_max()
-    {
-        int m = -(1 << 20);
-        for (int k = 0; k < NT; ++k) {
-            const ImgTask t = img_task(NH, k);
-            m = t.lo1 + 4 * t.nl1 > m ? t.lo1 + 4 * t.nl1 : m;
-            if (t.nl2 > 0) m = t.lo2 + 4 * t.nl2 > m ? t.lo2 + 4 * t.nl2 : m;
-        }
-        return m;
-    }
-    static constexpr int LO = lo_min();
-    static constexpr int UT = 128;                           // ut per parity per CTA (16 lanes x 8)
-    static constexpr int LD = UT;                            // D samples per parity
-    static constexpr int LL = UT - 8 + hi_max() - LO;        // L samples per parity: wt in [LO, UT - 8 + hi)
-    static constexpr int HCD = img_hc(LD), HCL = img_hc(LL);
-    static constexpr int OFFD = (8 * HCD + 31) / 32 * 32 + 16, OFFL = (8 * HCL + 31) / 32 * 32 + 16;
-    static constexpr int REGD = OFFD + 8 * HCD;              // D region (floats); the L region follows
-    static constexpr int STG = (REGD + OFFL + 8 * HCL + 3) / 4 * 4;
-    // with the local terms two more D-shaped regions follow (second adjoint field, scattered D2t)
-    static constexpr int STGL = STG + 2 * REGD;
-    static constexpr int NCD = (2 * LD + TX - 1) / TX, NCL = (2 * LL + TX - 1) / TX;
-    static constexpr size_t SMEM = (size_t)EXT_STAGES * STG * sizeof(float);
-    static constexpr size_t SMEML = (size_t)EXT_STAGES * STGL * sizeof(float);
-    static_assert(REGD % 8 == 0 && LO % 4 == 0, "alignment");
-};
-
-// one task's share of a pair: products of the lane's 8 D samples with its L window(s).  LOCAL: the task
-// that owns h = 0 also sums the local terms D M2 + Ds L at its 8 points (x = u, where it holds D(u) and L(u))
-template <int NH, int K, bool LOCAL = false>
-struct ImgTaskBody {
-    static constexpr ImgTask T = img_task(NH, K);
-    static constexpr bool LH0 = LOCAL && K == img_h0_task(NH);
-    static constexpr int HM = (NH - 1) / 2;
-    static constexpr int W1 = 4 * T.nl1, W2 = T.nl2 > 0 ? 4 * T.nl2 : 1;
-    // packed two-lane form: the products of one D sample with the L pair (2 q, 2 q + 1) of a window
-    // accumulate in one register pair when both lie in the band; the band's edge entries whose
-    // partner lies outside stay scalar
-    static constexpr bool PACK = FWIME_IMG_F32X2 && NH != FWIME_IMG_UNPACKED_NH;   // measured slower at nh 31
-    static constexpr int P1 = PACK ? W1 / 2 : 1, P2 = PACK && W2 >= 2 ? W2 / 2 : 1;
-    float acc1[8][W1], acc2[8][W2];
-    f32x2 pac1[8][P1], pac2[8][P2];
-    float loc[LH0 ? 8 : 1];
-
-    __device__ __forceinline__ static constexpr bool in1(int i, int j) { return (T.lo1 + j - i) <= HM && (T.lo1 + j - i) >= -HM; }
-    __device__ __forceinline__ static constexpr bool in2(int i, int j)
-    {
-        return T.nl2 > 0 && (T.lo2 + j - i) <= HM && (T.lo2 + j - i) >= -HM;
-    }
-    // entry (i, j) accumulates in the pair (i, j / 2)
-    __device__ __forceinline__ static constexpr bool pk1(int i, int j) { return PACK && in1(i, j & ~1) && in1(i, j | 1); }
-    __device__ __forceinline__ static constexpr bool pk2(int i, int j) { return PACK && in2(i, j & ~1) && in2(i, j | 1); }
-    __device__ __forceinline__ void zero()
-    {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-#pragma unroll
-            for (int j = 0; j < W1; ++j) acc1[i][j] = 0.f;
-#pragma unroll
-            for (int j = 0; j < W2; ++j) acc2[i][j] = 0.f;
-#pragma unroll
-            for (int q = 0; q < P1; ++q) pac1[i][q] = pk(0.f, 0.f);
-#pragma unroll
-            for (int q = 0; q < P2; ++q) pac2[i][q] = pk(0.f, 0.f);
-        }
-#pragma unroll
-        for (int i = 0; i < (LH0 ? 8 : 1); ++i) loc[i] = 0.f;
-    }
-    // loads the lane's L window [8 b + LOW, 8 b + LOW + 4 NL) of wt: chunks c0 + q of the L region
-    // (which starts at wt = LO), chunk c at slot (c & 1) hcl + (c >> 1)
-    template <int LOW, int NL>
-    __device__ __forceinline__ static void load_window(float (&lv)[4 * NL], const float *sl, int b, int hcl)
-    {
-        constexpr int c0 = (LOW - ImgShape<NH>::LO) / 4;
-#pragma unroll
-        for (int q = 0; q < NL; ++q) {
-            const int c = c0 + q;
-            const float4 v = *reinterpret_cast<const float4 *>(sl + 4 * ((c & 1) * hcl + b + (c >> 1)));
-            lv[4 * q] = v.x; lv[4 * q + 1] = v.y; lv[4 * q + 2] = v.z; lv[4 * q + 3] = v.w;
-        }
-    }
-    // the lane's 8 samples of a D-shaped region (its ut = 8 b .. 8 b + 7 of its parity)
-    __device__ __forceinline__ static void load8(float (&v)[8], const float *sd, int b)
-    {
-        const float4 d0 = *reinterpret_cast<const float4 *>(sd + 4 * b);
-        const float4 d1 = *reinterpret_cast<const float4 *>(sd + 4 * (ImgShape<NH>::HCD + b));
-        v[0] = d0.x; v[1] = d0.y; v[2] = d0.z; v[3] = d0.w;
-        v[4] = d1.x; v[5] = d1.y; v[6] = d1.z; v[7] = d1.w;
-    }
-    // sm2, sds: the lane's parity array of the second adjoint field and the scattered D2t (LOCAL only)
-    __device__ __forceinline__ void pair(const float *sd, const float *sl, int b, const float *sm2 = nullptr,
-                                         const float *sds = nullptr)
-    {
-        using Sh = ImgShape<NH>;
-        float dv[8];
-        load8(dv, sd, b);
-        float l1[W1];
-        load_window<T.lo1, T.nl1>(l1, sl, b, Sh::HCL);
-        if constexpr (LH0) {   // x = u_i: D(u_i) = dv[i], L(u_i) = l1[i - lo1]
-            float mv[8], sv[8];
-            load8(mv, sm2, b);
-            load8(sv, sds, b);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) loc[i] = fmaf(sv[i], l1[i - T.lo1], fmaf(dv[i], mv[i], loc[i]));
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const f32x2 dd = pk(dv[i], dv[i]);
-#pragma unroll
-            for (int j = 0; j < W1; ++j) {
-                if (pk1(i, j)) {
-                    if (!(j & 1)) pac1[i][j / 2] = fma2(dd, pk(l1[j], l1[j + 1]), pac1[i][j / 2]);
-                } else if (in1(i, j)) {
-                    acc1[i][j] = fmaf(dv[i], l1[j], acc1[i][j]);
-                }
-            }
-        }
-        if constexpr (T.nl2 > 0) {
-            float l2[W2];
-            load_window<T.lo2, (T.nl2 > 0 ? T.nl2 : 1)>(l2, sl, b, Sh::HCL);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const f32x2 dd = pk(dv[i], dv[i]);
-#pragma unroll
-                for (int j = 0; j < W2; ++j) {
-                    if (pk2(i, j)) {
-                        if (!(j & 1)) pac2[i][j / 2] = fma2(dd, pk(l2[j], l2[j + 1]), pac2[i][j / 2]);
-                    } else if (in2(i, j)) {
-                        acc2[i][j] = fmaf(dv[i], l2[j], acc2[i][j]);
-                    }
-                }
-            }
-        }
-    }
-    __device__ __forceinline__ float val1(int i, int j) const
-    {
-        if (pk1(i, j)) {
-            float lo, hi;
-            upk(pac1[i][(j / 2) % P1], lo, hi);
-            return (j & 1) ? hi : lo;
-        }
-        return acc1[i][j];
-    }
-    __device__ __forceinline__ float val2(int i, int j) const
-    {
-        if (pk2(i, j)) {
-            float lo, hi;
-            upk(pac2[i][(j / 2) % P2], lo, hi);
-            return (j & 1) ? hi : lo;
-        }
-        return acc2[i][j];
-    }
-    // adds the accumulators into img at x = x1 + i + o, h = o - i (o = lo + j), x1 = the lane's
-    // first u + its first ut offset; only physical columns [x_lo, x_hi).  LOCAL: img_local at x = x1 + 2 i
-    // gains alpha x (its h = 0 sum of D L) + its local terms
-    __device__ __forceinline__ void store(const ImgArgs &a, long long rowoff, int x1)
-    {
-        if constexpr (LH0) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int x = x1 + 2 * i;
-                if (x >= a.x_lo && x < a.x_hi)
-                    a.img_local[rowoff + x] += fmaf(a.alpha, val1(i, i - T.lo1), loc[i]);
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-#pragma unroll
-            for (int j = 0; j < W1; ++j) {
-                if (in1(i, j)) {
-                    const int x = x1 + i + T.lo1 + j;
-                    if (x >= a.x_lo && x < a.x_hi) a.img[(T.lo1 + j - i + HM) * a.P + rowoff + x] += val1(i, j);
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < W2; ++j) {
-                if (in2(i, j)) {
-                    const int x = x1 + i + T.lo2 + j;
-                    if (x >= a.x_lo && x < a.x_hi) a.img[(T.lo2 + j - i + HM) * a.P + rowoff + x] += val2(i, j);
-                }
-            }
-        }
-    }
-};
-
-// block-wide barrier that warps may reach from different code (each warp runs its own task's
-// instantiation of the same pipeline): the non-.aligned form of bar.sync
-__device__ __forceinline__ void cta_barrier() { asm volatile("barrier.sync 0;\n" ::: "memory"); }
-
-template <int NH, int K, bool LOCAL = false>
-__device__ __forceinline__ void img_task_run(const ImgArgs &a, int u_lo, float *sm, int lane)
-{
-    using Sh = ImgShape<NH>;
-    constexpr int NS = EXT_STAGES;
-    constexpr int STG = LOCAL ? Sh::STGL : Sh::STG;   // floats per stage
-    constexpr unsigned MOFF = 4u * Sh::STG, SOFF = 4u * (Sh::STG + Sh::REGD);   // bytes to the local regions
-    const int Z = a.z_lo + blockIdx.y;
-    const long long rowoff = (long long)Z * a.NXP;
-    const int ub = u_lo + 256 * blockIdx.x;         // even
-    const int t = threadIdx.x;
-    const int par = lane >> 4, b = lane & 15;
-    // copy plan: thread t copies window samples n = t + TX c; sample n of a window goes to parity n & 1,
-    // index k = n >> 1, chunk k >> 2 stored at slot (chunk & 1) HC + (chunk >> 1)
-    const int cw = (t & 1), ch = (t >> 3) & 1, cp = (t >> 4), ce = (t >> 1) & 3;
-    const unsigned sbase = static_cast<unsigned>(__cvta_generic_to_shared(sm));
-    const unsigned dD = sbase + 4u * (cw * Sh::OFFD + 4 * (ch * Sh::HCD + cp) + ce);
-    const unsigned dL = sbase + 4u * (Sh::REGD + cw * Sh::OFFL + 4 * (ch * Sh::HCL + cp) + ce);
-    constexpr unsigned CSTEP = 4u * 8u * Sh::NT;     // bytes between copies c and c + 1 (TX / 16 chunk pairs)
-    const int colD = ub + t, colL = ub + 2 * Sh::LO + t;
-    // all copied columns, [ub + 2 LO, ub + 2 LO + 2 LL) (which contains the D window), inside the row
-    const bool interior = ub + 2 * Sh::LO >= 0 && ub + 2 * Sh::LO + 2 * Sh::LL <= a.NXP;
-    PairRow pd, pl, pm, ps;
-    pd.init(a.D, a.n0, a.S, a.P, rowoff);
-    pl.init(a.L, a.n0, a.S, a.P, rowoff);
-    if constexpr (LOCAL) {
-        pm.init(a.M2, a.n0, a.S, a.P, rowoff);
-        ps.init(a.Ds, a.n0, a.S, a.P, rowoff);
-    }
-    int st_in = 0, st_c = 0;
-    constexpr int FD = 2 * Sh::LD / Sh::TX, RD = 2 * Sh::LD - FD * Sh::TX;   // full copy rounds, remainder
-    constexpr int FL = 2 * Sh::LL / Sh::TX, RL = 2 * Sh::LL - FL * Sh::TX;
-    auto issue = [&](int p) {
-        if (p < a.npair) {
-            const unsigned so = 4u * st_in * STG;
-            if (interior) {
-                const float *sd = pd.row + colD, *sl = pl.row + colL;
-                cpa4_run<CSTEP, 4 * Sh::TX>(dD + so, sd, std::make_integer_sequence<int, FD>{});
-                if (RD > 0 && t < RD) cpa4_imm<CSTEP * FD, 4 * Sh::TX * FD>(dD + so, sd);
-                cpa4_run<CSTEP, 4 * Sh::TX>(dL + so, sl, std::make_integer_sequence<int, FL>{});
-                if (RL > 0 && t < RL) cpa4_imm<CSTEP * FL, 4 * Sh::TX * FL>(dL + so, sl);
-                if constexpr (LOCAL) {   // the second adjoint field and the scattered D2t: D's window and layout
-                    const float *smv = pm.row + colD, *ssv = ps.row + colD;
-                    cpa4_run<CSTEP, 4 * Sh::TX>(dD + so + MOFF, smv, std::make_integer_sequence<int, FD>{});
-                    if (RD > 0 && t < RD) cpa4_imm<CSTEP * FD, 4 * Sh::TX * FD>(dD + so + MOFF, smv);
-                    cpa4_run<CSTEP, 4 * Sh::TX>(dD + so + SOFF, ssv, std::make_integer_sequence<int, FD>{});
-                    if (RD > 0 && t < RD) cpa4_imm<CSTEP * FD, 4 * Sh::TX * FD>(dD + so + SOFF, ssv);
-                }
-            } else {
-#pragma unroll
-                for (int c = 0; c < Sh::NCD; ++c) {
-                    if (t + Sh::TX * c < 2 * Sh::LD) {
-                        const int col = colD + Sh::TX * c;
-                        const bool ok = col >= 0 && col < a.NXP;
-                        cpa4(dD + so + CSTEP * c, pd.row + (ok ? col : 0), ok);
-                        if constexpr (LOCAL) {
-                            cpa4(dD + so + MOFF + CSTEP * c, pm.row + (ok ? col : 0), ok);
-                            cpa4(dD + so + SOFF + CSTEP * c, ps.row + (ok ? col : 0), ok);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < Sh::NCL; ++c) {
-                    if (t + Sh::TX * c < 2 * Sh::LL) {
-                        const int col = colL + Sh::TX * c;
-                        const bool ok = col >= 0 && col < a.NXP;
-                        cpa4(dL + so + CSTEP * c, pl.row + (ok ? col : 0), ok);
-                    }
-                }
-            }
-            pd.next();
-            pl.next();
-            if constexpr (LOCAL) {
-                pm.next();
-                ps.next();
-            }
-        }
-        st_in = st_in + 1 == NS ? 0 : st_in + 1;
-        cpa_commit();
-    };
-    ImgTaskBody<NH, K, LOCAL> body;
-    body.zero();
-    // two pairs per barrier: the prologue fills NS - 2 stages; iteration p waits for pairs p and p + 1,
-    // then refills the stages of pairs p - 2 and p - 1, which every warp finished before the barrier
-#pragma unroll 1
-    for (int q = 0; q < NS - 2; ++q) issue(q);
-    for (int p = 0; p < a.npair; p += 2) {
-        cpa_wait<NS - 4>();
-        cta_barrier();
-        issue(p + NS - 2);
-        issue(p + NS - 1);
-        const float *s0 = sm + st_c * STG;
-        st_c = st_c + 1 == NS ? 0 : st_c + 1;
-        const float *s1 = sm + st_c * STG;
-        st_c = st_c + 1 == NS ? 0 : st_c + 1;
-        const int pd0 = par * Sh::OFFD;
-        body.pair(s0 + pd0, s0 + Sh::REGD + par * Sh::OFFL, b, s0 + Sh::STG + pd0, s0 + Sh::STG + Sh::REGD + pd0);
-        if (p + 1 < a.npair)
-            body.pair(s1 + pd0, s1 + Sh::REGD + par * Sh::OFFL, b, s1 + Sh::STG + pd0, s1 + Sh::STG + Sh::REGD + pd0);
-    }
-    cpa_wait<0>();
-    // u of the lane's first sample: ub + par + 16 b; x = (u + w) / 2 = ub + par + 16 b + i + o
-    body.store(a, rowoff, ub + par + 16 * b);
-}
-
-// LOCAL: also the local imaging terms (alpha D L + D M2 + Ds L at h = 0) into img_local, which otherwise
-// take their own k_image_local launch re-reading D and L
-template <int NH, bool LOCAL = false>
-__global__ void __launch_bounds__(ImgShape<NH>::TX, FWIME_IMG_MINB) k_image_ps(const ImgArgs a, int u_lo)
-{
-    extern __shared__ float4 sm4[];
-    float *sm = reinterpret_cast<float *>(sm4);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int NT = ImgShape<NH>::NT;
-    // warp-uniform dispatch: every warp runs the same pipeline (barriers included) with its own task
-    if (warp == 0) img_task_run<NH, 0, LOCAL>(a, u_lo, sm, lane);
-    if constexpr (NT > 1) if (warp == 1) img_task_run<NH, 1 % NT, LOCAL>(a, u_lo, sm, lane);
-    if constexpr (NT > 2) if (warp == 2) img_task_run<NH, 2 % NT, LOCAL>(a, u_lo, sm, lane);
-    if constexpr (NT > 3) if (warp == 3) img_task_run<NH, 3 % NT, LOCAL>(a, u_lo, sm, lane);
-    if constexpr (NT > 4) if (warp == 4) img_task_run<NH, 4 % NT, LOCAL>(a, u_lo, sm, lane);
-}
-
-
-// Generic-nh fallback: one point per thread, accumulators in shared memory.
-template <int MODE>
-__global__ void __launch_bounds__(EXT_TX) k_image_gen(const ImgArgs a)
-{
-    extern __shared__ float sm[];
-    const int nh = a.nh, hm = (nh - 1) / 2;
-    const int Z = a.z_lo + blockIdx.y;
-    const int x0 = a.x_lo + blockIdx.x * EXT_TX;
-    const int X = x0 + threadIdx.x;
-    const bool xin = X < a.x_hi;
-    const int span = EXT_TX + 2 * hm;
-    const int wbase = x0 - hm;
-    const long long rowoff = (long long)Z * a.NXP;
-    float *bd = sm, *bl = sm + span, *gacc = sm + 2 * span;
-    if (MODE == IMG_EXT)
-        for (int ih = 0; ih < nh; ++ih) gacc[ih * EXT_TX + threadIdx.x] = 0.f;
-    float cacc = 0.f;
-    for (int p = 0; p < a.npair; ++p) {
-        const int j = p / a.S, s = p % a.S, n = a.n0 + j;
-        const float *sd = a.D.base + ring_off(a.D, n, j) + (long long)s * a.P + rowoff;
-        const float *sl = a.L.base + ring_off(a.L, n, j) + (long long)s * a.P + rowoff;
-        __syncthreads();
-        for (int i = threadIdx.x; i < span; i += EXT_TX) {
-            const int xp = wbase + i;
-            const bool ok = xp >= 0 && xp < a.NXP;
-            bd[i] = ok ? __ldg(sd + xp) : 0.f;
-            bl[i] = ok ? __ldg(sl + xp) : 0.f;
-        }
-        __syncthreads();
-        const int t = threadIdx.x;
-        for (int ih = 0; ih < nh; ++ih) {
-            const float prod = bd[t + 2 * hm - ih] * bl[t + ih];
-            if (MODE == IMG_EXT) gacc[ih * EXT_TX + t] += prod;
-            else cacc = fmaf(xin ? __ldg(a.pt + ih * a.P + rowoff + X) : 0.f, prod, cacc);
-        }
-    }
-    if (!xin) return;
-    if (MODE == IMG_EXT)
-        for (int ih = 0; ih < nh; ++ih) a.img[ih * a.P + rowoff + X] += gacc[ih * EXT_TX + threadIdx.x];
-    else
-        a.img[rowoff + X] += cacc;
-}
-
-// pointwise (h = 0) accumulation: G += sum_pairs D (alpha L + M2) + Ds L, four independent
-// pairs in flight per thread (coalesced: consecutive threads, consecutive points).
-// Local imaging: a thread owns 4 consecutive columns (16-byte loads) of one row, a CTA 512 columns, so
-// every (step, shot) pair is read as long contiguous row segments; columns start at x_lo rounded down to
-// a multiple of 4 and only [x_lo, x_hi) is accumulated.
-constexpr int LOC_TX = 128;
-__device__ __forceinline__ float4 ldg4e(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
-__global__ void __launch_bounds__(LOC_TX) k_image_local(const ImgArgs a, int xa)
-{
-    const int Z = a.z_lo + blockIdx.y;
-    const int X = xa + 4 * (blockIdx.x * LOC_TX + threadIdx.x);
-    if (X >= a.x_hi) return;
-    const long long off = (long long)Z * a.NXP + X;
-    RingIt itd, itl, itm, its;
-    itd.init(a.D, a.n0, a.S, a.P, off);
-    itl.init(a.L, a.n0, a.S, a.P, off);
-    if (a.M2.base) itm.init(a.M2, a.n0, a.S, a.P, off);
-    if (a.Ds.base) its.init(a.Ds, a.n0, a.S, a.P, off);
-    float acc[4][4] = {};
-    for (int p = 0; p < a.npair; p += 4) {
-        // four independent pairs per iteration: their loads are all in flight together
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (p + u < a.npair) {
-                const float4 l = ldg4e(itl.ptr());
-                const float4 d = ldg4e(itd.ptr());
-                float4 m2 = make_float4(0.f, 0.f, 0.f, 0.f), ds = m2;
-                if (a.M2.base) { m2 = ldg4e(itm.ptr()); itm.next(); }
-                if (a.Ds.base) { ds = ldg4e(its.ptr()); its.next(); }
-                const float lv[4] = {l.x, l.y, l.z, l.w}, dv[4] = {d.x, d.y, d.z, d.w};
-                const float mv[4] = {m2.x, m2.y, m2.z, m2.w}, sv[4] = {ds.x, ds.y, ds.z, ds.w};
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    float tt = a.alpha * lv[c];
-                    if (a.M2.base) tt += mv[c];
-                    float r = dv[c] * tt;
-                    if (a.Ds.base) r = fmaf(sv[c], lv[c], r);
-                    acc[c][u] += r;
-                }
-                itd.next();
-                itl.next();
-            }
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-        if (X + c >= a.x_lo && X + c < a.x_hi) a.img[off + c] += (acc[c][0] + acc[c][1]) + (acc[c][2] + acc[c][3]);
-}
-
-template <int MODE>
-static cudaError_t launch_image_gen(const ImgArgs &a, cudaStream_t st)
-{
-    const int hm = (a.nh - 1) / 2;
-    size_t smem = (2 * (EXT_TX + 2 * hm) + (MODE == IMG_EXT ? a.nh * EXT_TX : 0)) * sizeof(float);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_image_gen<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    dim3 grid((a.x_hi - a.x_lo + EXT_TX - 1) / EXT_TX, a.z_hi - a.z_lo);
-    k_image_gen<MODE><<<grid, EXT_TX, smem, st>>>(a);
-    return cudaGetLastError();
-}
-
-template <int NH>
-static void launch_image_ps(const ImgArgs &a, cudaStream_t st)
-{
-    using Sh = ImgShape<NH>;
-    int u_lo = a.x_lo - Sh::HM;    // first u = x - h of the physical columns, made even
-    u_lo -= ((u_lo % 2) + 2) % 2;
-    dim3 grid((a.x_hi + Sh::HM - u_lo + 255) / 256, a.z_hi - a.z_lo);
-    // once per instantiation, before any launch (and any capture), thread-safe (function-local static)
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_image_ps<NH, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::SMEM) ==
-                cudaSuccess
-            ? cudaFuncSetAttribute(k_image_ps<NH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::SMEML)
-            : cudaErrorUnknown;
-    (void)attr;
-    if (a.img_local) k_image_ps<NH, true><<<grid, Sh::TX, Sh::SMEML, st>>>(a, u_lo);
-    else k_image_ps<NH, false><<<grid, Sh::TX, Sh::SMEM, st>>>(a, u_lo);
-}
-
-template <int MODE>
-static cudaError_t launch_image_mode(const ImgArgs &a, cudaStream_t st)
-{
-    if (MODE != IMG_EXT) return launch_image_gen<MODE>(a, st);
-    if (a.img_local && (a.nh != 1 && a.nh != 3 && a.nh != 5 && a.nh != 11 && a.nh != 21 && a.nh != 31 && a.nh != 41)) {
-        // generic nh: the extended image, then the local terms in their own kernel
-        ImgArgs e = a;
-        e.img_local = nullptr;
-        const cudaError_t err = launch_image_gen<MODE>(e, st);
-        if (err != cudaSuccess) return err;
-        ImgArgs l = a;
-        l.img = a.img_local;
-        l.img_local = nullptr;
-        return launch_image(l, IMG_LOCAL, st);
-    }
-    switch (a.nh) {
-    case 1: launch_image_ps<1>(a, st); break;
-    case 3: launch_image_ps<3>(a, st); break;
-    case 5: launch_image_ps<5>(a, st); break;
-    case 11: launch_image_ps<11>(a, st); break;
-    case 21: launch_image_ps<21>(a, st); break;
-    case 31: launch_image_ps<31>(a, st); break;
-    case 41: launch_image_ps<41>(a, st); break;
-    default: return launch_image_gen<MODE>(a, st);
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_image(const ImgArgs &a, int mode, cudaStream_t st)
-{
-    if (a.npair <= 0 || a.x_hi <= a.x_lo || a.z_hi <= a.z_lo) return cudaSuccess;
-    if (mode == IMG_LOCAL) {
-        const int xa = a.x_lo - a.x_lo % 4;   // 16-byte aligned: rows are NXP (a multiple of 32) floats apart
-        dim3 grid((a.x_hi - xa + 4 * LOC_TX - 1) / (4 * LOC_TX), a.z_hi - a.z_lo);
-        k_image_local<<<grid, LOC_TX, 0, st>>>(a, xa);
-        return cudaGetLastError();
-    }
-    if (mode == IMG_EXT) return launch_image_mode<IMG_EXT>(a, st);
-    return launch_image_mode<IMG_CONTRACT>(a, st);
-}
-
 }  // namespace fwk
