@@ -19,7 +19,6 @@ namespace fwk {
 
 constexpr int STRIP = 128;      // x-points per warp in the stencil kernel (32 lanes x float4)
 constexpr int PROP_WARPS = 4;   // warps per CTA in the stencil kernel
-constexpr int EXT_TX = 128;     // x-points per CTA in the generic scatter kernel
 constexpr int MAX_NH = 201;     // largest supported number of subsurface offsets
 
 // status bits latched by kernels

@@ -35,10 +35,10 @@ namespace fwk {
 // blocks, M = KA / 2 chunks apart, fall on distinct banks: an exclusive or with the line number for M = 2, 4,
 // nothing for M = 3.
 
-// NW warps per CTA; MINB resident CTAs the registers are capped for; G groups of two pairs in the copy ring
-template <int S_, int LB_, int KA_, int NW_, int MINB_, int G_>
+// NW warps per CTA; MINB (MINBL: with the local terms) resident CTAs the registers are capped for; G groups of PB pairs in the copy ring
+template <int S_, int LB_, int KA_, int NW_, int MINB_, int MINBL_, int G_, int PB_>
 struct ImgShape {
-    static constexpr int S = S_, LB = LB_, KA = KA_, NW = NW_, MINB = MINB_, G = G_;
+    static constexpr int S = S_, LB = LB_, KA = KA_, NW = NW_, MINB = MINB_, MINBL = MINBL_, G = G_, PB = PB_;
     static constexpr int C = S * LB, M = KA / 2, RL = LB / KA;
     static constexpr int NI = 32 / S * NW;                     // lane groups of a CTA
     static constexpr int TX = 32 * NW, UC = 2 * KA * NI;       // threads, columns u of a CTA and s
@@ -50,7 +50,7 @@ struct ImgShape {
     static constexpr int ND = (UC / 4 + SKEW / 2 + 7) / 8 * 8, NL = (UC / 4 + LB / 2 + 7 + 7) / 8 * 8;
     static constexpr int NM = (UC / 4 + 7 + 31) / 32 * 32;    // swz(c + NM) = swz(c) + NM
     template <bool LOCAL> static constexpr int stg() { return ND + NL + (LOCAL ? 2 * NM : 0); }   // chunks
-    template <bool LOCAL> static constexpr int smem_chunks() { return 2 * G * stg<LOCAL>(); }
+    template <bool LOCAL> static constexpr int smem_chunks() { return PB * G * stg<LOCAL>(); }
     static_assert(KA % 2 == 0 && LB % KA == 0 && M >= 2 && M <= 4 && UC % 32 == 0 && SKEW % HALIGN == 0, "block shape");
     __device__ __forceinline__ static int swz(int c)
     {
@@ -63,11 +63,12 @@ struct ImgShape {
 // LOCAL: also the local imaging terms (alpha D L + D M2 + Ds L at h = 0) into img_local, which otherwise
 // take their own k_image_local launch re-reading D and L
 template <class Sh, bool LOCAL>
-__global__ void __launch_bounds__(Sh::TX, Sh::MINB) k_image_band(const ImgArgs a, int u_lo, int ha, int h_lo, int h_hi)
+__global__ void __launch_bounds__(Sh::TX, LOCAL ? Sh::MINBL : Sh::MINB)
+    k_image_band(const ImgArgs a, int u_lo, int ha, int h_lo, int h_hi)
 {
     constexpr int S = Sh::S, KA = Sh::KA, LB = Sh::LB, M = Sh::M, C = Sh::C, TX = Sh::TX, UC = Sh::UC;
     constexpr int ND = Sh::ND, NL = Sh::NL, NM = Sh::NM;
-    constexpr int STG = Sh::template stg<LOCAL>(), NS = 2 * Sh::G;
+    constexpr int STG = Sh::template stg<LOCAL>(), NS = Sh::PB * Sh::G;
     extern __shared__ float4 sm4[];
     const int t = threadIdx.x, lane = t & 31;
     const int s = lane % S, ig = t / S;                         // lane group of the CTA
@@ -112,9 +113,9 @@ __global__ void __launch_bounds__(Sh::TX, Sh::MINB) k_image_band(const ImgArgs a
     };
     int p_in = 0, s_in = 0;
     unsigned so = 0;                                            // byte offset of the stage being filled
-    auto issue2 = [&]() {                                       // the next two pairs, one copy group
+    auto issue = [&]() {                                        // the next PB pairs, one copy group
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < Sh::PB; ++u) {
             if (p_in < a.npair) {
 #pragma unroll
                 for (int r = 0; r < RC; ++r)
@@ -163,8 +164,7 @@ __global__ void __launch_bounds__(Sh::TX, Sh::MINB) k_image_band(const ImgArgs a
     int o_l[NA];
 #pragma unroll
     for (int k = 0; k < NA; ++k) o_l[k] = 16 * Sh::swz(ND + M * (ig + k) + lsh);
-    auto pair = [&](int st, int half) {                         // st: byte offset of the iteration's two stages
-        const int so2 = half * 16 * STG;                        // compile time
+    auto pair = [&](int st, int so2) {                          // byte offset of the group's stages, of the pair's in it
         f32x2 d[KA];
 #pragma unroll
         for (int q = 0; q < M; ++q) {
@@ -190,19 +190,21 @@ __global__ void __launch_bounds__(Sh::TX, Sh::MINB) k_image_band(const ImgArgs a
             loc[r] = fma2(ld(o_lm[r] + 16 * NM), ld(o_ll[r]), fma2(ld(o_ld[r]), ld(o_lm[r]), loc[r]));
         }
     };
-    // two pairs per barrier; iteration p waits for its group, then refills the stages of the iteration before,
+    // PB pairs per barrier; an iteration waits for its group, then refills the stages of the iteration before,
     // which every warp has left
 #pragma unroll 1
-    for (int g = 0; g < Sh::G - 1; ++g) issue2();
+    for (int g = 0; g < Sh::G - 1; ++g) issue();
     int st_c = 0;
 #pragma unroll 1
-    for (int p = 0; p < a.npair; p += 2) {
+    for (int p = 0; p < a.npair; p += Sh::PB) {
         cpa_wait<Sh::G - 2>();
-        __syncthreads();
-        issue2();
-        pair(st_c, 0);
-        if (p + 1 < a.npair) pair(st_c, 1);
-        st_c = st_c + 32 * STG == 16 * NS * STG ? 0 : st_c + 32 * STG;
+        if constexpr (Sh::NW == 1) __syncwarp();
+        else __syncthreads();
+        issue();
+#pragma unroll
+        for (int u = 0; u < Sh::PB; ++u)
+            if (u == 0 || p + u < a.npair) pair(st_c, u * 16 * STG);
+        st_c = st_c + Sh::PB * 16 * STG == 16 * NS * STG ? 0 : st_c + Sh::PB * 16 * STG;
     }
     cpa_wait<0>();
     // Image update through shared memory, HP planes at a time: plane h of the CTA's columns u is the
@@ -269,24 +271,25 @@ static int launch_band(const ImgArgs &a, int h_lo, cudaStream_t st)
     return h_hi;
 }
 
-// Shapes <S, LB, KA, NW, MINB, G> by chunk size C = S LB, the best of about eight measured per size.  Smaller lane
-// blocks at 128 registers (16 warps per SM) beat larger ones with fewer shared loads per product: at C = 32 a
-// 4 x 16 block at 168 registers read 2.8 TB/s against 4.1, since the kernel waits on fixed latencies, not on one
-// unit (FMA pipe 46 %, shared memory 57 %, DRAM 53 %, issue slots 55 %).  Algorithmic GB/s of a segment's launch
-// against the parity-split kernel before (Marmousi2-shaped nh 21, North-Sea-shaped nh 31 with the local terms,
-// Salt-shaped nh 41 with them): 3548 -> 4737, 2554 -> 5518, 1335 -> 1934 (56 pairs per launch; 3659 with 256).
-// Another nh had a generic kernel (101 offsets: 176 -> 419 GB/s).
+// Shapes <S, LB, KA, NW, MINB, MINBL, G, PB> by chunk size C = S LB, the best of about twenty measured per size.
+// Small lane blocks at 128 registers (16 warps per SM) beat larger ones with fewer shared loads per product: at
+// C = 32 a 4 x 16 block at 168 registers read 2.8 TB/s against 4.1, since the kernel waits on fixed latencies, not
+// on one unit (FMA pipe 46 %, shared memory 57 %, DRAM 53 %, issue slots 55 %).  Two warps per CTA beat four (the
+// barrier couples them: C = 24 4735 -> 4970 GB/s) and one (more window per column).  Algorithmic GB/s of a
+// segment's launch against the parity-split kernel before (Marmousi2-shaped nh 21, North-Sea-shaped nh 31 with the
+// local terms, Salt-shaped nh 41 with them): 3548 -> 4970, 2554 -> 5815, 1335 -> 1893 (56 pairs per launch; 3715
+// with 256).  Another nh had a generic kernel (101 offsets: 176 -> 419 GB/s).
 #ifndef FWIME_IMG_S16
-#define FWIME_IMG_S16 4, 4, 4, 2, 8, 6
+#define FWIME_IMG_S16 4, 4, 4, 2, 8, 8, 5, 2
 #endif
 #ifndef FWIME_IMG_S24
-#define FWIME_IMG_S24 4, 6, 6, 4, 4, 4
+#define FWIME_IMG_S24 4, 6, 6, 2, 8, 6, 4, 2
 #endif
 #ifndef FWIME_IMG_S32
-#define FWIME_IMG_S32 4, 8, 4, 4, 4, 5
+#define FWIME_IMG_S32 4, 8, 4, 2, 8, 6, 5, 2
 #endif
 #ifndef FWIME_IMG_S48
-#define FWIME_IMG_S48 4, 12, 4, 2, 6, 5
+#define FWIME_IMG_S48 4, 12, 4, 2, 6, 6, 4, 2
 #endif
 
 static cudaError_t launch_image_ext(const ImgArgs &a, cudaStream_t st)
