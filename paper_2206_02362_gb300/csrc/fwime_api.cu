@@ -54,16 +54,17 @@ struct fwime_ctx {
     cudaStream_t st = nullptr;
     size_t max_ws = 0;
     int device = 0;
+    size_t dev_mem = 0;             // total memory of the device
     // options
     int opt_S = 0, opt_K = 0, opt_plain = 0, opt_graph = 0, opt_host_io = 0, opt_zchunk = 0, opt_reuse_bg = 0;
     int opt_tlag = 0;               // > 0: B~ / B~* extend with time lags spaced opt_tlag steps
     int opt_fs = 0;                 // 1: free surface at the top physical row
-    // background-wavefield checkpoints of every shot, [nseg][2][nshot][P], written by B and B~ and
-    // read by B* and B~* on the same v, w (FWIME_OPT_REUSE_BACKGROUND)
+    // background wavefield kept by B and B~ for a B* or B~* on the same v, w (FWIME_OPT_REUSE_BACKGROUND): its D2t at
+    // every step, [nt-1][nshot][P] (hist), where that fits, else its states at the segment starts, [nseg][2][nshot][P]
     struct BgCache {
         float *buf = nullptr;
         size_t bytes = 0;
-        bool valid = false;
+        bool valid = false, hist = false;
         const float *v = nullptr, *w = nullptr;
         int K = 0;
     } bg;
@@ -228,6 +229,15 @@ static int auto_K(int nt)
     return std::min(std::max(K, 8), 128);
 }
 
+// Segment length of the schedules without time lags: longer than sqrt(nt) for few shots, because the extension
+// kernels load their weights or update the image once per launch, which 256 (step, shot) pairs make a few percent of
+// what they read (imaging, nh 41, 4 shots: 56 pairs 1893 GB/s, 256 pairs 3715).  It depends on the problem alone,
+// not on memory or on batches: the same segments give the same sums bit for bit.
+static int seg_len(int nt, int nshot)
+{
+    return std::max(auto_K(nt), std::min(64, (256 + nshot - 1) / nshot));
+}
+
 // Floats of workspace: model part (independent of S) and per-shot part.
 struct Sizes {
     size_t model = 0, per_shot = 0, staging = 0;
@@ -241,10 +251,10 @@ static int tlag_Hs(const fwime_grid &g, int lag) { return (g.nh - 1) * lag; }
 static int tlag_blocks(const fwime_grid &g, int K, int lag) { return (g.nt - 2 + tlag_Hs(g, lag)) / K + 1; }
 
 static Sizes op_sizes(const fwime_grid &g, int nshot, int nrec, long long P, int NZ, int NXP, int op, int K,
-                      bool host_io, bool no_ckpt = false, int tlag = 0)
+                      bool host_io, bool no_ckpt = false, int tlag = 0, bool hist = false)
 {
     Sizes s;
-    const size_t nh = g.nh, nseg = (size_t)((g.nt - 1 + K - 1) / K), R = K + 2;
+    const size_t T = g.nt - 1, nh = g.nh, nseg = (size_t)((g.nt - 1 + K - 1) / K), R = K + 2;
     if (tlag > 0 && op != FWIME_OP_FORWARD && op != FWIME_OP_BORN && op != FWIME_OP_BORN_ADJ) {
         const size_t Hs = tlag_Hs(g, tlag), RD = (size_t)K + 2 * Hs, NB = tlag_blocks(g, K, tlag);
         s.model = al(P) * 2 + al(NZ) + al(NXP);
@@ -271,11 +281,11 @@ static Sizes op_sizes(const fwime_grid &g, int nshot, int nrec, long long P, int
     case FWIME_OP_FORWARD: f = 2; break;
     case FWIME_OP_BORN: s.model += al(P); f = 5; break;
     case FWIME_OP_BORN_EXT: s.model += al(nh * P); f = 4 + 2 * K; break;
-    case FWIME_OP_BORN_ADJ: s.model += al(P); f = 2 + K + R + (no_ckpt ? 0 : 2 * nseg); break;
-    case FWIME_OP_BORN_EXT_ADJ: s.model += al(nh * P); f = 2 + K + R + (no_ckpt ? 0 : 2 * nseg); break;
+    case FWIME_OP_BORN_ADJ: s.model += al(P); f = 2 + (hist ? T : K) + R + (no_ckpt || hist ? 0 : 2 * nseg); break;
+    case FWIME_OP_BORN_EXT_ADJ: s.model += al(nh * P); f = 2 + (hist ? T : K) + R + (no_ckpt || hist ? 0 : 2 * nseg); break;
     case FWIME_OP_TOMO: s.model += 2 * al(nh * P) + al(P); f = 8 + 4 * K; break;
     case FWIME_OP_TOMO_ADJ:
-    case FWIME_OP_GRADIENT: s.model += 2 * al(nh * P) + 2 * al(P); f = 4 + 3 * K + 3 * R + (no_ckpt ? 0 : 4 * nseg); break;
+    case FWIME_OP_GRADIENT: s.model += 2 * al(nh * P) + 2 * al(P); f = 4 + K + 2 * (hist ? T : (size_t)K) + 3 * R + (no_ckpt || hist ? 0 : 4 * nseg); break;
     case FWIME_OP_OBJECTIVE: s.model += 2 * al(nh * P) + 2 * al(P); f = 4 + 2 * K; break;
     default: break;
     }
@@ -312,6 +322,7 @@ static int validate(const fwime_grid *g, const fwime_geom *geo, fwime_ctx *x)
 
 struct WS {
     int S = 1, K = 8, nseg = 1, R = 10;
+    bool hist = false;  // adjoint ops: the source side's D2t of every step kept instead of recomputed
     // model
     float *c, *bpad, *gz, *gx, *coef, *W, *W2, *ptp, *acc1, *acc2;
     // per batch
@@ -322,9 +333,30 @@ struct WS {
     float *sv, *sw, *sd1, *sd2, *sm1, *sdv, *smo;
 };
 
+// Device memory the kept D2t histories may take: a third of the card, so that two more contexts of the same kind
+// (and the caller's own arrays) still fit beside this one.
+static size_t hist_cap(const fwime_ctx *x, size_t budget)
+{
+    return std::min(budget, x->max_ws ? x->max_ws : x->dev_mem / 3);
+}
+
+// Does keeping the histories at S_h shots per launch beat recomputing at S_c?  Stencil launches per step with and
+// without (B*, B~*: 2 against 3; T*, gradient: 4 against 6), each costing about 6 us plus 12 B per point and shot at
+// 6.2 TB/s (measured: 8.2 us for one Marmousi2-shaped shot, 179 us for 100).  Kept against recomputed, in ms: B*
+// North-Sea-shaped 60 shots nt 400 (60 per launch) 126 / 177, nt 2000 (12 per launch) 663 / 880; gradient nh 31 nt
+// 300 (30 per launch) 292 / 387; Salt-shaped gradient 4 shots nt 200 151 / 225; one shot nt 1000 34 / 50.
+static bool hist_pays(const fwime_ctx *x, int op, int S_h, int S_c)
+{
+    const bool two = op == FWIME_OP_TOMO_ADJ || op == FWIME_OP_GRADIENT;
+    const double per = 12.0 * (double)x->P / 6.2e6, launch = 6.0;   // us
+    const double h = (two ? 4.0 : 2.0) * (launch / S_h + per), c = (two ? 6.0 : 3.0) * (launch / S_c + per);
+    return h < c;
+}
+
+// no_ckpt: the source side's states or history are kept outside the workspace
 static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
 {
-    w.K = x->opt_K > 0 ? x->opt_K : auto_K(x->g.nt);
+    w.K = x->opt_K > 0 ? x->opt_K : x->opt_tlag > 0 ? auto_K(x->g.nt) : seg_len(x->g.nt, x->nshot);
     // time lags: segments of at least 4 Hs steps keep the lag halo (2 Hs samples per segment, read once per
     // residue class) at half the segment's own K samples or less
     if (x->opt_tlag > 0 && x->opt_K == 0) w.K = std::max(w.K, 4 * tlag_Hs(x->g, x->opt_tlag));
@@ -342,6 +374,15 @@ static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
         budget = x->ws_bytes + fr;
         budget = budget > ((size_t)2 << 30) ? budget - ((size_t)2 << 30) : budget / 2;   // keep 2 GB slack
     }
+    // a default segment longer than sqrt(nt) that does not fit falls back to that (not where stored states tie it)
+    const int S_least = x->opt_S > 0 && !x->opt_plain ? std::min(x->opt_S, x->nshot) : 1;
+    if (x->opt_tlag == 0 && x->opt_K == 0 && !no_ckpt && w.K > auto_K(x->g.nt) &&
+        (sz.model + sz.staging + sz.per_shot * S_least) * sizeof(float) + 4096 > budget) {
+        w.K = std::max(std::min(auto_K(x->g.nt), x->g.nt - 1), 1);
+        w.nseg = (x->g.nt - 1 + w.K - 1) / w.K;
+        w.R = w.K + 2;
+        sz = op_sizes(x->g, x->nshot, x->nrec, x->P, x->NZ, x->NXP, op, w.K, x->opt_host_io != 0, no_ckpt, 0);
+    }
     // a default time-lag segment of 4 Hs that does not fit one shot falls back to 2 Hs (the halo then
     // equals the segment's own samples; the kernels stay correct for any K)
     if (x->opt_tlag > 0 && x->opt_K == 0 && w.K > 2 * tlag_Hs(x->g, x->opt_tlag) &&
@@ -352,10 +393,45 @@ static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
         sz = op_sizes(x->g, x->nshot, x->nrec, x->P, x->NZ, x->NXP, op, w.K, x->opt_host_io != 0, no_ckpt,
                       x->opt_tlag);
     }
-    const size_t fixed = (sz.model + sz.staging) * sizeof(float);
-    const size_t per = sz.per_shot * sizeof(float);
+    size_t fixed = (sz.model + sz.staging) * sizeof(float);
+    size_t per = sz.per_shot * sizeof(float);
     int S;
+    const int S_max = x->opt_S > 0 ? std::min(x->opt_S, x->nshot) : x->nshot;
+    // the largest equal batches of at most `cap` bytes
+    auto batch = [&](size_t cap, size_t fx, size_t pr) {
+        int n = fx + pr > cap ? 1 : (int)std::min<size_t>((size_t)S_max, (cap - fx) / pr);
+        n = std::max(n, 1);
+        const int nb = (x->nshot + n - 1) / n;
+        return std::min(n, (x->nshot + nb - 1) / nb);
+    };
+    const bool adj_op = op == FWIME_OP_BORN_ADJ || op == FWIME_OP_BORN_EXT_ADJ || op == FWIME_OP_TOMO_ADJ ||
+                        op == FWIME_OP_GRADIENT;
+    w.hist = false;
+    int hist_S = 0;
+    if (adj_op && !no_ckpt && x->opt_K == 0 && x->opt_tlag == 0 && !x->opt_plain) {
+        const size_t cap = hist_cap(x, budget);
+        const Sizes sh = op_sizes(x->g, x->nshot, x->nrec, x->P, x->NZ, x->NXP, op, w.K, x->opt_host_io != 0, false, 0, true);
+        const size_t hf = (sh.model + sh.staging) * sizeof(float) + 4096, hp = sh.per_shot * sizeof(float);
+        int S_h = x->opt_S > 0 ? S_max : batch(cap, hf, hp);
+        if (x->opt_S == 0) {
+            // The history's memory is mapped once per context, at about 870 GB/s; more batches map less and launch
+            // more (6 us per stencil launch).  The number of batches that is best for four calls on a context:
+            const double T = x->g.nt - 1, two = op == FWIME_OP_TOMO_ADJ || op == FWIME_OP_GRADIENT ? 2.0 : 1.0;
+            const double map_us = two * T * 4.0 * (double)x->P * x->nshot / 0.87e6, launch_us = two * T * 2.0 * 6.0;
+            const int nb = std::max(1, (int)std::lround(std::sqrt(map_us / 4.0 / launch_us)));
+            // (not below the 256 pairs per segment that the extension kernels' launches want)
+            S_h = std::min(S_h, std::max((x->nshot + nb - 1) / nb, (256 + w.K - 1) / w.K));
+        }
+        const int S_c = x->opt_S > 0 ? S_max : batch(budget, fixed, per);
+        if (hf + hp * (size_t)S_h <= cap && hist_pays(x, op, S_h, S_c)) {
+            w.hist = true;
+            hist_S = S_h;
+            fixed = hf;
+            per = hp;
+        }
+    }
     if (x->opt_plain) S = 1;
+    else if (w.hist) S = hist_S;
     else if (x->opt_S > 0) S = std::min(x->opt_S, x->nshot);
     else {
         if (fixed + per > budget) S = 1;
@@ -452,13 +528,14 @@ static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
     case FWIME_OP_BORN: nf = 5; break;
     case FWIME_OP_BORN_EXT: nf = 4; nk = 2; break;
     case FWIME_OP_BORN_ADJ:
-    case FWIME_OP_BORN_EXT_ADJ: nf = 2; nk = 1; nr = 1; nck = no_ckpt ? 0 : 2; break;
+    case FWIME_OP_BORN_EXT_ADJ: nf = 2; nk = 1; nr = 1; nck = no_ckpt || w.hist ? 0 : 2; break;
     case FWIME_OP_TOMO: nf = 8; nk = 4; break;
     case FWIME_OP_OBJECTIVE: nf = 4; nk = 2; break;
-    default: nf = 4; nk = 3; nr = 3; nck = no_ckpt ? 0 : 4; break;
+    default: nf = 4; nk = 3; nr = 3; nck = no_ckpt || w.hist ? 0 : 4; break;
     }
     for (int i = 0; i < nf; ++i) w.f[i] = take(SP);
-    for (int i = 0; i < nk; ++i) w.ring[i] = take((size_t)w.K * SP);
+    // (kept histories: D2t of q0 in ring[0], of the scattered field in ring[2], every step)
+    for (int i = 0; i < nk; ++i) w.ring[i] = take((w.hist && i != 1 ? (size_t)x->g.nt - 1 : (size_t)w.K) * SP);
     for (int i = 0; i < nr; ++i) w.ring[nk + i] = take((size_t)w.R * SP);
     if (nck) w.ckpt = take((size_t)w.nseg * nck * SP);
     if ((op == FWIME_OP_GRADIENT || op == FWIME_OP_OBJECTIVE) && !no_ckpt)
@@ -655,29 +732,38 @@ static int prep_model(fwime_ctx *x, Run &r, const float *v)
 
 static int seg_K(const fwime_ctx *x)
 {
-    int K = x->opt_K > 0 ? x->opt_K : auto_K(x->g.nt);
+    int K = x->opt_K > 0 ? x->opt_K : x->opt_tlag > 0 ? auto_K(x->g.nt) : seg_len(x->g.nt, x->nshot);
     return std::max(std::min(K, x->g.nt - 1), 1);
 }
 
-static size_t bg_bytes(const fwime_ctx *x, int K)
+static size_t bg_bytes(const fwime_ctx *x, int K, bool hist)
 {
-    const size_t nseg = (size_t)((x->g.nt - 1 + K - 1) / K);
-    return nseg * 2 * (size_t)x->nshot * (size_t)x->P * sizeof(float);
+    const size_t planes = hist ? (size_t)x->g.nt - 1 : 2 * (size_t)((x->g.nt - 1 + K - 1) / K);
+    return planes * (size_t)x->nshot * (size_t)x->P * sizeof(float);
 }
 
-// Makes room for the cache; false when it does not fit (the call then runs without it).
+// Makes room for the cache; false when it does not fit (the call then runs without it).  The D2t of every step
+// (one propagation fewer than the states: nothing is recomputed) where it fits hist_cap and the segment length is
+// not the caller's, else the states; what a context holds it keeps.
 static bool bg_reserve(fwime_ctx *x, int K)
 {
-    const size_t need = bg_bytes(x, K);
-    if (x->bg.buf && x->bg.bytes >= need) return true;
+    const bool may_hist = x->opt_K == 0 && !x->opt_plain;
+    const size_t hneed = bg_bytes(x, K, true), need_st = bg_bytes(x, K, false);
+    if (x->bg.buf && (x->capturing || !x->bg.hist || may_hist) && x->bg.bytes >= (x->bg.hist ? hneed : need_st))
+        return true;
     if (x->capturing) return false;
-    if (x->max_ws && x->ws_bytes + need > x->max_ws) return false;
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    if (need + ((size_t)4 << 30) > fr + x->bg.bytes) return false;   // leave room for the operator's workspace
+    // room: within the caller's cap, and leaving room for the operator's workspace
+    const auto fits = [&](size_t n) {
+        return !(x->max_ws && x->ws_bytes + n > x->max_ws) && n + ((size_t)4 << 30) <= fr + x->bg.bytes;
+    };
+    const bool hist = may_hist && hneed <= hist_cap(x, tot) && fits(hneed);
+    const size_t need = hist ? hneed : need_st;
+    if (!fits(need)) return false;
     if (x->bg.buf) cudaFreeAsync(x->bg.buf, x->st);
     x->bg = fwime_ctx::BgCache{};
     if (cudaMallocAsync(reinterpret_cast<void **>(&x->bg.buf), need, x->st) != cudaSuccess) {
@@ -686,6 +772,7 @@ static bool bg_reserve(fwime_ctx *x, int K)
         return false;
     }
     x->bg.bytes = need;
+    x->bg.hist = hist;
     return true;
 }
 
@@ -694,6 +781,8 @@ static float *bg_slot(fwime_ctx *x, int j, int t, int s0)
 {
     return x->bg.buf + ((2LL * j + t) * x->nshot + s0) * x->P;
 }
+// kept D2t of step n for the batch starting at shot s0 (steps are nshot P apart)
+static float *bg_d2t(fwime_ctx *x, int n, int s0) { return x->bg.buf + ((long long)n * x->nshot + s0) * x->P; }
 
 // ---------------------------------------------------------------- gradient state (split gradient)
 static size_t gs_bytes(const fwime_ctx *x, int K)
@@ -771,7 +860,8 @@ static int run_born(fwime_ctx *x, Run &r, const float *v, const float *w, const 
         float *db = d + s0 * nd;
         TRY(zero(x, db, sizeof(float) * Sb * nd));
         for (int n = 0; n + 1 < nt; ++n) {
-            if (x->bg_written && n % r.w.K == 0) {
+            if (x->bg_written && x->bg.hist) D = bg_d2t(x, n, s0);
+            else if (x->bg_written && n % r.w.K == 0) {
                 TRY(copyf(x, bg_slot(x, n / r.w.K, 0, s0), c0, (size_t)Sb * x->P));
                 TRY(copyf(x, bg_slot(x, n / r.w.K, 1, s0), p0, (size_t)Sb * x->P));
             }
@@ -796,6 +886,7 @@ static int run_born_ext(fwime_ctx *x, Run &r, const float *v, const float *w, co
            launch_ext_weights(pt, r.w.bpad, nullptr, nullptr, r.w.W, x->g.nh, x->g.nz, x->g.nx, x->o, x->NXP, x->P, 0,
                               x->st));
     float *Dr = r.w.ring[0], *Er = r.w.ring[1];
+    const bool keep = x->bg_written && x->bg.hist;   // the D2t of every step stays for a following adjoint
     TRY(zero(x, Er, sizeof(float) * K * SP));
     for (int s0 = 0; s0 < x->nshot; s0 += S) {
         const int Sb = std::min(S, x->nshot - s0);
@@ -806,15 +897,16 @@ static int run_born_ext(fwime_ctx *x, Run &r, const float *v, const float *w, co
         TRY(zero(x, db, sizeof(float) * Sb * nd));
         for (int n0 = 0; n0 < nt - 1; n0 += K) {
             const int n1 = std::min(n0 + K, nt - 1), kk = n1 - n0;
-            if (x->bg_written) {
+            if (x->bg_written && !keep) {
                 TRY(copyf(x, bg_slot(x, n0 / K, 0, s0), c0, (size_t)Sb * x->P));
                 TRY(copyf(x, bg_slot(x, n0 / K, 1, s0), p0, (size_t)Sb * x->P));
             }
             for (int n = n0; n < n1; ++n) {
-                TRY(prop(r, Sb, c0, p0, p0, Dr + (n - n0) * SP, w + (size_t)s0 * nt + n, s0));
+                TRY(prop(r, Sb, c0, p0, p0, keep ? bg_d2t(x, n, s0) : Dr + (n - n0) * SP, w + (size_t)s0 * nt + n, s0));
                 std::swap(c0, p0);
             }
-            TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(Dr, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
+            const RingRef dring = keep ? ringref(bg_d2t(x, n0, s0), x->nshot * x->P, 0, 0) : ringref(Dr, SP, 0, 0);
+            TRY(scatter(r, Sb, n0, kk, r.w.W, dring, ringref(Er, SP, 0, 0), +1, 0));
             for (int n = n0; n < n1; ++n) {
                 TRY(prop(r, Sb, c1, p1, p1, nullptr, nullptr, 0, Er + (n - n0) * SP, 1.f, nullptr, 0.f, nullptr, 0.f,
                          nullptr, nullptr, RecTo{db + (size_t)n * x->nrec, 0}));
@@ -844,9 +936,16 @@ static int run_born_adj(fwime_ctx *x, Run &r, bool ext, const float *v, const fl
         for (int i = 0; i < 2; ++i) TRY(zero(x, r.w.f[i], fb));
         TRY(zero(x, Mu, sizeof(float) * R * SP));
         const float *ws = w + (size_t)s0 * nt;
-        // checkpoint (q^{n0}, q^{n0-1}) at every segment start: from the background cache, or a forward sweep
+        // The D2t of q0: kept at every step (by this call's forward sweep, or by the B or B~ before it), or
+        // recomputed segment by segment from the states (q^{n0}, q^{n0-1}) at every segment start (from the
+        // background cache, or a forward sweep)
+        const bool kept = r.w.hist || (use_bg && x->bg.hist);
         auto ckp = [&](int j, int t) -> float * { return use_bg ? bg_slot(x, j, t, s0) : ck + (2LL * j + t) * SP; };
-        for (int j = 0; j < nseg && !use_bg; ++j) {
+        for (int n = 0; n + 1 < nt && r.w.hist; ++n) {
+            TRY(prop(r, Sb, cur, prv, prv, Dr + n * SP, ws + n, s0));
+            std::swap(cur, prv);
+        }
+        for (int j = 0; j < nseg && !use_bg && !kept; ++j) {
             TRY(copyf(x, ck + (2LL * j) * SP, cur, (size_t)Sb * x->P));
             TRY(copyf(x, ck + (2LL * j + 1) * SP, prv, (size_t)Sb * x->P));
             if (j == nseg - 1) break;
@@ -858,21 +957,26 @@ static int run_born_adj(fwime_ctx *x, Run &r, bool ext, const float *v, const fl
         // backward sweep
         for (int j = nseg - 1; j >= 0; --j) {
             const int n0 = j * K, n1 = std::min(n0 + K, nt - 1), kk = n1 - n0;
-            TRY(copyf(x, cur, ckp(j, 0), (size_t)Sb * x->P));
-            TRY(copyf(x, prv, ckp(j, 1), (size_t)Sb * x->P));
-            for (int n = n0; n < n1; ++n) {
-                TRY(prop(r, Sb, cur, prv, prv, Dr + (n - n0) * SP, ws + n, s0));
-                std::swap(cur, prv);
+            if (!kept) {
+                TRY(copyf(x, cur, ckp(j, 0), (size_t)Sb * x->P));
+                TRY(copyf(x, prv, ckp(j, 1), (size_t)Sb * x->P));
+                for (int n = n0; n < n1; ++n) {
+                    TRY(prop(r, Sb, cur, prv, prv, Dr + (n - n0) * SP, ws + n, s0));
+                    std::swap(cur, prv);
+                }
             }
+            const RingRef dring = r.w.hist ? ringref(Dr + n0 * SP, SP, 0, 0)
+                                  : kept   ? ringref(bg_d2t(x, n0, s0), x->nshot * x->P, 0, 0)
+                                           : ringref(Dr, SP, 0, 0);
             for (int m = n1; m >= n0 + 1; --m) {
                 float *mo = Mu + (m % R) * SP;
                 TRY(adj_step(r, Sb, Mu + ((m + 1) % R) * SP, Mu + ((m + 2) % R) * SP, mo, d + s0 * nd + (size_t)m * x->nrec));
             }
             if (ext)
-                TRY(image(r, Sb, n0, kk, IMG_EXT, ringref(Dr, SP, 0, 0), ringref(Mu, SP, R, 1), ringref(nullptr, 0, 0, 0),
+                TRY(image(r, Sb, n0, kk, IMG_EXT, dring, ringref(Mu, SP, R, 1), ringref(nullptr, 0, 0, 0),
                           ringref(nullptr, 0, 0, 0), 1.f, r.w.acc1));
             else
-                TRY(image(r, Sb, n0, kk, IMG_LOCAL, ringref(Dr, SP, 0, 0), ringref(Mu, SP, R, 1),
+                TRY(image(r, Sb, n0, kk, IMG_LOCAL, dring, ringref(Mu, SP, R, 1),
                           ringref(nullptr, 0, 0, 0), ringref(nullptr, 0, 0, 0), 1.f, r.w.acc1));
         }
     }
@@ -1312,7 +1416,7 @@ static int run_tomo_adj(fwime_ctx *x, Run &r, int mode, const float *v, const fl
         float *pred = state ? res_state + s0 * nd : r.w.pred;
         const float *rr = d + s0 * nd;
         if (fwd) {
-            const bool keep = bwd || state;   // checkpoints for an adjoint sweep
+            const bool keep = (bwd || state) && !r.w.hist;   // states for an adjoint sweep that recomputes
             if (grad) TRY(zero(x, pred, sizeof(float) * Sb * nd));
             // forward sweep
             for (int j = 0; j < nseg; ++j) {
@@ -1322,18 +1426,19 @@ static int run_tomo_adj(fwime_ctx *x, Run &r, int mode, const float *v, const fl
                     TRY(copyf(x, ckp(j, 2), qsc, fn));
                     TRY(copyf(x, ckp(j, 3), qsp, fn));
                 }
-                if (!grad && j == nseg - 1) break;
+                if (!grad && !r.w.hist && j == nseg - 1) break;
                 const int n0 = j * K, n1 = std::min(n0 + K, nt - 1), kk = n1 - n0;
+                float *D0 = D0r + (r.w.hist ? n0 * SP : 0);
                 // with the gradient, the launch of step n adds its input (q0^n, then the scattered field's)
                 // to the prediction's row n (zeroed above; a + b is exact in either order of the two)
                 for (int n = n0; n < n1; ++n) {
-                    TRY(prop(r, Sb, q0c, q0p, q0p, D0r + (n - n0) * SP, ws + n, s0, nullptr, 0.f, nullptr, 0.f,
+                    TRY(prop(r, Sb, q0c, q0p, q0p, D0 + (n - n0) * SP, ws + n, s0, nullptr, 0.f, nullptr, 0.f,
                              nullptr, 0.f, nullptr, nullptr, RecTo{grad ? pred + (size_t)n * x->nrec : nullptr, 1}));
                     std::swap(q0c, q0p);
                 }
-                TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0r, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
+                TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
                 for (int n = n0; n < n1; ++n) {
-                    TRY(prop(r, Sb, qsc, qsp, qsp, nullptr, nullptr, 0, Er + (n - n0) * SP, 1.f, nullptr, 0.f, nullptr,
+                    TRY(prop(r, Sb, qsc, qsp, qsp, r.w.hist ? Dsr + n * SP : nullptr, nullptr, 0, Er + (n - n0) * SP, 1.f, nullptr, 0.f, nullptr,
                              0.f, nullptr, nullptr, RecTo{grad ? pred + (size_t)n * x->nrec : nullptr, 1}));
                     std::swap(qsc, qsp);
                 }
@@ -1350,19 +1455,23 @@ static int run_tomo_adj(fwime_ctx *x, Run &r, int mode, const float *v, const fl
         // backward sweep
         for (int j = nseg - 1; j >= 0; --j) {
             const int n0 = j * K, n1 = std::min(n0 + K, nt - 1), kk = n1 - n0;
-            TRY(copyf(x, q0c, ckp(j, 0), fn));
-            TRY(copyf(x, q0p, ckp(j, 1), fn));
-            TRY(copyf(x, qsc, ckp(j, 2), fn));
-            TRY(copyf(x, qsp, ckp(j, 3), fn));
-            for (int n = n0; n < n1; ++n) {
-                TRY(prop(r, Sb, q0c, q0p, q0p, D0r + (n - n0) * SP, ws + n, s0));
-                std::swap(q0c, q0p);
+            if (!r.w.hist) {   // the source side's D2t of this segment again, from its start's states
+                TRY(copyf(x, q0c, ckp(j, 0), fn));
+                TRY(copyf(x, q0p, ckp(j, 1), fn));
+                TRY(copyf(x, qsc, ckp(j, 2), fn));
+                TRY(copyf(x, qsp, ckp(j, 3), fn));
+                for (int n = n0; n < n1; ++n) {
+                    TRY(prop(r, Sb, q0c, q0p, q0p, D0r + (n - n0) * SP, ws + n, s0));
+                    std::swap(q0c, q0p);
+                }
+                TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0r, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
+                for (int n = n0; n < n1; ++n) {
+                    TRY(prop(r, Sb, qsc, qsp, qsp, Dsr + (n - n0) * SP, nullptr, 0, Er + (n - n0) * SP, 1.f));
+                    std::swap(qsc, qsp);
+                }
             }
-            TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0r, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
-            for (int n = n0; n < n1; ++n) {
-                TRY(prop(r, Sb, qsc, qsp, qsp, Dsr + (n - n0) * SP, nullptr, 0, Er + (n - n0) * SP, 1.f));
-                std::swap(qsc, qsp);
-            }
+            const RingRef d0ring = ringref(D0r + (r.w.hist ? n0 * SP : 0), SP, 0, 0);
+            const RingRef dsring = ringref(Dsr + (r.w.hist ? n0 * SP : 0), SP, 0, 0);
             // adjoint of the residual: mu^m, m = n1 .. n0+1 (lambda^ at step n is mu^{n+1}), each step also
             // writing its D2t, (mu^m - 2 mu^{m+1} + mu^{m+2}) / dt^2, at slot m - n0 - 1 of Zr
             for (int m = n1; m >= n0 + 1; --m) {
@@ -1382,8 +1491,8 @@ static int run_tomo_adj(fwime_ctx *x, Run &r, int mode, const float *v, const fl
             }
             // the extended image of the residual's adjoint field (contracted with p~ at the end) and, in the
             // same launch, the local terms D0 (alpha lambda^ + mu2) + Ds lambda^
-            TRY(image(r, Sb, n0, kk, IMG_EXT, ringref(D0r, SP, 0, 0), ringref(Mu, SP, R, 1), ringref(Mu2, SP, R, 1),
-                      ringref(Dsr, SP, 0, 0), grad ? 1.f : 0.f, r.w.acc2, r.w.acc1));
+            TRY(image(r, Sb, n0, kk, IMG_EXT, d0ring, ringref(Mu, SP, R, 1), ringref(Mu2, SP, R, 1), dsring,
+                      grad ? 1.f : 0.f, r.w.acc2, r.w.acc1));
         }
     }
     if (bwd)
@@ -1452,6 +1561,7 @@ static int enqueue(fwime_ctx *x, const Call &c)
                             c.op == OP_GRAD_FWD ? PH_FORWARD : PH_BACKWARD);
     }
     TRY(plan(x, c.op, r.w, use_bg));
+    if (r.w.K < seg_K(x) && !(x->bg_written && x->bg.hist)) x->bg_written = false;   // shorter segments than the cache's
     init_run(x, r, r.w.S);
     TRY(prep_model(x, r, c.v));
     switch (c.op) {
@@ -1601,7 +1711,7 @@ int fwime_workspace_bytes(const fwime_grid *g, const fwime_geom *geo, int op, in
     if (validate(g, geo, nullptr) != FWIME_OK || !bytes || op < 0 || op > FWIME_OP_OBJECTIVE) return FWIME_EINVAL;
     const int NZ = g->nz + 2 * (g->sponge + 4), NX = g->nx + 2 * (g->sponge + 4), NXP = (NX + 31) / 32 * 32;
     const long long P = (long long)NZ * NXP;
-    int K = segment > 0 ? segment : auto_K(g->nt);
+    int K = segment > 0 ? segment : seg_len(g->nt, geo->nshot);
     K = std::max(1, std::min(K, g->nt - 1));
     Sizes s = op_sizes(*g, geo->nshot, geo->nrec, P, NZ, NXP, op, K, false);
     const int S = shots_per_batch > 0 ? std::min(shots_per_batch, geo->nshot) : geo->nshot;
@@ -1631,6 +1741,11 @@ int fwime_create(fwime_ctx **out, const fwime_grid *g, const fwime_geom *geo, si
     x->st = reinterpret_cast<cudaStream_t>(cuda_stream);
     x->max_ws = max_workspace_bytes;
     cudaGetDevice(&x->device);
+    size_t free_mem = 0;
+    if (cudaMemGetInfo(&free_mem, &x->dev_mem) != cudaSuccess) {
+        cudaGetLastError();
+        x->dev_mem = 0;
+    }
     // offsets: [src_off(nshot)][rec_off(nrec)]
     x->h_off.resize(x->nshot + x->nrec);
     for (int s = 0; s < x->nshot; ++s) x->h_off[s] = (x->src_iz[s] + x->o) * x->NXP + x->src_ix[s] + x->o;
@@ -2237,7 +2352,7 @@ int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
     std::vector<int> Ks;
     if (saved_K > 0) Ks = {saved_K};
     else {
-        const int K0 = seg_K(x);
+        const int K0 = std::max(std::min(auto_K(x->g.nt), x->g.nt - 1), 1);
         Ks = {K0, std::max(K0 / 2, 8), std::min(2 * K0, x->g.nt - 1)};
         std::sort(Ks.begin(), Ks.end());
         Ks.erase(std::unique(Ks.begin(), Ks.end()), Ks.end());
