@@ -556,7 +556,7 @@ struct Run {
 static void init_run(fwime_ctx *x, Run &r, int S)
 {
     r.x = x;
-    const int rows = x->NZ - 8;
+    const int rows = x->NZ - 4 - (x->opt_fs ? x->o : 4);   // updated rows
     r.nstrip = (x->NXP + STRIP - 1) / STRIP;
     int zc = x->opt_zchunk;
     if (zc <= 0) {
@@ -579,6 +579,8 @@ static void init_run(fwime_ctx *x, Run &r, int S)
     a.inv_dt2 = (float)(1.0 / ((double)x->g.dt * x->g.dt));
     a.src_scale = (float)(1.0 / ((double)x->g.dx * x->g.dz));
     a.zs_lo = x->o; a.zs_hi = x->o + x->g.nz;
+    a.z_first = x->opt_fs ? x->o : 4;
+    a.fs_row = x->opt_fs ? x->o : 0;
 }
 
 // Receivers of a stencil launch's input field, recorded by the launch itself: row d of the data (=, or +=).
@@ -624,9 +626,6 @@ static int prop(Run &r, int Sb, const float *cur, const float *prev, float *out,
                         (inj.val ? (double)Sb * x->nrec * 4.0 : 0.0);
     LAUNCH(FWIME_K_PROP, pts * (Sb * 12.0 + 4.0) + spts * (Sb * srcb + (coef ? 4.0 : 0.0)) + recb,
            launch_prop(a, Sb, x->st));
-    if (x->opt_fs)
-        LAUNCH(FWIME_K_OTHER, (double)Sb * x->NXP * (d2 ? 44.0 : 40.0),
-               launch_free_surface(out, d2, Sb, x->P, x->NXP, x->o, x->st));
     return FWIME_OK;
 }
 

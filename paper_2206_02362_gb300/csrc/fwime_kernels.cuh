@@ -60,6 +60,8 @@ struct PropArgs {
     // (read there only, zero elsewhere) and where D2t is written (its readers, the extension and
     // imaging kernels, read physical rows only)
     int zs_lo, zs_hi;
+    int z_first;                   // first row updated: 4, or the free surface's row
+    int fs_row;                    // padded row of the free surface (>= 4), 0: none
     int naux_max;                  // rows per aux stage (set by launch_prop)
     // optional receiver recording of the INPUT field: d[s * rec_dstride + r] (=, or += with rec_acc)
     // = cur[s * P + rec_off[r]] for r < nrec, done by the first CTA of every shot (cur is complete
@@ -197,7 +199,6 @@ struct PrepArgs {
     int fs;                        // 1: free surface at the top physical row
 };
 cudaError_t launch_prep(const PrepArgs &a, cudaStream_t st);
-cudaError_t launch_free_surface(float *q, float *d2, int nshot, long long P, int NXP, int o, cudaStream_t st);
 
 // elementwise helpers on padded / physical grids
 cudaError_t launch_embed_scale(const float *phys, const float *scale_pad, float *out_pad, int nz, int nx,

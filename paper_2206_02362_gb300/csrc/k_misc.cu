@@ -43,25 +43,6 @@ __global__ void k_prep(const PrepArgs a)
                        : 0.f;
 }
 
-// free surface (pressure release at the top physical row IZ = o): after a step, q = 0 on the surface row
-// and the 4 rows above hold the odd mirror -q of the 4 rows below; D2t is 0 on the surface row
-__global__ void k_free_surface(float *q, float *d2, long long P, int NXP, int o)
-{
-    const int IX = blockIdx.x * blockDim.x + threadIdx.x;
-    if (IX >= NXP) return;
-    const long long f = (long long)blockIdx.y * P + IX;
-    q[f + (long long)o * NXP] = 0.f;
-#pragma unroll
-    for (int k = 1; k <= 4; ++k) q[f + (long long)(o - k) * NXP] = -q[f + (long long)(o + k) * NXP];
-    if (d2) d2[f + (long long)o * NXP] = 0.f;
-}
-
-cudaError_t launch_free_surface(float *q, float *d2, int nshot, long long P, int NXP, int o, cudaStream_t st)
-{
-    k_free_surface<<<dim3((NXP + 127) / 128, nshot), 128, 0, st>>>(q, d2, P, NXP, o);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_prep(const PrepArgs &a, cudaStream_t st)
 {
     dim3 grid((a.NXP + 127) / 128, a.NZ);
