@@ -110,6 +110,7 @@ struct fwime_ctx {
     long long prof_n[5] = {0, 0, 0, 0, 0};
     int last_err = 0;
     char err[320] = {0};
+    bool shared = false;            // one of several requests in flight on the GPU (the request server's contexts)
     Server *srv = nullptr;          // a server context (fwime_server_create): no grid, no operators
 };
 
@@ -121,6 +122,7 @@ fwime_ctx *ctx_for_server(Server *srv)
     return x;
 }
 Server *ctx_server(const fwime_ctx *x) { return x ? x->srv : nullptr; }
+void ctx_set_shared(fwime_ctx *x) { x->shared = true; }
 }  // namespace fwk
 
 // operator entry points refuse a server context
@@ -421,6 +423,8 @@ static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
             const int nb = std::max(1, (int)std::lround(std::sqrt(map_us / 4.0 / launch_us)));
             // (not below the 256 pairs per segment that the extension kernels' launches want)
             S_h = std::min(S_h, std::max((x->nshot + nb - 1) / nb, (256 + w.K - 1) / w.K));
+            const int batches = (x->nshot + S_h - 1) / S_h;
+            S_h = (x->nshot + batches - 1) / batches;   // of equal size
         }
         const int S_c = x->opt_S > 0 ? S_max : batch(budget, fixed, per);
         if (hf + hp * (size_t)S_h <= cap && hist_pays(x, op, S_h, S_c)) {
@@ -560,11 +564,10 @@ static void init_run(fwime_ctx *x, Run &r, int S)
     r.nstrip = (x->NXP + STRIP - 1) / STRIP;
     int zc = x->opt_zchunk;
     if (zc <= 0) {
-        const long long target = 152LL * 32;   // resident warps to aim for
-        long long per = (long long)r.nstrip * std::max(S, 1);
-        long long nchunk_t = std::max<long long>(1, (target + per - 1) / per);
-        zc = (int)((rows + nchunk_t - 1) / nchunk_t);
-        zc = std::min(std::max(zc, 8), 256);
+        // 4 CTAs of 4 warps per SM.  Beside other requests the total work counts, not one launch's latency: items of a
+        // few rows load three times the rows that they write.
+        zc = chunk_rows(rows, r.nstrip, std::max(S, 1), 152LL * 16, nullptr);
+        if (x->shared) zc = std::max(zc, 8);
     }
     r.zchunk = zc;
     r.nchunk = (rows + zc - 1) / zc;
@@ -2171,7 +2174,10 @@ int fwime_forward_group(fwime_ctx *const *ctxs, int n, const float *const *v, co
         TRY(plan(m, FWIME_OP_FORWARD, runs[i].w));
         if (runs[i].w.S < m->nshot)
             return fail(x, FWIME_ENOMEM, "group member %d: %d shots do not fit one batch", i, m->nshot);
+        const bool alone = !m->shared;
+        if (n > 1) m->shared = true;   // the members fill the launch together
         init_run(m, runs[i], m->nshot);
+        if (alone) m->shared = false;
         const long long before = m->launches;
         TRY(prep_model(m, runs[i], v[i]));
         if (m != x) x->launches += m->launches - before;   // the group's count includes every member's prep

@@ -180,6 +180,7 @@ struct TlagArgs {
 // launchers (return cudaGetLastError())
 cudaError_t launch_prop(const PropArgs &a, int nshot, cudaStream_t st);
 cudaError_t prop_occupancy(int *blocks_per_sm);
+int chunk_rows(int rows, int nstrip, int S, long long warps, long long *cost_out);   // rows per warp
 cudaError_t launch_prop_group(const GroupMember *m, int nactive, int ctas, const GroupRec *g, int nrec_threads,
                               int step, cudaStream_t st, bool record);
 cudaError_t launch_points(const PointsArgs &a, int nshot, cudaStream_t st);

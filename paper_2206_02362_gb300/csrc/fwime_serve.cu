@@ -114,6 +114,7 @@ void enqueue_group(Server *s, Group *g)
         fwime_request &r = j->req;
         fwime_geom geo{r.geom.nshot, j->siz.data(), j->six.data(), r.geom.nrec, j->riz.data(), j->rix.data()};
         int rc = fwime_create(&j->ctx, &r.grid, &geo, j->ws, st);
+        if (rc == FWIME_OK) ctx_set_shared(j->ctx);
         if (rc == FWIME_OK) rc = fwime_set_option(j->ctx, FWIME_OPT_SHOTS_PER_BATCH, r.geom.nshot);
         if (rc == FWIME_OK && (s->options & FWIME_SERVE_PLAIN)) rc = fwime_set_option(j->ctx, FWIME_OPT_PLAIN, 1);
         const float *v = r.v, *w = r.w, *pt = r.pt, *dobs = r.dobs;

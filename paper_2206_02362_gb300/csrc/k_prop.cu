@@ -1,4 +1,6 @@
 // Stencil launches without a free surface, grouped forward steps, receiver points (kernel: fwime_prop.cuh).
+#include <algorithm>
+
 #include "fwime_prop.cuh"
 
 namespace fwk {
@@ -69,6 +71,24 @@ cudaError_t prop_occupancy(int *blocks_per_sm)
     const size_t smem = (size_t)PROP_WARPS * (CUR_SLOTS * CUR_ROW + AUX_SLOTS * 2 * STRIP) * sizeof(float);
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_prop<0, false, false, false, false>, PROP_WARPS * 32,
                                                          smem);
+}
+
+// Rows per warp's item: the items (strip, chunk of rows) of S shots go to `warps` resident warps in rounds of equal
+// length; the split of the rows with the least rounds x (rows + 6, about what an item's start costs) wins.
+// Marmousi2-shaped, us per launch with the former aim of 4864 warps and with this: 32 shots 69 / 60, 50 shots 100 / 87,
+// 100 shots 178 / 169.
+int chunk_rows(int rows, int nstrip, int S, long long warps, long long *cost_out)
+{
+    long long best = -1;
+    int best_zc = rows;
+    for (int c = 1; c <= (rows + 1) / 2; ++c) {
+        const int zc = (rows + c - 1) / c;
+        const long long items = (long long)nstrip * S * ((rows + zc - 1) / zc);
+        const long long cost = (items + warps - 1) / warps * (zc + 6);
+        if (best < 0 || cost <= best) { best = cost; best_zc = zc; }   // ties: the more, shorter items
+    }
+    if (cost_out) *cost_out = std::max(best, 0LL);
+    return std::max(best_zc, 1);
 }
 
 cudaError_t launch_prop(const PropArgs &a, int nshot, cudaStream_t st)
