@@ -55,6 +55,8 @@ struct fwime_ctx {
     size_t max_ws = 0;
     int device = 0;
     size_t dev_mem = 0;             // total memory of the device
+    int coop_sms = 0;               // SMs for cooperative launches (0: not supported)
+    unsigned *d_bar = nullptr;      // grid barrier of the many-step launches: arrivals, generation
     // options
     int opt_S = 0, opt_K = 0, opt_plain = 0, opt_graph = 0, opt_host_io = 0, opt_zchunk = 0, opt_reuse_bg = 0;
     int opt_tlag = 0;               // > 0: B~ / B~* extend with time lags spaced opt_tlag steps
@@ -123,6 +125,12 @@ fwime_ctx *ctx_for_server(Server *srv)
 }
 Server *ctx_server(const fwime_ctx *x) { return x ? x->srv : nullptr; }
 void ctx_set_shared(fwime_ctx *x) { x->shared = true; }
+
+// No other stream's work is expected beside this context's: it runs on the default stream, where calls follow one
+// another whoever makes them.  Only then is one call's latency bought with the whole chip (many steps per cooperative
+// launch, items of a few rows): on streams of their own, eight threads with one small shot each complete 657 calls/s
+// without either, 463 with the short items and 316 with both.
+static bool alone(const fwime_ctx *x) { return !x->shared && x->st == nullptr; }
 }  // namespace fwk
 
 // operator entry points refuse a server context
@@ -564,10 +572,10 @@ static void init_run(fwime_ctx *x, Run &r, int S)
     r.nstrip = (x->NXP + STRIP - 1) / STRIP;
     int zc = x->opt_zchunk;
     if (zc <= 0) {
-        // 4 CTAs of 4 warps per SM.  Beside other requests the total work counts, not one launch's latency: items of a
+        // 4 CTAs of 4 warps per SM.  Beside other streams the total work counts, not one launch's latency: items of a
         // few rows load three times the rows that they write.
         zc = chunk_rows(rows, r.nstrip, std::max(S, 1), 152LL * 16, nullptr);
-        if (x->shared) zc = std::max(zc, 8);
+        if (!alone(x)) zc = std::max(zc, 8);
     }
     r.zchunk = zc;
     r.nchunk = (rows + zc - 1) / zc;
@@ -597,10 +605,21 @@ struct InjFrom {
     const float *val = nullptr;
 };
 
-static int prop(Run &r, int Sb, const float *cur, const float *prev, float *out, float *d2, const float *wsrc,
-                int src_shot0, const float *f0 = nullptr, float a0 = 0.f, const float *f1 = nullptr, float a1 = 0.f,
-                const float *f2 = nullptr, float a2 = 0.f, const float *coef = nullptr, const float *fc = nullptr,
-                RecTo rec = RecTo{}, InjFrom inj = InjFrom{})
+// Compulsory bytes of a stencil step: per shot-point read q^n, q^{n-1}, write q^{n+1}, and per point once per launch
+// the shared c, over the padded grid; D2t out and the local source fields (and coef) over the physical rows only
+// (zero elsewhere, not needed there); receivers.
+static double prop_bytes(const fwime_ctx *x, const PropArgs &a, int Sb)
+{
+    const double pts = (double)x->NZ * x->NX, spts = (double)x->g.nz * x->NX;
+    const double srcb = (a.d2 ? 4 : 0) + 4.0 * ((a.f0 != nullptr) + (a.f1 != nullptr) + (a.f2 != nullptr)) + (a.fc ? 4 : 0);
+    const double recb = (a.rec_d ? (double)Sb * x->nrec * (a.rec_acc ? 12.0 : 8.0) : 0.0) +
+                        (a.inj_val ? (double)Sb * x->nrec * 4.0 : 0.0);
+    return pts * (Sb * 12.0 + 4.0) + spts * (Sb * srcb + (a.coef ? 4.0 : 0.0)) + recb;
+}
+
+static PropArgs prop_args(Run &r, const float *cur, const float *prev, float *out, float *d2, const float *wsrc,
+                          int src_shot0, const float *f0, float a0, const float *coef, const float *fc, RecTo rec,
+                          InjFrom inj)
 {
     fwime_ctx *x = r.x;
     PropArgs a = r.base;
@@ -611,7 +630,7 @@ static int prop(Run &r, int Sb, const float *cur, const float *prev, float *out,
         a.src_amp = wsrc;
         a.src_stride = x->g.nt;
     }
-    a.f0 = f0; a.a0 = a0; a.f1 = f1; a.a1 = a1; a.f2 = f2; a.a2 = a2; a.coef = coef; a.fc = fc;
+    a.f0 = f0; a.a0 = a0; a.coef = coef; a.fc = fc;
     if (rec.d) {
         a.rec_off = x->d_rec_off; a.rec_d = rec.d; a.rec_dstride = (long long)x->g.nt * x->nrec;
         a.nrec = x->nrec; a.rec_acc = rec.acc;
@@ -620,15 +639,77 @@ static int prop(Run &r, int Sb, const float *cur, const float *prev, float *out,
         a.inj_map = x->d_inj_map; a.inj_next = x->d_inj_next; a.inj_val = inj.val;
         a.inj_vstride = (long long)x->g.nt * x->nrec; a.inj_lo = x->inj_lo; a.inj_hi = x->inj_hi;
     }
-    // compulsory bytes: per shot-point read q^n, q^{n-1}, write q^{n+1}, and per point once per launch
-    // the shared c, over the padded grid; D2t out and the local source fields (and coef) over the
-    // physical rows only (zero elsewhere, not needed there)
-    const double pts = (double)x->NZ * x->NX, spts = (double)x->g.nz * x->NX;
-    const double srcb = (d2 ? 4 : 0) + 4.0 * ((f0 != nullptr) + (f1 != nullptr) + (f2 != nullptr)) + (fc ? 4 : 0);
-    const double recb = (rec.d ? (double)Sb * x->nrec * (rec.acc ? 12.0 : 8.0) : 0.0) +
-                        (inj.val ? (double)Sb * x->nrec * 4.0 : 0.0);
-    LAUNCH(FWIME_K_PROP, pts * (Sb * 12.0 + 4.0) + spts * (Sb * srcb + (coef ? 4.0 : 0.0)) + recb,
-           launch_prop(a, Sb, x->st));
+    return a;
+}
+
+static int prop(Run &r, int Sb, const float *cur, const float *prev, float *out, float *d2, const float *wsrc,
+                int src_shot0, const float *f0 = nullptr, float a0 = 0.f, const float *f1 = nullptr, float a1 = 0.f,
+                const float *f2 = nullptr, float a2 = 0.f, const float *coef = nullptr, const float *fc = nullptr,
+                RecTo rec = RecTo{}, InjFrom inj = InjFrom{})
+{
+    fwime_ctx *x = r.x;
+    PropArgs a = prop_args(r, cur, prev, out, d2, wsrc, src_shot0, f0, a0, coef, fc, rec, inj);
+    a.f1 = f1; a.a1 = a1; a.f2 = f2; a.a2 = a2;
+    LAUNCH(FWIME_K_PROP, prop_bytes(x, a, Sb), launch_prop(a, Sb, x->st));
+    return FWIME_OK;
+}
+
+// A run of time steps whose operands move by fixed strides.  Fields: cur and prev swap (every step writes over
+// prev; after an odd number of steps the caller swaps), or, with R > 0, slots of the ring `ring` (SP floats apart)
+// for m = m0, m0 - 1, ...: slot m from m + 1 and m + 2.
+struct Steps {
+    float *cur = nullptr, *prev = nullptr;
+    float *ring = nullptr;
+    int R = 0, m0 = 0;
+    float *d2 = nullptr;
+    long long d2_step = 0;
+    const float *wsrc = nullptr;    // source amplitude of the first step (the next one follows)
+    int shot0 = 0;
+    const float *f0 = nullptr;      // local source of weight 1
+    long long f0_step = 0;
+    const float *coef = nullptr, *fc = nullptr;
+    long long fc_step = 0;
+    float *rec = nullptr;           // data row of the first step (the next row follows)
+    int rec_acc = 0;
+    const float *inj = nullptr;     // data row of the first step (the row before follows)
+};
+constexpr int MARCH_STEPS = 256;    // steps per launch at most: other streams get the SMs in between
+
+static int steps(Run &r, int Sb, int n, const Steps &p)
+{
+    fwime_ctx *x = r.x;
+    const long long SP = (long long)r.w.S * x->P;
+    const auto slot = [&](int m) { return p.ring + (m % p.R) * SP; };
+    // operands of step k
+    const auto args = [&](int k) {
+        float *c = p.R ? slot(p.m0 - k + 1) : k & 1 ? p.prev : p.cur, *q = p.R ? slot(p.m0 - k + 2) : k & 1 ? p.cur : p.prev;
+        return prop_args(r, c, q, p.R ? slot(p.m0 - k) : q, p.d2 ? p.d2 + k * p.d2_step : nullptr,
+                         p.wsrc ? p.wsrc + k : nullptr, p.shot0, p.f0 ? p.f0 + k * p.f0_step : nullptr, p.f0 ? 1.f : 0.f,
+                         p.coef, p.fc ? p.fc + k * p.fc_step : nullptr,
+                         RecTo{p.rec ? p.rec + (long long)k * x->nrec : nullptr, p.rec_acc},
+                         InjFrom{p.inj ? p.inj - (long long)k * x->nrec : nullptr});
+    };
+    // few shots on a small grid: many steps per launch (not in the plain path, nor where every step is timed, nor
+    // beside other streams, whose launches a cooperative one would wait for and hold up)
+    const bool many = n > 2 && x->coop_sms > 0 && alone(x) && !x->opt_plain && !x->opt_profile &&
+                      march_pays(args(0), Sb, x->coop_sms);
+    for (int k = 0; k < n;) {
+        const PropArgs a = args(k);
+        if (!many) {
+            LAUNCH(FWIME_K_PROP, prop_bytes(x, a, Sb), launch_prop(a, Sb, x->st));
+            ++k;
+            continue;
+        }
+        MarchArgs m{};
+        m.a = a;
+        m.nsteps = std::min(n - k, MARCH_STEPS);
+        m.S = Sb;
+        m.ring = p.ring; m.rstride = SP; m.R = p.R; m.m0 = p.m0 - k;
+        m.d2_step = p.d2_step; m.f0_step = p.f0_step; m.fc_step = p.fc_step; m.rec_step = x->nrec; m.inj_step = -x->nrec;
+        m.bar = x->d_bar; m.status = x->d_status;
+        LAUNCH(FWIME_K_PROP, m.nsteps * prop_bytes(x, a, Sb), launch_march(m, x->coop_sms, x->st));
+        k += m.nsteps;
+    }
     return FWIME_OK;
 }
 
@@ -838,11 +919,10 @@ static int run_forward(fwime_ctx *x, Run &r, const float *v, const float *w, flo
         float *db = d + s0 * nd;
         TRY(zero(x, db, sizeof(float) * Sb * nd));
         // the launch of step n records its input q^n; the last sample q^{nt-1} is recorded after the loop
-        for (int n = 0; n + 1 < nt; ++n) {
-            TRY(prop(r, Sb, cur, prv, prv, nullptr, w + (size_t)s0 * nt + n, s0, nullptr, 0.f, nullptr, 0.f, nullptr,
-                     0.f, nullptr, nullptr, RecTo{db + (size_t)n * x->nrec, 0}));
-            std::swap(cur, prv);
-        }
+        Steps sp;
+        sp.cur = cur; sp.prev = prv; sp.wsrc = w + (size_t)s0 * nt; sp.shot0 = s0; sp.rec = db;
+        TRY(steps(r, Sb, nt - 1, sp));
+        if ((nt - 1) & 1) std::swap(cur, prv);
         TRY(record(r, Sb, cur, nullptr, db + (size_t)(nt - 1) * x->nrec, 0));
     }
     return FWIME_OK;
@@ -903,17 +983,17 @@ static int run_born_ext(fwime_ctx *x, Run &r, const float *v, const float *w, co
                 TRY(copyf(x, bg_slot(x, n0 / K, 0, s0), c0, (size_t)Sb * x->P));
                 TRY(copyf(x, bg_slot(x, n0 / K, 1, s0), p0, (size_t)Sb * x->P));
             }
-            for (int n = n0; n < n1; ++n) {
-                TRY(prop(r, Sb, c0, p0, p0, keep ? bg_d2t(x, n, s0) : Dr + (n - n0) * SP, w + (size_t)s0 * nt + n, s0));
-                std::swap(c0, p0);
-            }
+            Steps bgs;
+            bgs.cur = c0; bgs.prev = p0; bgs.wsrc = w + (size_t)s0 * nt + n0; bgs.shot0 = s0;
+            bgs.d2 = keep ? bg_d2t(x, n0, s0) : Dr; bgs.d2_step = keep ? x->nshot * x->P : SP;
+            TRY(steps(r, Sb, kk, bgs));
+            if (kk & 1) std::swap(c0, p0);
             const RingRef dring = keep ? ringref(bg_d2t(x, n0, s0), x->nshot * x->P, 0, 0) : ringref(Dr, SP, 0, 0);
             TRY(scatter(r, Sb, n0, kk, r.w.W, dring, ringref(Er, SP, 0, 0), +1, 0));
-            for (int n = n0; n < n1; ++n) {
-                TRY(prop(r, Sb, c1, p1, p1, nullptr, nullptr, 0, Er + (n - n0) * SP, 1.f, nullptr, 0.f, nullptr, 0.f,
-                         nullptr, nullptr, RecTo{db + (size_t)n * x->nrec, 0}));
-                std::swap(c1, p1);
-            }
+            Steps scs;
+            scs.cur = c1; scs.prev = p1; scs.f0 = Er; scs.f0_step = SP; scs.rec = db + (size_t)n0 * x->nrec;
+            TRY(steps(r, Sb, kk, scs));
+            if (kk & 1) std::swap(c1, p1);
         }
         TRY(record(r, Sb, c1, nullptr, db + (size_t)(nt - 1) * x->nrec, 0));
     }
@@ -943,18 +1023,17 @@ static int run_born_adj(fwime_ctx *x, Run &r, bool ext, const float *v, const fl
         // background cache, or a forward sweep)
         const bool kept = r.w.hist || (use_bg && x->bg.hist);
         auto ckp = [&](int j, int t) -> float * { return use_bg ? bg_slot(x, j, t, s0) : ck + (2LL * j + t) * SP; };
-        for (int n = 0; n + 1 < nt && r.w.hist; ++n) {
-            TRY(prop(r, Sb, cur, prv, prv, Dr + n * SP, ws + n, s0));
-            std::swap(cur, prv);
-        }
+        Steps fw;
+        fw.cur = cur; fw.prev = prv; fw.wsrc = ws; fw.shot0 = s0; fw.d2 = Dr; fw.d2_step = SP;
+        if (r.w.hist) TRY(steps(r, Sb, nt - 1, fw));
         for (int j = 0; j < nseg && !use_bg && !kept; ++j) {
             TRY(copyf(x, ck + (2LL * j) * SP, cur, (size_t)Sb * x->P));
             TRY(copyf(x, ck + (2LL * j + 1) * SP, prv, (size_t)Sb * x->P));
             if (j == nseg - 1) break;
-            for (int n = j * K; n < (j + 1) * K; ++n) {
-                TRY(prop(r, Sb, cur, prv, prv, nullptr, ws + n, s0));
-                std::swap(cur, prv);
-            }
+            Steps ck_fw;
+            ck_fw.cur = cur; ck_fw.prev = prv; ck_fw.wsrc = ws + j * K; ck_fw.shot0 = s0;
+            TRY(steps(r, Sb, K, ck_fw));
+            if (K & 1) std::swap(cur, prv);
         }
         // backward sweep
         for (int j = nseg - 1; j >= 0; --j) {
@@ -962,18 +1041,15 @@ static int run_born_adj(fwime_ctx *x, Run &r, bool ext, const float *v, const fl
             if (!kept) {
                 TRY(copyf(x, cur, ckp(j, 0), (size_t)Sb * x->P));
                 TRY(copyf(x, prv, ckp(j, 1), (size_t)Sb * x->P));
-                for (int n = n0; n < n1; ++n) {
-                    TRY(prop(r, Sb, cur, prv, prv, Dr + (n - n0) * SP, ws + n, s0));
-                    std::swap(cur, prv);
-                }
+                fw.cur = cur; fw.prev = prv; fw.wsrc = ws + n0;
+                TRY(steps(r, Sb, kk, fw));
             }
             const RingRef dring = r.w.hist ? ringref(Dr + n0 * SP, SP, 0, 0)
                                   : kept   ? ringref(bg_d2t(x, n0, s0), x->nshot * x->P, 0, 0)
                                            : ringref(Dr, SP, 0, 0);
-            for (int m = n1; m >= n0 + 1; --m) {
-                float *mo = Mu + (m % R) * SP;
-                TRY(adj_step(r, Sb, Mu + ((m + 1) % R) * SP, Mu + ((m + 2) % R) * SP, mo, d + s0 * nd + (size_t)m * x->nrec));
-            }
+            Steps ad;
+            ad.ring = Mu; ad.R = R; ad.m0 = n1; ad.inj = d + s0 * nd + (size_t)n1 * x->nrec;
+            TRY(steps(r, Sb, kk, ad));
             if (ext)
                 TRY(image(r, Sb, n0, kk, IMG_EXT, dring, ringref(Mu, SP, R, 1), ringref(nullptr, 0, 0, 0),
                           ringref(nullptr, 0, 0, 0), 1.f, r.w.acc1));
@@ -1336,27 +1412,24 @@ static int run_tomo(fwime_ctx *x, Run &r, const float *v, const float *w, const 
         const float *ws = w + (size_t)s0 * nt;
         for (int n0 = 0; n0 < nt - 1; n0 += K) {
             const int n1 = std::min(n0 + K, nt - 1), kk = n1 - n0;
-            for (int n = n0; n < n1; ++n) {   // background q0
-                TRY(prop(r, Sb, f[0], f[1], f[1], D0r + (n - n0) * SP, ws + n, s0));
-                std::swap(f[0], f[1]);
-            }
-            for (int n = n0; n < n1; ++n) {   // Born wavefield of dv
-                TRY(prop(r, Sb, f[2], f[3], f[3], D0d + (n - n0) * SP, nullptr, 0, nullptr, 0, nullptr, 0, nullptr, 0,
-                         r.w.coef, D0r + (n - n0) * SP));
-                std::swap(f[2], f[3]);
-            }
+            const auto run = [&](float *&cur, float *&prv, Steps sp) {
+                sp.cur = cur; sp.prev = prv;
+                if (kk & 1) std::swap(cur, prv);
+                return steps(r, Sb, kk, sp);
+            };
+            Steps q0, qd, qs, qt;
+            q0.wsrc = ws + n0; q0.shot0 = s0; q0.d2 = D0r; q0.d2_step = SP;
+            TRY(run(f[0], f[1], q0));         // background q0
+            qd.coef = r.w.coef; qd.fc = D0r; qd.fc_step = SP; qd.d2 = D0d; qd.d2_step = SP;
+            TRY(run(f[2], f[3], qd));         // Born wavefield of dv
             TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0r, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
-            for (int n = n0; n < n1; ++n) {   // extended Born wavefield of p~
-                TRY(prop(r, Sb, f[4], f[5], f[5], Dsr + (n - n0) * SP, nullptr, 0, Er + (n - n0) * SP, 1.f));
-                std::swap(f[4], f[5]);
-            }
+            qs.f0 = Er; qs.f0_step = SP; qs.d2 = Dsr; qs.d2_step = SP;
+            TRY(run(f[4], f[5], qs));         // extended Born wavefield of p~
             TRY(scatter(r, Sb, n0, kk, r.w.W2, ringref(D0r, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
             TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0d, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 1));
-            for (int n = n0; n < n1; ++n) {   // tomographic wavefield
-                TRY(prop(r, Sb, f[6], f[7], f[7], nullptr, nullptr, 0, Er + (n - n0) * SP, 1.f, nullptr, 0, nullptr, 0,
-                         r.w.coef, Dsr + (n - n0) * SP, RecTo{db + (size_t)n * x->nrec, 0}));
-                std::swap(f[6], f[7]);
-            }
+            qt.f0 = Er; qt.f0_step = SP; qt.coef = r.w.coef; qt.fc = Dsr; qt.fc_step = SP;
+            qt.rec = db + (size_t)n0 * x->nrec;
+            TRY(run(f[6], f[7], qt));         // tomographic wavefield
         }
         TRY(record(r, Sb, f[6], nullptr, db + (size_t)(nt - 1) * x->nrec, 0));
     }
@@ -1433,15 +1506,16 @@ static int run_tomo_adj(fwime_ctx *x, Run &r, int mode, const float *v, const fl
                 float *D0 = D0r + (r.w.hist ? n0 * SP : 0);
                 // with the gradient, the launch of step n adds its input (q0^n, then the scattered field's)
                 // to the prediction's row n (zeroed above; a + b is exact in either order of the two)
-                for (int n = n0; n < n1; ++n) {
-                    TRY(prop(r, Sb, q0c, q0p, q0p, D0 + (n - n0) * SP, ws + n, s0, nullptr, 0.f, nullptr, 0.f,
-                             nullptr, 0.f, nullptr, nullptr, RecTo{grad ? pred + (size_t)n * x->nrec : nullptr, 1}));
-                    std::swap(q0c, q0p);
-                }
+                Steps q0, qs;
+                q0.cur = q0c; q0.prev = q0p; q0.d2 = D0; q0.d2_step = SP; q0.wsrc = ws + n0; q0.shot0 = s0;
+                q0.rec = grad ? pred + (size_t)n0 * x->nrec : nullptr; q0.rec_acc = 1;
+                TRY(steps(r, Sb, kk, q0));
                 TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
-                for (int n = n0; n < n1; ++n) {
-                    TRY(prop(r, Sb, qsc, qsp, qsp, r.w.hist ? Dsr + n * SP : nullptr, nullptr, 0, Er + (n - n0) * SP, 1.f, nullptr, 0.f, nullptr,
-                             0.f, nullptr, nullptr, RecTo{grad ? pred + (size_t)n * x->nrec : nullptr, 1}));
+                qs.cur = qsc; qs.prev = qsp; qs.d2 = r.w.hist ? Dsr + n0 * SP : nullptr; qs.d2_step = SP;
+                qs.f0 = Er; qs.f0_step = SP; qs.rec = q0.rec; qs.rec_acc = 1;
+                TRY(steps(r, Sb, kk, qs));
+                if (kk & 1) {
+                    std::swap(q0c, q0p);
                     std::swap(qsc, qsp);
                 }
             }
@@ -1462,35 +1536,29 @@ static int run_tomo_adj(fwime_ctx *x, Run &r, int mode, const float *v, const fl
                 TRY(copyf(x, q0p, ckp(j, 1), fn));
                 TRY(copyf(x, qsc, ckp(j, 2), fn));
                 TRY(copyf(x, qsp, ckp(j, 3), fn));
-                for (int n = n0; n < n1; ++n) {
-                    TRY(prop(r, Sb, q0c, q0p, q0p, D0r + (n - n0) * SP, ws + n, s0));
-                    std::swap(q0c, q0p);
-                }
+                Steps q0, qs;
+                q0.cur = q0c; q0.prev = q0p; q0.d2 = D0r; q0.d2_step = SP; q0.wsrc = ws + n0; q0.shot0 = s0;
+                TRY(steps(r, Sb, kk, q0));
                 TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0r, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
-                for (int n = n0; n < n1; ++n) {
-                    TRY(prop(r, Sb, qsc, qsp, qsp, Dsr + (n - n0) * SP, nullptr, 0, Er + (n - n0) * SP, 1.f));
-                    std::swap(qsc, qsp);
-                }
+                qs.cur = qsc; qs.prev = qsp; qs.d2 = Dsr; qs.d2_step = SP; qs.f0 = Er; qs.f0_step = SP;
+                TRY(steps(r, Sb, kk, qs));
             }
             const RingRef d0ring = ringref(D0r + (r.w.hist ? n0 * SP : 0), SP, 0, 0);
             const RingRef dsring = ringref(Dsr + (r.w.hist ? n0 * SP : 0), SP, 0, 0);
             // adjoint of the residual: mu^m, m = n1 .. n0+1 (lambda^ at step n is mu^{n+1}), each step also
             // writing its D2t, (mu^m - 2 mu^{m+1} + mu^{m+2}) / dt^2, at slot m - n0 - 1 of Zr
-            for (int m = n1; m >= n0 + 1; --m) {
-                float *mo = Mu + (m % R) * SP;
-                TRY(adj_step(r, Sb, Mu + ((m + 1) % R) * SP, Mu + ((m + 2) % R) * SP, mo, rr + (size_t)m * x->nrec,
-                             Zr + (m - n0 - 1) * SP));
-            }
+            Steps ad;
+            ad.ring = Mu; ad.R = R; ad.m0 = n1; ad.inj = rr + (size_t)n1 * x->nrec; ad.d2 = Zr + (kk - 1) * SP; ad.d2_step = -SP;
+            TRY(steps(r, Sb, kk, ad));
             // The second adjoint field's source d2t^T z, z^n = E_D^T(W, lambda^n): E_D^T acts on space only,
             // so y^m = (z^{m-1} - 2 z^m + z^{m+1}) / dt^2 = E_D^T(W, D2t of the step producing mu^m): one
             // transposed scatter of those D2t into slots m - n0 - 1 of the scattered-field ring (free again
             // once the recomputed q_s is past this segment; zero outside the scatter's columns, which only
             // scatters write)
             TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(Zr, SP, 0, 0), ringref(Er, SP, 0, 0), -1, 0));
-            for (int m = n1; m >= n0 + 1; --m) {
-                TRY(prop(r, Sb, Mu2 + ((m + 1) % R) * SP, Mu2 + ((m + 2) % R) * SP, Mu2 + (m % R) * SP, nullptr,
-                         nullptr, 0, Er + (m - n0 - 1) * SP, 1.f));
-            }
+            Steps a2;
+            a2.ring = Mu2; a2.R = R; a2.m0 = n1; a2.f0 = Er + (kk - 1) * SP; a2.f0_step = -SP;
+            TRY(steps(r, Sb, kk, a2));
             // the extended image of the residual's adjoint field (contracted with p~ at the end) and, in the
             // same launch, the local terms D0 (alpha lambda^ + mu2) + Ds lambda^
             TRY(image(r, Sb, n0, kk, IMG_EXT, d0ring, ringref(Mu, SP, R, 1), ringref(Mu2, SP, R, 1), dsring,
@@ -1748,6 +1816,10 @@ int fwime_create(fwime_ctx **out, const fwime_grid *g, const fwime_geom *geo, si
         cudaGetLastError();
         x->dev_mem = 0;
     }
+    int coop = 0, nsm = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, x->device) == cudaSuccess && coop &&
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, x->device) == cudaSuccess)
+        x->coop_sms = nsm;
     // offsets: [src_off(nshot)][rec_off(nrec)]
     x->h_off.resize(x->nshot + x->nrec);
     for (int s = 0; s < x->nshot; ++s) x->h_off[s] = (x->src_iz[s] + x->o) * x->NXP + x->src_ix[s] + x->o;
@@ -1772,7 +1844,7 @@ int fwime_create(fwime_ctx **out, const fwime_grid *g, const fwime_geom *geo, si
             last[pos] = r;
         }
     }
-    const size_t off_inj = ((1 + 1024) * sizeof(double) + sizeof(int) * (1 + x->h_off.size()) + 15) / 16 * 16;
+    const size_t off_inj = ((1 + 1024) * sizeof(double) + sizeof(int) * (3 + x->h_off.size()) + 15) / 16 * 16;
     const size_t small_bytes = off_inj + sizeof(int) * x->h_inj.size();
     double *slot = pinned_slot();
     bool ok = slot != nullptr &&
@@ -1783,7 +1855,8 @@ int fwime_create(fwime_ctx **out, const fwime_grid *g, const fwime_geom *geo, si
         x->d_J = reinterpret_cast<double *>(x->small);
         x->d_part = x->d_J + 1;
         x->d_status = reinterpret_cast<int *>(x->d_part + 1024);
-        x->d_src_off = x->d_status + 1;
+        x->d_bar = reinterpret_cast<unsigned *>(x->d_status + 1);
+        x->d_src_off = x->d_status + 3;
         x->d_rec_off = x->d_src_off + x->nshot;
         x->d_inj_map = reinterpret_cast<int *>(reinterpret_cast<char *>(x->small) + off_inj);
         x->d_inj_next = x->d_inj_map + nmap;
@@ -2174,10 +2247,10 @@ int fwime_forward_group(fwime_ctx *const *ctxs, int n, const float *const *v, co
         TRY(plan(m, FWIME_OP_FORWARD, runs[i].w));
         if (runs[i].w.S < m->nshot)
             return fail(x, FWIME_ENOMEM, "group member %d: %d shots do not fit one batch", i, m->nshot);
-        const bool alone = !m->shared;
-        if (n > 1) m->shared = true;   // the members fill the launch together
+        const bool was = m->shared;
+        m->shared = was || n > 1;      // the members fill the launch together
         init_run(m, runs[i], m->nshot);
-        if (alone) m->shared = false;
+        m->shared = was;
         const long long before = m->launches;
         TRY(prep_model(m, runs[i], v[i]));
         if (m != x) x->launches += m->launches - before;   // the group's count includes every member's prep
@@ -2488,6 +2561,10 @@ int fwime_sync(fwime_ctx *x)
             CK(cudaMemcpy(x->vp_hist_user, x->vp_hist_dev, x->vp_hist_n * sizeof(double), cudaMemcpyDeviceToHost));
         CK(cudaFreeAsync(x->vp_hist_dev, x->st));
         x->vp_hist_dev = x->vp_hist_user = nullptr;
+    }
+    if (st & ST_TIMEOUT) {
+        CK(cudaMemsetAsync(x->d_bar, 0, 2 * sizeof(unsigned), x->st));
+        return fail(x, FWIME_ETIMEOUT, "a many-step launch gave up waiting at its grid barrier");
     }
     if (st & ST_CFL) return fail(x, FWIME_ECFL, "velocity violates the CFL bound or is not positive");
     return FWIME_OK;

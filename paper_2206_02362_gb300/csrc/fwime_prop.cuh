@@ -252,29 +252,31 @@ __device__ __forceinline__ void row_math(const PropArgs &a, const PropK &K, cons
 
 // Adds the injections of the receivers chained from r at one output point: o + c v per receiver, each
 // product and sum rounded separately (the arithmetic of a separate injection launch after the step).
-__device__ __forceinline__ void inject_point(const PropArgs &a, int shot, int r, float c, float &o)
+__device__ __forceinline__ void inject_point(const PropArgs &a, const float *val, int shot, int r, float c, float &o)
 {
     for (; r >= 0; r = __ldg(a.inj_next + r))
-        o = __fadd_rn(o, __fmul_rn(c, __ldg(a.inj_val + (long long)shot * a.inj_vstride + r)));
+        o = __fadd_rn(o, __fmul_rn(c, __ldg(val + (long long)shot * a.inj_vstride + r)));
 }
 
 // The time step of one warp's work item (strip, chunk) of shot `shot`; wsm is the warp's shared
-// memory (CUR_SLOTS x CUR_ROW + AUX_SLOTS x naux_max x STRIP floats).
-template <int LOC, bool D2, bool SRC, bool INJ = false, bool FS = false>
-__device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, const int shot, float *wsm)
+// memory (CUR_SLOTS x CUR_ROW + AUX_SLOTS x naux_max x STRIP floats).  sp: the operands that change from step to step
+// (the same members of PropArgs).  COH: the fields change during the kernel (several steps per launch), so no read of
+// them may come from a non-coherent cache.
+template <int LOC, bool D2, bool SRC, bool INJ, bool FS, bool COH, class SP>
+__device__ __forceinline__ void prop_body(const PropArgs &a, const SP &sp, const int wid, const int shot, float *wsm)
 {
     constexpr bool LOCAL = LOC > 0;
     const int lane = threadIdx.x & 31;
     const int strip = wid % a.nstrip, chunk = wid / a.nstrip;
     const int x0 = strip * STRIP;
     const int x = x0 + lane * 4;
-    const int z0 = (FS ? a.z_first : 4) + chunk * a.zchunk;
+    const int z0 = (FS || COH ? a.z_first : 4) + chunk * a.zchunk;
     const int z1 = min(z0 + a.zchunk, a.NZ - 4);
     const bool xin = x < a.NXP;
     const long long so = (long long)shot * a.P;
-    const float *__restrict__ cur = a.cur + so;
-    const float *prev = a.prev + so;
-    float *out = a.out + so;
+    const float *__restrict__ cur = sp.cur + so;
+    const float *prev = sp.prev + so;
+    float *out = sp.out + so;
     const long long NXP = a.NXP;
 
     // aux row layout: [prev][c][f0?][f1?][f2?][coef, fc?]
@@ -311,14 +313,14 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, cons
             // local sources vanish outside the source rows: zero-filled there, not read
             const bool lin = xin && zr >= a.zs_lo && zr < a.zs_hi;
             if (LOC == 1) {
-                cp16(dst + i_f0 * STRIP, a.f0 + so + o2, lin);
+                cp16(dst + i_f0 * STRIP, sp.f0 + so + o2, lin);
             } else {
-                if (a.f0) cp16(dst + i_f0 * STRIP, a.f0 + so + o2, lin);
+                if (a.f0) cp16(dst + i_f0 * STRIP, sp.f0 + so + o2, lin);
                 if (a.f1) cp16(dst + i_f1 * STRIP, a.f1 + so + o2, lin);
                 if (a.f2) cp16(dst + i_f2 * STRIP, a.f2 + so + o2, lin);
                 if (a.fc) {
                     cp16(dst + i_cf * STRIP, a.coef + o2, lin);
-                    cp16(dst + (i_cf + 1) * STRIP, a.fc + so + o2, lin);
+                    cp16(dst + (i_cf + 1) * STRIP, sp.fc + so + o2, lin);
                 }
             }
         }
@@ -327,7 +329,10 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, cons
     // register queue rows z0-4 .. z0+3
     float4 q[9];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) q[k] = xin ? ldg4(cur + (long long)(z0 - 4 + k) * NXP + x) : f4zero();
+    for (int k = 0; k < 8; ++k) {
+        const float *qp = cur + (long long)(z0 - 4 + k) * NXP + x;
+        q[k] = !xin ? f4zero() : COH ? __ldcg(reinterpret_cast<const float4 *>(qp)) : ldg4(qp);
+    }
     // prologue: one group per iteration of look-ahead (rows z0 .. z0+3 feed the first x-taps)
 #pragma unroll
     for (int g = 0; g < AUX_SLOTS; ++g) {
@@ -343,7 +348,7 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, cons
     float amp = 0.f;
     if (SRC) {
         soff = a.src_off[shot];
-        amp = a.src_amp[(long long)shot * a.src_stride] * a.src_scale;
+        amp = sp.src_amp[(long long)shot * a.src_stride] * a.src_scale;
     }
 
     // One output row zz; the queue's logical row k (zz-4+k) lives in q[(k + R) % 9], so nine
@@ -382,7 +387,7 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, cons
                                  q[(8 + (R)) % 9], Rr, pv, cv, lf0, lf1, lf2, lcf, lfc, gzz, gxv, sj, amp, o, d2); \
         if (xin) {                                                                                           \
             st4(out + idx, o);                                                                               \
-            if (D2 && zz >= a.zs_lo && zz < a.zs_hi) st4(a.d2 + so + idx, d2);                               \
+            if (D2 && zz >= a.zs_lo && zz < a.zs_hi) st4(sp.d2 + so + idx, d2);                               \
         }                                                                                                    \
         __syncwarp(); /* every lane is done with this row's slots before they are refilled */              \
         issue_cur(zz + 4 + AUX_SLOTS);                                                                       \
@@ -413,14 +418,14 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, cons
             const float4 o0 = *reinterpret_cast<const float4 *>(out + idx);
             float4 o = o0;
             const float4 cv = ldg4(a.c + idx);
-            inject_point(a, shot, m4.x, cv.x, o.x);
-            inject_point(a, shot, m4.y, cv.y, o.y);
-            inject_point(a, shot, m4.z, cv.z, o.z);
-            inject_point(a, shot, m4.w, cv.w, o.w);
+            inject_point(a, sp.inj_val, shot, m4.x, cv.x, o.x);
+            inject_point(a, sp.inj_val, shot, m4.y, cv.y, o.y);
+            inject_point(a, sp.inj_val, shot, m4.z, cv.z, o.z);
+            inject_point(a, sp.inj_val, shot, m4.w, cv.w, o.w);
             st4(out + idx, o);
             if (D2 && zz >= a.zs_lo && zz < a.zs_hi) {
                 // the D2t output gains the injection too: d2 + (o - o0) / dt^2
-                float *dp = a.d2 + so + idx;
+                float *dp = sp.d2 + so + idx;
                 float4 d = *reinterpret_cast<const float4 *>(dp);
                 d.x = fmaf(o.x - o0.x, a.inv_dt2, d.x);
                 d.y = fmaf(o.y - o0.y, a.inv_dt2, d.y);
@@ -430,17 +435,17 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, cons
             }
         }
     }
-    if (FS && xin) {
+    if ((FS || COH) && a.fs_row > 0 && xin) {
         // Free surface (pressure release on row fs_row, where the march starts): q = 0 and D2t = 0 there, and the four
         // rows above hold the odd mirror of the four below, each written by the lane that owns the row below (which
-        // it reads back: its own stores, injection included); rows further up stay zero.  As a launch of its own after every step this took 6.6 us, a fifth of
-        // an objective call (16 shots on 302 x 1001 points).
+        // it reads back: its own stores, injection included); rows further up stay zero.  As a launch of its own
+        // after every step this took 6.6 us, a fifth of an objective call (16 shots on 302 x 1001 points).
         const int zlo = max(z0, a.fs_row), zhi = min(z1, a.fs_row + 5);
         for (int zz = zlo; zz < zhi; ++zz) {
             const long long idx = (long long)zz * NXP + x;
             if (zz == a.fs_row) {
                 st4(out + idx, f4zero());
-                if (D2) st4(a.d2 + so + idx, f4zero());
+                if (D2) st4(sp.d2 + so + idx, f4zero());
             } else {
                 const float4 o = *reinterpret_cast<const float4 *>(out + idx);
                 st4(out + (long long)(2 * a.fs_row - zz) * NXP + x, make_float4(-o.x, -o.y, -o.z, -o.w));
@@ -453,7 +458,9 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, cons
 // INJ: the receivers' injection into the output (the adjoint step; LOC = 0, no point source; with D2 the
 // injection reaches the D2t output as well)
 template <int LOC, bool D2, bool SRC, bool INJ, bool FS>
-__global__ void __launch_bounds__(PROP_WARPS * 32, LOC == 2 ? FWIME_PROP_MIN_BLOCKS : (LOC == 1 ? FWIME_PROP_MINB_LOC1 : FWIME_PROP_MINB_PLAIN)) k_prop(const PropArgs a)
+__global__ void __launch_bounds__(PROP_WARPS * 32, LOC == 2 ? FWIME_PROP_MIN_BLOCKS
+                                                            : (LOC == 1 ? FWIME_PROP_MINB_LOC1 : FWIME_PROP_MINB_PLAIN))
+    k_prop(const PropArgs a)
 {
     extern __shared__ float4 smem4[];
     if (a.rec_d && blockIdx.x == 0) {         // receivers of the input field (the previous step's output)
@@ -468,7 +475,7 @@ __global__ void __launch_bounds__(PROP_WARPS * 32, LOC == 2 ? FWIME_PROP_MIN_BLO
     const int wid = blockIdx.x * PROP_WARPS + wic;
     if (wid >= a.nstrip * a.nchunk) return;   // warp-uniform
     float *wsm = reinterpret_cast<float *>(smem4) + wic * (CUR_SLOTS * CUR_ROW + AUX_SLOTS * a.naux_max * STRIP);
-    prop_body<LOC, D2, SRC, INJ, FS>(a, wid, blockIdx.y, wsm);
+    prop_body<LOC, D2, SRC, INJ, FS, false>(a, a, wid, blockIdx.y, wsm);
 }
 
 template <bool FS, int LOC, bool D2, bool SRC, bool INJ = false>

@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(PROP_WARPS * 32, 4) k_prop_group(const GroupMe
     const int wid = (local - shot * cps) * PROP_WARPS + wic;
     if (wid >= sa.nstrip * sa.nchunk) return;   // warp-uniform
     float *wsm = reinterpret_cast<float *>(smem4) + wic * (CUR_SLOTS * CUR_ROW + AUX_SLOTS * 2 * STRIP);
-    prop_body<0, false, true>(sa, wid, shot, wsm);
+    prop_body<0, false, true, false, false, false>(sa, sa, wid, shot, wsm);
 }
 
 // after step n the new field q^{n+1} of a member is in buffer B for even n, A for odd n
