@@ -463,6 +463,10 @@ __global__ void __launch_bounds__(PROP_WARPS * 32, LOC == 2 ? FWIME_PROP_MIN_BLO
     k_prop(const PropArgs a)
 {
     extern __shared__ float4 smem4[];
+    // Launched while the previous launch's last CTAs still run (below): its results are there after the wait.  Only
+    // this kernel lets its successor in early, and after its own wait, so whatever older launches wrote is there too.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (a.rec_d && blockIdx.x == 0) {         // receivers of the input field (the previous step's output)
         const long long s = blockIdx.y;
         for (int r = threadIdx.x; r < a.nrec; r += PROP_WARPS * 32) {
@@ -485,7 +489,19 @@ static void launch_prop_t(const PropArgs &a, dim3 grid, dim3 block, size_t smem,
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_prop<LOC, D2, SRC, INJ, FS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
     (void)attr;
-    k_prop<LOC, D2, SRC, INJ, FS><<<grid, block, smem, st>>>(a);
+    // The next step's CTAs come in as soon as this one's are all under way and wait there, so that a step starts
+    // without the launch gap: 2 to 3 us per step (100 shots on 408 x 1816 points 170 / 167 us, 30 shots 61 / 59 us).
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&cfg, k_prop<LOC, D2, SRC, INJ, FS>, a);   // the caller reads the last error
 }
 template <bool FS>
 static cudaError_t dispatch_prop(const PropArgs &a0, int nshot, cudaStream_t st)
