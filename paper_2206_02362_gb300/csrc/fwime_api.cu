@@ -337,6 +337,7 @@ struct WS {
     float *c, *bpad, *gz, *gx, *coef, *W, *W2, *ptp, *acc1, *acc2;
     // per batch
     float *f[8];
+    float *alt[2] = {nullptr, nullptr};   // two more fields, where they fit: the outputs of two-step launches
     float *ring[6];    // rings of K slots (ring[0..3]) and of R slots (ring[3..5] in adjoint ops)
     float *ckpt, *pred;
     // host-io staging
@@ -456,9 +457,14 @@ static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
     }
     w.S = std::max(S, 1);
     x->last_S = w.S;
-    const size_t need = fixed + per * (size_t)w.S + 4096;
+    size_t need = fixed + per * (size_t)w.S + 4096;
     if (x->max_ws && need > x->max_ws)
         return fail(x, FWIME_ENOMEM, "operator needs %zu bytes for S=%d, K=%d; budget %zu", need, w.S, w.K, x->max_ws);
+    const size_t alt_bytes = 2 * al((size_t)w.S * x->P) * sizeof(float);
+    const bool tlag_op = x->opt_tlag > 0 && op != FWIME_OP_FORWARD && op != FWIME_OP_BORN && op != FWIME_OP_BORN_ADJ;
+    const bool alt = op != FWIME_OP_BORN && !tlag_op && !x->opt_plain && !x->opt_fs && pair_pays(x->P, w.S) &&
+                     need + alt_bytes <= budget;
+    if (alt) need += alt_bytes;
     if (need > x->ws_bytes) {
         if (x->capturing) return fail(x, FWIME_EBUSY, "workspace growth during graph capture");
         // stream-ordered (re)allocation: no device-wide synchronisation, so contexts of other
@@ -507,6 +513,7 @@ static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
     for (auto &q : w.f) q = nullptr;
     for (auto &q : w.ring) q = nullptr;
     w.ckpt = w.pred = nullptr;
+    for (auto &q : w.alt) q = alt ? take(SP) : nullptr;
     int nf = 0, nk = 0, nr = 0, nck = 0;
     if (x->opt_tlag > 0 && op != FWIME_OP_FORWARD && op != FWIME_OP_BORN && op != FWIME_OP_BORN_ADJ) {
         const size_t RD = (size_t)w.K + 2 * tlag_Hs(x->g, x->opt_tlag), NB = tlag_blocks(x->g, w.K, x->opt_tlag);
@@ -561,6 +568,7 @@ static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
 struct Run {
     fwime_ctx *x;
     WS w;
+    float *alt[2] = {nullptr, nullptr};   // the free pair of fields (pair_reset)
     int zchunk, nstrip, nchunk;
     PropArgs base{};
 };
@@ -654,8 +662,7 @@ static int prop(Run &r, int Sb, const float *cur, const float *prev, float *out,
     return FWIME_OK;
 }
 
-// A run of time steps whose operands move by fixed strides.  Fields: cur and prev swap (every step writes over
-// prev; after an odd number of steps the caller swaps), or, with R > 0, slots of the ring `ring` (SP floats apart)
+// A run of time steps whose operands move by fixed strides.  Fields: cur and prev (at the end the last two steps), or, with R > 0, slots of the ring `ring` (SP floats apart)
 // for m = m0, m0 - 1, ...: slot m from m + 1 and m + 2.
 struct Steps {
     float *cur = nullptr, *prev = nullptr;
@@ -675,44 +682,6 @@ struct Steps {
 };
 constexpr int MARCH_STEPS = 256;    // steps per launch at most: other streams get the SMs in between
 
-static int steps(Run &r, int Sb, int n, const Steps &p)
-{
-    fwime_ctx *x = r.x;
-    const long long SP = (long long)r.w.S * x->P;
-    const auto slot = [&](int m) { return p.ring + (m % p.R) * SP; };
-    // operands of step k
-    const auto args = [&](int k) {
-        float *c = p.R ? slot(p.m0 - k + 1) : k & 1 ? p.prev : p.cur, *q = p.R ? slot(p.m0 - k + 2) : k & 1 ? p.cur : p.prev;
-        return prop_args(r, c, q, p.R ? slot(p.m0 - k) : q, p.d2 ? p.d2 + k * p.d2_step : nullptr,
-                         p.wsrc ? p.wsrc + k : nullptr, p.shot0, p.f0 ? p.f0 + k * p.f0_step : nullptr, p.f0 ? 1.f : 0.f,
-                         p.coef, p.fc ? p.fc + k * p.fc_step : nullptr,
-                         RecTo{p.rec ? p.rec + (long long)k * x->nrec : nullptr, p.rec_acc},
-                         InjFrom{p.inj ? p.inj - (long long)k * x->nrec : nullptr});
-    };
-    // few shots on a small grid: many steps per launch (not in the plain path, nor where every step is timed, nor
-    // beside other streams, whose launches a cooperative one would wait for and hold up)
-    const bool many = n > 2 && x->coop_sms > 0 && alone(x) && !x->opt_plain && !x->opt_profile &&
-                      march_pays(args(0), Sb, x->coop_sms);
-    for (int k = 0; k < n;) {
-        const PropArgs a = args(k);
-        if (!many) {
-            LAUNCH(FWIME_K_PROP, prop_bytes(x, a, Sb), launch_prop(a, Sb, x->st));
-            ++k;
-            continue;
-        }
-        MarchArgs m{};
-        m.a = a;
-        m.nsteps = std::min(n - k, MARCH_STEPS);
-        m.S = Sb;
-        m.ring = p.ring; m.rstride = SP; m.R = p.R; m.m0 = p.m0 - k;
-        m.d2_step = p.d2_step; m.f0_step = p.f0_step; m.fc_step = p.fc_step; m.rec_step = x->nrec; m.inj_step = -x->nrec;
-        m.bar = x->d_bar; m.status = x->d_status;
-        LAUNCH(FWIME_K_PROP, m.nsteps * prop_bytes(x, a, Sb), launch_march(m, x->coop_sms, x->st));
-        k += m.nsteps;
-    }
-    return FWIME_OK;
-}
-
 static int record(Run &r, int Sb, const float *f1, const float *f2, float *d, int accumulate)
 {
     fwime_ctx *x = r.x;
@@ -721,6 +690,77 @@ static int record(Run &r, int Sb, const float *f1, const float *f2, float *d, in
     a.f1 = f1; a.f2 = f2; a.d = d; a.dstride = (long long)x->g.nt * x->nrec; a.accumulate = accumulate;
     LAUNCH(FWIME_K_POINTS, (double)Sb * x->nrec * (8.0 + (f2 ? 4 : 0) + (accumulate ? 4 : 0)),
            launch_points(a, Sb, x->st));
+    return FWIME_OK;
+}
+
+static int steps(Run &r, int Sb, int n, Steps &p)
+{
+    fwime_ctx *x = r.x;
+    const long long SP = (long long)r.w.S * x->P;
+    const auto slot = [&](int m) { return p.ring + (m % p.R) * SP; };
+    const float *inj = p.inj;
+    // operands of step k, into `out`
+    const auto args = [&](int k, float *out) {
+        float *c = p.R ? slot(p.m0 - k + 1) : p.cur, *q = p.R ? slot(p.m0 - k + 2) : p.prev;
+        return prop_args(r, c, q, out, p.d2 ? p.d2 + k * p.d2_step : nullptr,
+                         p.wsrc ? p.wsrc + k : nullptr, p.shot0, p.f0 ? p.f0 + k * p.f0_step : nullptr, p.f0 ? 1.f : 0.f,
+                         p.coef, p.fc ? p.fc + k * p.fc_step : nullptr,
+                         RecTo{p.rec ? p.rec + (long long)k * x->nrec : nullptr, p.rec_acc},
+                         InjFrom{inj ? inj - (long long)k * x->nrec : nullptr});
+    };
+    const auto first = args(0, p.R ? slot(p.m0) : p.prev);
+    // few shots on a small grid: many steps per launch (not in the plain path, nor where every step is timed, nor
+    // beside other streams, whose launches a cooperative one would wait for and hold up)
+    const bool many = n > 2 && x->coop_sms > 0 && alone(x) && !x->opt_plain && !x->opt_profile &&
+                      march_pays(first, Sb, x->coop_sms);
+    // large batches: two steps per launch (a first single one where their number is odd)
+    const bool pairs = !many && n >= 2 && !x->opt_plain && (p.R || r.alt[0]) && pair_pays(x->P, Sb) && pair_runs(first);
+    int paired = 0;
+    for (int k = 0; k < n;) {
+        if (many) {
+            MarchArgs m{};
+            m.a = args(k, p.R ? slot(p.m0 - k) : p.prev);
+            m.nsteps = std::min(n - k, MARCH_STEPS);
+            m.S = Sb;
+            m.ring = p.ring; m.rstride = SP; m.R = p.R; m.m0 = p.m0 - k;
+            m.d2_step = p.d2_step; m.f0_step = p.f0_step; m.fc_step = p.fc_step; m.rec_step = x->nrec; m.inj_step = -x->nrec;
+            m.bar = x->d_bar; m.status = x->d_status;
+            LAUNCH(FWIME_K_PROP, m.nsteps * prop_bytes(x, m.a, Sb), launch_march(m, x->coop_sms, x->st));
+            k += m.nsteps;
+            if (m.nsteps & 1) std::swap(p.cur, p.prev);
+        } else if (pairs && (n - k) % 2 == 0) {
+            PairArgs m{};
+            m.a = args(k, p.R ? slot(p.m0 - k) : r.alt[0]);
+            m.out2 = p.R ? slot(p.m0 - k - 1) : r.alt[1];
+            m.d2b = p.d2 ? p.d2 + (k + 1) * p.d2_step : nullptr;
+            m.f0b = p.f0 ? p.f0 + (k + 1) * p.f0_step : nullptr;
+            m.inj_val2 = inj ? inj - (long long)(k + 1) * x->nrec : nullptr;
+            m.rec_prev = paired;
+            LAUNCH(FWIME_K_PROP, 2.0 * prop_bytes(x, m.a, Sb) - 8.0 * Sb * x->NZ * x->NX, launch_pair(m, Sb, x->st));
+            if (!p.R) {
+                std::swap(p.prev, r.alt[0]);
+                std::swap(p.cur, r.alt[1]);
+            }
+            paired = 1;
+            k += 2;
+        } else {
+            const PropArgs a = args(k, p.R ? slot(p.m0 - k) : p.prev);
+            LAUNCH(FWIME_K_PROP, prop_bytes(x, a, Sb), launch_prop(a, Sb, x->st));
+            if (!p.R) std::swap(p.cur, p.prev);
+            ++k;
+        }
+    }
+    // the last pair's first step has not been an input yet
+    if (paired && p.rec) TRY(record(r, Sb, p.prev, nullptr, p.rec + (long long)(n - 1) * x->nrec, p.rec_acc));
+    return FWIME_OK;
+}
+
+// n steps of the fields (cur, prev), which then hold the last two steps
+static int steps(Run &r, int Sb, int n, float *&cur, float *&prev, Steps p)
+{
+    p.cur = cur; p.prev = prev;
+    TRY(steps(r, Sb, n, p));
+    cur = p.cur; prev = p.prev;
     return FWIME_OK;
 }
 
@@ -907,6 +947,16 @@ static bool gs_reserve(fwime_ctx *x, int K)
     return true;
 }
 
+// The free pair of fields at the start of a batch (zero: the stencil never writes the inactive rows and columns).
+static int pair_reset(Run &r, int Sb)
+{
+    for (int i = 0; i < 2; ++i) {
+        r.alt[i] = r.w.alt[i];
+        if (r.alt[i]) TRY(zero(r.x, r.alt[i], sizeof(float) * Sb * r.x->P));
+    }
+    return FWIME_OK;
+}
+
 static int run_forward(fwime_ctx *x, Run &r, const float *v, const float *w, float *d)
 {
     const int nt = x->g.nt, S = r.w.S;
@@ -920,9 +970,9 @@ static int run_forward(fwime_ctx *x, Run &r, const float *v, const float *w, flo
         TRY(zero(x, db, sizeof(float) * Sb * nd));
         // the launch of step n records its input q^n; the last sample q^{nt-1} is recorded after the loop
         Steps sp;
-        sp.cur = cur; sp.prev = prv; sp.wsrc = w + (size_t)s0 * nt; sp.shot0 = s0; sp.rec = db;
-        TRY(steps(r, Sb, nt - 1, sp));
-        if ((nt - 1) & 1) std::swap(cur, prv);
+        sp.wsrc = w + (size_t)s0 * nt; sp.shot0 = s0; sp.rec = db;
+        TRY(pair_reset(r, Sb));
+        TRY(steps(r, Sb, nt - 1, cur, prv, sp));
         TRY(record(r, Sb, cur, nullptr, db + (size_t)(nt - 1) * x->nrec, 0));
     }
     return FWIME_OK;
@@ -977,6 +1027,7 @@ static int run_born_ext(fwime_ctx *x, Run &r, const float *v, const float *w, co
         for (int i = 0; i < 4; ++i) TRY(zero(x, r.w.f[i], sizeof(float) * Sb * x->P));
         float *db = d + s0 * nd;
         TRY(zero(x, db, sizeof(float) * Sb * nd));
+        TRY(pair_reset(r, Sb));
         for (int n0 = 0; n0 < nt - 1; n0 += K) {
             const int n1 = std::min(n0 + K, nt - 1), kk = n1 - n0;
             if (x->bg_written && !keep) {
@@ -984,16 +1035,14 @@ static int run_born_ext(fwime_ctx *x, Run &r, const float *v, const float *w, co
                 TRY(copyf(x, bg_slot(x, n0 / K, 1, s0), p0, (size_t)Sb * x->P));
             }
             Steps bgs;
-            bgs.cur = c0; bgs.prev = p0; bgs.wsrc = w + (size_t)s0 * nt + n0; bgs.shot0 = s0;
+            bgs.wsrc = w + (size_t)s0 * nt + n0; bgs.shot0 = s0;
             bgs.d2 = keep ? bg_d2t(x, n0, s0) : Dr; bgs.d2_step = keep ? x->nshot * x->P : SP;
-            TRY(steps(r, Sb, kk, bgs));
-            if (kk & 1) std::swap(c0, p0);
+            TRY(steps(r, Sb, kk, c0, p0, bgs));
             const RingRef dring = keep ? ringref(bg_d2t(x, n0, s0), x->nshot * x->P, 0, 0) : ringref(Dr, SP, 0, 0);
             TRY(scatter(r, Sb, n0, kk, r.w.W, dring, ringref(Er, SP, 0, 0), +1, 0));
             Steps scs;
-            scs.cur = c1; scs.prev = p1; scs.f0 = Er; scs.f0_step = SP; scs.rec = db + (size_t)n0 * x->nrec;
-            TRY(steps(r, Sb, kk, scs));
-            if (kk & 1) std::swap(c1, p1);
+            scs.f0 = Er; scs.f0_step = SP; scs.rec = db + (size_t)n0 * x->nrec;
+            TRY(steps(r, Sb, kk, c1, p1, scs));
         }
         TRY(record(r, Sb, c1, nullptr, db + (size_t)(nt - 1) * x->nrec, 0));
     }
@@ -1024,16 +1073,16 @@ static int run_born_adj(fwime_ctx *x, Run &r, bool ext, const float *v, const fl
         const bool kept = r.w.hist || (use_bg && x->bg.hist);
         auto ckp = [&](int j, int t) -> float * { return use_bg ? bg_slot(x, j, t, s0) : ck + (2LL * j + t) * SP; };
         Steps fw;
-        fw.cur = cur; fw.prev = prv; fw.wsrc = ws; fw.shot0 = s0; fw.d2 = Dr; fw.d2_step = SP;
-        if (r.w.hist) TRY(steps(r, Sb, nt - 1, fw));
+        fw.wsrc = ws; fw.shot0 = s0; fw.d2 = Dr; fw.d2_step = SP;
+        TRY(pair_reset(r, Sb));
+        if (r.w.hist) TRY(steps(r, Sb, nt - 1, cur, prv, fw));
         for (int j = 0; j < nseg && !use_bg && !kept; ++j) {
             TRY(copyf(x, ck + (2LL * j) * SP, cur, (size_t)Sb * x->P));
             TRY(copyf(x, ck + (2LL * j + 1) * SP, prv, (size_t)Sb * x->P));
             if (j == nseg - 1) break;
             Steps ck_fw;
-            ck_fw.cur = cur; ck_fw.prev = prv; ck_fw.wsrc = ws + j * K; ck_fw.shot0 = s0;
-            TRY(steps(r, Sb, K, ck_fw));
-            if (K & 1) std::swap(cur, prv);
+            ck_fw.wsrc = ws + j * K; ck_fw.shot0 = s0;
+            TRY(steps(r, Sb, K, cur, prv, ck_fw));
         }
         // backward sweep
         for (int j = nseg - 1; j >= 0; --j) {
@@ -1041,8 +1090,8 @@ static int run_born_adj(fwime_ctx *x, Run &r, bool ext, const float *v, const fl
             if (!kept) {
                 TRY(copyf(x, cur, ckp(j, 0), (size_t)Sb * x->P));
                 TRY(copyf(x, prv, ckp(j, 1), (size_t)Sb * x->P));
-                fw.cur = cur; fw.prev = prv; fw.wsrc = ws + n0;
-                TRY(steps(r, Sb, kk, fw));
+                fw.wsrc = ws + n0;
+                TRY(steps(r, Sb, kk, cur, prv, fw));
             }
             const RingRef dring = r.w.hist ? ringref(Dr + n0 * SP, SP, 0, 0)
                                   : kept   ? ringref(bg_d2t(x, n0, s0), x->nshot * x->P, 0, 0)
@@ -1409,27 +1458,23 @@ static int run_tomo(fwime_ctx *x, Run &r, const float *v, const float *w, const 
         }
         float *db = d + s0 * nd;
         TRY(zero(x, db, sizeof(float) * Sb * nd));
+        TRY(pair_reset(r, Sb));
         const float *ws = w + (size_t)s0 * nt;
         for (int n0 = 0; n0 < nt - 1; n0 += K) {
             const int n1 = std::min(n0 + K, nt - 1), kk = n1 - n0;
-            const auto run = [&](float *&cur, float *&prv, Steps sp) {
-                sp.cur = cur; sp.prev = prv;
-                if (kk & 1) std::swap(cur, prv);
-                return steps(r, Sb, kk, sp);
-            };
             Steps q0, qd, qs, qt;
             q0.wsrc = ws + n0; q0.shot0 = s0; q0.d2 = D0r; q0.d2_step = SP;
-            TRY(run(f[0], f[1], q0));         // background q0
+            TRY(steps(r, Sb, kk, f[0], f[1], q0));         // background q0
             qd.coef = r.w.coef; qd.fc = D0r; qd.fc_step = SP; qd.d2 = D0d; qd.d2_step = SP;
-            TRY(run(f[2], f[3], qd));         // Born wavefield of dv
+            TRY(steps(r, Sb, kk, f[2], f[3], qd));         // Born wavefield of dv
             TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0r, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
             qs.f0 = Er; qs.f0_step = SP; qs.d2 = Dsr; qs.d2_step = SP;
-            TRY(run(f[4], f[5], qs));         // extended Born wavefield of p~
+            TRY(steps(r, Sb, kk, f[4], f[5], qs));         // extended Born wavefield of p~
             TRY(scatter(r, Sb, n0, kk, r.w.W2, ringref(D0r, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
             TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0d, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 1));
             qt.f0 = Er; qt.f0_step = SP; qt.coef = r.w.coef; qt.fc = Dsr; qt.fc_step = SP;
             qt.rec = db + (size_t)n0 * x->nrec;
-            TRY(run(f[6], f[7], qt));         // tomographic wavefield
+            TRY(steps(r, Sb, kk, f[6], f[7], qt));         // tomographic wavefield
         }
         TRY(record(r, Sb, f[6], nullptr, db + (size_t)(nt - 1) * x->nrec, 0));
     }
@@ -1482,6 +1527,7 @@ static int run_tomo_adj(fwime_ctx *x, Run &r, int mode, const float *v, const fl
         };
         float *q0c = r.w.f[0], *q0p = r.w.f[1], *qsc = r.w.f[2], *qsp = r.w.f[3];
         for (int i = 0; i < 4; ++i) TRY(zero(x, r.w.f[i], fb));
+        TRY(pair_reset(r, Sb));
         if (bwd) {
             TRY(zero(x, Mu, sizeof(float) * R * SP));
             TRY(zero(x, Zr, sizeof(float) * R * SP));
@@ -1507,17 +1553,13 @@ static int run_tomo_adj(fwime_ctx *x, Run &r, int mode, const float *v, const fl
                 // with the gradient, the launch of step n adds its input (q0^n, then the scattered field's)
                 // to the prediction's row n (zeroed above; a + b is exact in either order of the two)
                 Steps q0, qs;
-                q0.cur = q0c; q0.prev = q0p; q0.d2 = D0; q0.d2_step = SP; q0.wsrc = ws + n0; q0.shot0 = s0;
+                q0.d2 = D0; q0.d2_step = SP; q0.wsrc = ws + n0; q0.shot0 = s0;
                 q0.rec = grad ? pred + (size_t)n0 * x->nrec : nullptr; q0.rec_acc = 1;
-                TRY(steps(r, Sb, kk, q0));
+                TRY(steps(r, Sb, kk, q0c, q0p, q0));
                 TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
-                qs.cur = qsc; qs.prev = qsp; qs.d2 = r.w.hist ? Dsr + n0 * SP : nullptr; qs.d2_step = SP;
+                qs.d2 = r.w.hist ? Dsr + n0 * SP : nullptr; qs.d2_step = SP;
                 qs.f0 = Er; qs.f0_step = SP; qs.rec = q0.rec; qs.rec_acc = 1;
-                TRY(steps(r, Sb, kk, qs));
-                if (kk & 1) {
-                    std::swap(q0c, q0p);
-                    std::swap(qsc, qsp);
-                }
+                TRY(steps(r, Sb, kk, qsc, qsp, qs));
             }
             if (grad) {   // the last sample of both fields
                 TRY(record(r, Sb, q0c, qsc, pred + (size_t)(nt - 1) * x->nrec, 1));
@@ -1537,11 +1579,11 @@ static int run_tomo_adj(fwime_ctx *x, Run &r, int mode, const float *v, const fl
                 TRY(copyf(x, qsc, ckp(j, 2), fn));
                 TRY(copyf(x, qsp, ckp(j, 3), fn));
                 Steps q0, qs;
-                q0.cur = q0c; q0.prev = q0p; q0.d2 = D0r; q0.d2_step = SP; q0.wsrc = ws + n0; q0.shot0 = s0;
-                TRY(steps(r, Sb, kk, q0));
+                q0.d2 = D0r; q0.d2_step = SP; q0.wsrc = ws + n0; q0.shot0 = s0;
+                TRY(steps(r, Sb, kk, q0c, q0p, q0));
                 TRY(scatter(r, Sb, n0, kk, r.w.W, ringref(D0r, SP, 0, 0), ringref(Er, SP, 0, 0), +1, 0));
-                qs.cur = qsc; qs.prev = qsp; qs.d2 = Dsr; qs.d2_step = SP; qs.f0 = Er; qs.f0_step = SP;
-                TRY(steps(r, Sb, kk, qs));
+                qs.d2 = Dsr; qs.d2_step = SP; qs.f0 = Er; qs.f0_step = SP;
+                TRY(steps(r, Sb, kk, qsc, qsp, qs));
             }
             const RingRef d0ring = ringref(D0r + (r.w.hist ? n0 * SP : 0), SP, 0, 0);
             const RingRef dsring = ringref(Dsr + (r.w.hist ? n0 * SP : 0), SP, 0, 0);

@@ -98,6 +98,14 @@ inline void prop_pairs(PropArgs &a)
     a.a22 = make_float2(a.a2, a.a2);
 }
 
+// two time steps in one launch (k_prop_pair): the first step's operands in `a` (out aliases no input), the second's
+struct PairArgs {
+    PropArgs a;
+    float *out2, *d2b;
+    const float *f0b, *inj_val2;   // (the second step's source amplitude follows the first's)
+    int rec_prev;                  // record prev's receivers too, one row of the data earlier
+};
+
 // several time steps in one cooperative launch (k_march): step k's operands from those of step 0 in `a`
 struct MarchArgs {
     PropArgs a;
@@ -196,9 +204,13 @@ struct TlagArgs {
 // launchers (return cudaGetLastError())
 cudaError_t launch_prop(const PropArgs &a, int nshot, cudaStream_t st);
 cudaError_t prop_occupancy(int *blocks_per_sm);
-int chunk_rows(int rows, int nstrip, int S, long long warps, long long *cost_out);   // rows per warp
+int chunk_rows(int rows, int nstrip, int S, long long warps, long long *cost_out, int overhead = 6,
+               int start = 0);   // rows per warp
 bool march_pays(const PropArgs &a, int S, int nsm);
 cudaError_t launch_march(const MarchArgs &m, int nsm, cudaStream_t st);
+cudaError_t launch_pair(const PairArgs &m, int nshot, cudaStream_t st);
+bool pair_runs(const PropArgs &a);
+bool pair_pays(long long P, int S);
 cudaError_t launch_prop_group(const GroupMember *m, int nactive, int ctas, const GroupRec *g, int nrec_threads,
                               int step, cudaStream_t st, bool record);
 cudaError_t launch_points(const PointsArgs &a, int nshot, cudaStream_t st);

@@ -258,6 +258,26 @@ __device__ __forceinline__ void inject_point(const PropArgs &a, const float *val
         o = __fadd_rn(o, __fmul_rn(c, __ldg(val + (long long)shot * a.inj_vstride + r)));
 }
 
+// The same for the four points of a lane at (zz, x), before they are stored; D2t gains what the point gains.
+template <bool D2>
+__device__ __forceinline__ void inject_row(const PropArgs &a, const float *val, int shot, int zz, int x, const float4 &cv,
+                                           float4 &o, float4 &d2)
+{
+    const int4 m4 = *reinterpret_cast<const int4 *>(a.inj_map + (long long)(zz - a.inj_lo) * a.NXP + x);
+    if ((m4.x & m4.y & m4.z & m4.w) < 0) return;   // none of the four
+    const float4 o0 = o;
+    inject_point(a, val, shot, m4.x, cv.x, o.x);
+    inject_point(a, val, shot, m4.y, cv.y, o.y);
+    inject_point(a, val, shot, m4.z, cv.z, o.z);
+    inject_point(a, val, shot, m4.w, cv.w, o.w);
+    if (D2) {
+        d2.x = fmaf(o.x - o0.x, a.inv_dt2, d2.x);
+        d2.y = fmaf(o.y - o0.y, a.inv_dt2, d2.y);
+        d2.z = fmaf(o.z - o0.z, a.inv_dt2, d2.z);
+        d2.w = fmaf(o.w - o0.w, a.inv_dt2, d2.w);
+    }
+}
+
 // The time step of one warp's work item (strip, chunk) of shot `shot`; wsm is the warp's shared
 // memory (CUR_SLOTS x CUR_ROW + AUX_SLOTS x naux_max x STRIP floats).  sp: the operands that change from step to step
 // (the same members of PropArgs).  COH: the fields change during the kernel (several steps per launch), so no read of

@@ -74,20 +74,21 @@ cudaError_t prop_occupancy(int *blocks_per_sm)
 }
 
 // Rows per warp's item: the items (strip, chunk of rows) of S shots go to `warps` resident warps in rounds of equal
-// length; the split of the rows with the least rounds x (rows + 6, about what an item's start costs) wins.
+// length; the split of the rows with the least (rounds + start / 2) x (rows + overhead) wins: overhead is about what an
+// item's start costs, start / 2 the part of a round that a launch's ramp and drain take.
 // Marmousi2-shaped, us per launch with the former aim of 4864 warps and with this: 32 shots 69 / 60, 50 shots 100 / 87,
 // 100 shots 178 / 169.
-int chunk_rows(int rows, int nstrip, int S, long long warps, long long *cost_out)
+int chunk_rows(int rows, int nstrip, int S, long long warps, long long *cost_out, int overhead, int start)
 {
     long long best = -1;
     int best_zc = rows;
     for (int c = 1; c <= (rows + 1) / 2; ++c) {
         const int zc = (rows + c - 1) / c;
         const long long items = (long long)nstrip * S * ((rows + zc - 1) / zc);
-        const long long cost = (items + warps - 1) / warps * (zc + 6);
+        const long long cost = (2 * ((items + warps - 1) / warps) + start) * (zc + overhead);
         if (best < 0 || cost <= best) { best = cost; best_zc = zc; }   // ties: the more, shorter items
     }
-    if (cost_out) *cost_out = std::max(best, 0LL);
+    if (cost_out) *cost_out = std::max(best, 0LL) / 2;
     return std::max(best_zc, 1);
 }
 
