@@ -461,8 +461,7 @@ static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
     if (x->max_ws && need > x->max_ws)
         return fail(x, FWIME_ENOMEM, "operator needs %zu bytes for S=%d, K=%d; budget %zu", need, w.S, w.K, x->max_ws);
     const size_t alt_bytes = 2 * al((size_t)w.S * x->P) * sizeof(float);
-    const bool tlag_op = x->opt_tlag > 0 && op != FWIME_OP_FORWARD && op != FWIME_OP_BORN && op != FWIME_OP_BORN_ADJ;
-    const bool alt = op != FWIME_OP_BORN && !tlag_op && !x->opt_plain && !x->opt_fs && pair_pays(x->P, w.S) &&
+    const bool alt = op != FWIME_OP_BORN && !x->opt_plain && !x->opt_fs && pair_pays(x->P, w.S) &&
                      need + alt_bytes <= budget;
     if (alt) need += alt_bytes;
     if (need > x->ws_bytes) {
@@ -762,16 +761,6 @@ static int steps(Run &r, int Sb, int n, float *&cur, float *&prev, Steps p)
     TRY(steps(r, Sb, n, p));
     cur = p.cur; prev = p.prev;
     return FWIME_OK;
-}
-
-// One adjoint time step with the residual's injection at the receivers folded into the stencil launch
-// (the transpose of recording; the same arithmetic as a separate injection after the step), and
-// optionally the D2t of its output, injection included
-static int adj_step(Run &r, int Sb, const float *cur, const float *prev, float *out, const float *val,
-                    float *d2 = nullptr)
-{
-    return prop(r, Sb, cur, prev, out, d2, nullptr, 0, nullptr, 0.f, nullptr, 0.f, nullptr, 0.f, nullptr,
-                nullptr, RecTo{}, InjFrom{val});
 }
 
 static RingRef ringref(const float *base, long long slot_stride, int mod, int shift)
@@ -1131,6 +1120,20 @@ static int tlag_launch(Run &r, int Sb, int n0, int n1, bool image, RingRef D, Ri
     return FWIME_OK;
 }
 
+// Background steps [n, end) of (cur, prev), their D2t into slots (step mod RD) of the ring D
+static int ring_steps(Run &r, int Sb, int n, int end, float *&cur, float *&prev, const float *w, int s0, float *D, int RD)
+{
+    const long long SP = (long long)r.w.S * r.x->P;
+    while (n < end) {
+        const int k = std::min(end - n, RD - n % RD);   // up to the ring's end
+        Steps q;
+        q.wsrc = w + n; q.shot0 = s0; q.d2 = D ? D + (long long)(n % RD) * SP : nullptr; q.d2_step = SP;
+        TRY(steps(r, Sb, k, cur, prev, q));
+        n += k;
+    }
+    return FWIME_OK;
+}
+
 // B~ with time lags: the background runs Hs = 2 hm lag steps ahead of the scattered field so that every
 // segment's secondary sources find D2t q0 at n - 2 s_i for all lags in the ring
 static int run_born_tlag(fwime_ctx *x, Run &r, const float *w, const float *pt, float *d)
@@ -1150,20 +1153,17 @@ static int run_born_tlag(fwime_ctx *x, Run &r, const float *w, const float *pt, 
         for (int i = 0; i < 4; ++i) TRY(zero(x, r.w.f[i], sizeof(float) * Sb * x->P));
         float *db = d + s0 * nd;
         TRY(zero(x, db, sizeof(float) * Sb * nd));
+        TRY(pair_reset(r, Sb));
         int bg = 0;   // next background step (produces D2t of that step)
         for (int n0 = 0; n0 < nt - 1; n0 += K) {
-            const int n1 = std::min(n0 + K, nt - 1);
-            for (const int top = std::min(n1 - 1 + Hs, nt - 2); bg <= top; ++bg) {
-                TRY(prop(r, Sb, c0, p0, p0, Dr + (long long)(bg % RD) * SP, w + (size_t)s0 * nt + bg, s0));
-                std::swap(c0, p0);
-            }
+            const int n1 = std::min(n0 + K, nt - 1), end = std::min(n1 + Hs, nt - 1);
+            TRY(ring_steps(r, Sb, bg, end, c0, p0, w + (size_t)s0 * nt, s0, Dr, RD));
+            bg = end;
             TRY(tlag_launch(r, Sb, n0, n1, false, ringref(Dr, SP, RD, 0), ringref(Er, SP, 0, 0),
                             ringref(nullptr, 0, 0, 0), nullptr));
-            for (int n = n0; n < n1; ++n) {
-                TRY(prop(r, Sb, c1, p1, p1, nullptr, nullptr, 0, Er + (n - n0) * SP, 1.f, nullptr, 0.f, nullptr, 0.f,
-                         nullptr, nullptr, RecTo{db + (size_t)n * x->nrec, 0}));
-                std::swap(c1, p1);
-            }
+            Steps sc;
+            sc.f0 = Er; sc.f0_step = SP; sc.rec = db + (size_t)n0 * x->nrec;
+            TRY(steps(r, Sb, n1 - n0, c1, p1, sc));
         }
         TRY(record(r, Sb, c1, nullptr, db + (size_t)(nt - 1) * x->nrec, 0));
     }
@@ -1191,16 +1191,15 @@ static int run_born_tlag_adj(fwime_ctx *x, Run &r, const float *v, const float *
         TRY(zero(x, cur, fb));
         TRY(zero(x, prv, fb));
         TRY(zero(x, Mu, sizeof(float) * R * SP));
+        TRY(pair_reset(r, Sb));
         const float *ws = w + (size_t)s0 * nt;
         // checkpointing sweep: the state at the start of every block
         int n = 0;
         for (int j = 0; j < NB; ++j) {
             const int b0 = bstart(j);
             if (b0 >= bend(j)) continue;   // empty block (all before step 0)
-            for (; n < b0; ++n) {
-                TRY(prop(r, Sb, cur, prv, prv, nullptr, ws + n, s0));
-                std::swap(cur, prv);
-            }
+            TRY(ring_steps(r, Sb, n, b0, cur, prv, ws, s0, nullptr, RD));
+            n = b0;
             TRY(copyf(x, ck + (2LL * j) * SP, cur, (size_t)Sb * x->P));
             TRY(copyf(x, ck + (2LL * j + 1) * SP, prv, (size_t)Sb * x->P));
         }
@@ -1209,20 +1208,15 @@ static int run_born_tlag_adj(fwime_ctx *x, Run &r, const float *v, const float *
             if (b0 >= b1) return FWIME_OK;
             TRY(copyf(x, cur, ck + (2LL * j) * SP, (size_t)Sb * x->P));
             TRY(copyf(x, prv, ck + (2LL * j + 1) * SP, (size_t)Sb * x->P));
-            for (int m = b0; m < b1; ++m) {
-                TRY(prop(r, Sb, cur, prv, prv, Dr + (long long)(m % RD) * SP, ws + m, s0));
-                std::swap(cur, prv);
-            }
-            return FWIME_OK;
+            return ring_steps(r, Sb, b0, b1, cur, prv, ws, s0, Dr, RD);
         };
         int next_block = NB - 1;   // blocks > next_block are in the ring
         for (int j = nseg - 1; j >= 0; --j) {
             const int n0 = j * K, n1 = std::min(n0 + K, nt - 1);
             for (; next_block >= j; --next_block) TRY(block(next_block));
-            for (int m = n1; m >= n0 + 1; --m) {
-                float *mo = Mu + (m % R) * SP;
-                TRY(adj_step(r, Sb, Mu + ((m + 1) % R) * SP, Mu + ((m + 2) % R) * SP, mo, d + s0 * nd + (size_t)m * x->nrec));
-            }
+            Steps ad;
+            ad.ring = Mu; ad.R = R; ad.m0 = n1; ad.inj = d + s0 * nd + (size_t)n1 * x->nrec;
+            TRY(steps(r, Sb, n1 - n0, ad));
             TRY(tlag_launch(r, Sb, n0, n1, true, ringref(Dr, SP, RD, 0), ringref(nullptr, 0, 0, 0),
                             ringref(Mu, SP, R, 1), r.w.acc1));
         }
@@ -1332,6 +1326,7 @@ static int run_tomo_adj_tlag(fwime_ctx *x, Run &r, int mode, const float *v, con
         const size_t fn = (size_t)Sb * x->P;
         float *q0c = r.w.f[0], *q0p = r.w.f[1], *qsc = r.w.f[2], *qsp = r.w.f[3];
         for (int i = 0; i < 4; ++i) TRY(zero(x, r.w.f[i], fb));
+        TRY(pair_reset(r, Sb));
         if (!objective_only) {
             TRY(zero(x, Mu, sizeof(float) * RM * SP));
             TRY(zero(x, Zr, sizeof(float) * R * SP));
@@ -1383,25 +1378,20 @@ static int run_tomo_adj_tlag(fwime_ctx *x, Run &r, int mode, const float *v, con
                 if (b0 >= b1) continue;
                 TRY(copyf(x, q0c, ckq + (2LL * next_block) * SP, fn));
                 TRY(copyf(x, q0p, ckq + (2LL * next_block + 1) * SP, fn));
-                for (int m = b0; m < b1; ++m) {
-                    TRY(prop(r, Sb, q0c, q0p, q0p, D0r + (long long)(m % RD) * SP, ws + m, s0));
-                    std::swap(q0c, q0p);
-                }
+                TRY(ring_steps(r, Sb, b0, b1, q0c, q0p, ws, s0, D0r, RD));
             }
             TRY(copyf(x, qsc, cks + (2LL * j) * SP, fn));
             TRY(copyf(x, qsp, cks + (2LL * j + 1) * SP, fn));
             TRY(tlag_launch(r, Sb, n0, n1, false, dring, er, none, nullptr));
-            for (int n = n0; n < n1; ++n) {
-                TRY(prop(r, Sb, qsc, qsp, qsp, Dsr + (n - n0) * SP, nullptr, 0, Er + (n - n0) * SP, 1.f));
-                std::swap(qsc, qsp);
-            }
+            Steps qs;
+            qs.f0 = Er; qs.f0_step = SP; qs.d2 = Dsr; qs.d2_step = SP;
+            TRY(steps(r, Sb, kk, qsc, qsp, qs));
             // the residual's adjoint field, Hs steps ahead: mu^k down to k = n0 - Hs + 1
-            for (const int lo = std::max(n0 - Hs + 1, 1); mu_lo - 1 >= lo; --mu_lo) {
-                const int k = mu_lo - 1;
-                float *mo = Mu + (long long)(k % RM) * SP;
-                TRY(adj_step(r, Sb, Mu + (long long)((k + 1) % RM) * SP, Mu + (long long)((k + 2) % RM) * SP, mo,
-                             rr + (size_t)k * x->nrec));
-            }
+            const int lo = std::max(n0 - Hs + 1, 1);
+            Steps ad;
+            ad.ring = Mu; ad.R = RM; ad.m0 = mu_lo - 1; ad.inj = rr + (size_t)(mu_lo - 1) * x->nrec;
+            if (mu_lo > lo) TRY(steps(r, Sb, mu_lo - lo, ad));
+            mu_lo = std::min(mu_lo, lo);
             // z^m = sum_i W_i lambda^(m + 2 s_i) for m in [n0, n1) (lambda^n = mu^(n+1))
             TRY(tlag_launch(r, Sb, n0, n1, false, ringref(Mu, SP, RM, 1), ringref(Zr, SP, R, n0), none, nullptr, r.w.W,
                             -1, 0));

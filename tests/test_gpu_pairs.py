@@ -42,7 +42,8 @@ def call(ctx, op, t):
 # of odd and even numbers of rows; odd and even numbers of steps and segments
 @pytest.mark.parametrize("op,nh,opts", [
     ("forward", 1, {}), ("born_ext", 5, {}), ("tomo", 5, {}), ("born_adj", 1, {}), ("born_ext_adj", 7, {}),
-    ("tomo_adj", 5, {}), ("gradient", 5, {}), ("gradient", 5, {"segment": 5}), ("born_ext_adj", 5, {"segment": 6})])
+    ("tomo_adj", 5, {}), ("gradient", 5, {}), ("gradient", 5, {"segment": 5}), ("born_ext_adj", 5, {"segment": 6}),
+    ("born_ext", 3, {"time_lag": 1}), ("born_ext_adj", 3, {"time_lag": 1}), ("gradient", 3, {"time_lag": 1})])
 @pytest.mark.parametrize("nz,nx,sponge,nt", [(43, 460, 6, 24), (150, 1001, 20, 25), (401, 130, 9, 13), (3, 700, 1, 20)])
 def test_pairs_of_steps(op, nh, opts, nz, nx, sponge, nt):
     pad = 2 * (sponge + 4)
