@@ -23,6 +23,7 @@
 #include <atomic>
 #include <mutex>
 #include <cstdarg>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -584,6 +585,7 @@ static void init_run(fwime_ctx *x, Run &r, int S)
         zc = chunk_rows(rows, r.nstrip, std::max(S, 1), 152LL * 16, nullptr);
         if (!alone(x)) zc = std::max(zc, 8);
     }
+    zc = std::min(zc, std::max(1, INT_MAX / x->NXP - 16));   // (offsets within an item are 32-bit)
     r.zchunk = zc;
     r.nchunk = (rows + zc - 1) / zc;
     PropArgs &a = r.base;

@@ -22,6 +22,8 @@
 
 namespace fwk {
 
+// the warp's index in its CTA, as a value that is known to be the same in all its lanes
+__device__ __forceinline__ int warp_in_cta() { return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0); }
 __device__ __forceinline__ float4 f4zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 __device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
 __device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
@@ -47,45 +49,26 @@ __device__ __forceinline__ float4 shfl_down4(float4 v)
     return v;
 }
 
-// ---- asynchronous global -> shared copies (LDGSTS); src_bytes = 0 zero-fills the 16 bytes
-__device__ __forceinline__ void cp16(float *dst, const float *src, bool valid)
+// ---- asynchronous global -> shared copies (LDGSTS); 
+__device__ __forceinline__ void cp16n(float *dst, const float *src, int n)   // n: 16, or 0 to zero-fill
 {
     const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
-    const int n = valid ? 16 : 0;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
-}
-// the same copy issued only where `pred` holds (a predicated instruction instead of a divergent branch)
-__device__ __forceinline__ void cp16p(float *dst, const float *src, bool valid, bool pred)
-{
-    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
-    const int n = valid ? 16 : 0;
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %3, 0;\n @p cp.async.cg.shared.global [%0], [%1], 16, %2;\n}\n" ::"r"(d),
-                 "l"(src), "r"(n), "r"((int)pred)
-                 : "memory");
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 __device__ __forceinline__ float4 lds4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 
-// Per-warp pipeline: an 8-slot ring of q^n rows (128 points + 4-point halos) feeds the x-taps
-// and the register queue; a 4-slot ring holds the q^{n-1}, c and local-source rows of the
-// output row.  Iteration z waits for the copy group issued 4 iterations earlier, so about four
-// rows of every input stream are in flight per warp.
-#ifndef FWIME_PROP_CUR_SLOTS
-#define FWIME_PROP_CUR_SLOTS 8
-#endif
-#ifndef FWIME_PROP_AUX_SLOTS
-#define FWIME_PROP_AUX_SLOTS 4
-#endif
+// Per-warp pipeline: rings of nine rows of q^n (128 points + 4-point halos, for the x-taps and the register queue),
+// q^{n-1} and c; with local sources rings of three rows of those, of q^{n-1} and of c.  Nine is the period of the unrolled register queue, so every
+// slot is a compile-time constant.  Row z waits for the copy group issued four rows (with local sources three) earlier.
+constexpr int RING = 9, LRING = 3;
 // Variants k_prop<LOC, D2, SRC>: LOC = 0 no dense local source, 1 exactly one (f0, weight a0), 2 the
 // general sum a0 f0 + a1 f1 + a2 f2 + coef fc; D2 writes D2t; SRC adds the point source.  Register
 // bounds (minimum resident CTAs) per kind:
 #ifndef FWIME_PROP_MIN_BLOCKS
 #define FWIME_PROP_MIN_BLOCKS 1   // general local sources (up to five extra rows per stage)
-#endif
-#ifndef FWIME_PROP_PRED
-#define FWIME_PROP_PRED 1   // halo copies predicated, not branched (-0.5 %)
 #endif
 #ifndef FWIME_PROP_MINB_LOC1
 #define FWIME_PROP_MINB_LOC1 3   // one local source: up to 128 registers, 4 CTAs per SM like the plain variants
@@ -93,10 +76,12 @@ __device__ __forceinline__ float4 lds4(const float *p) { return *reinterpret_cas
 #ifndef FWIME_PROP_MINB_PLAIN
 #define FWIME_PROP_MINB_PLAIN 3   // up to 128 registers: still 4 CTAs per SM, fewer rematerialised operands
 #endif
-constexpr int CUR_SLOTS = FWIME_PROP_CUR_SLOTS;   // q^n rows in flight: the queue reads row z+4 of slots
-constexpr int AUX_SLOTS = FWIME_PROP_AUX_SLOTS;   // pipeline depth of the q^{n-1}, c, local-source rows
 constexpr int CUR_ROW = STRIP + 8;
-static_assert(CUR_SLOTS >= AUX_SLOTS + 4, "the q^n ring must hold rows z .. z+4+depth");
+// floats of shared memory per warp; naux = 2 + the number of local source rows
+__host__ __device__ constexpr int prop_smem(int naux)
+{
+    return RING * CUR_ROW + (naux > 2 ? LRING : RING) * naux * STRIP;
+}
 
 // The arithmetic of one output row of a lane (four consecutive columns): the Laplacian from the
 // x-neighbours (L | Q4 | Rr, 12 consecutive samples) and the nine queue rows Q0..Q8 (the output row
@@ -279,7 +264,8 @@ __device__ __forceinline__ void inject_row(const PropArgs &a, const float *val, 
 }
 
 // The time step of one warp's work item (strip, chunk) of shot `shot`; wsm is the warp's shared
-// memory (CUR_SLOTS x CUR_ROW + AUX_SLOTS x naux_max x STRIP floats).  sp: the operands that change from step to step
+// memory (prop_smem(naux_max) floats).  wid is warp-uniform and known to be so (a shuffle's result): the address
+// arithmetic is then done once per warp.  sp: the operands that change from step to step
 // (the same members of PropArgs).  COH: the fields change during the kernel (several steps per launch), so no read of
 // them may come from a non-coherent cache.
 template <int LOC, bool D2, bool SRC, bool INJ, bool FS, bool COH, class SP>
@@ -293,55 +279,51 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const SP &sp, const
     const int z0 = (FS || COH ? a.z_first : 4) + chunk * a.zchunk;
     const int z1 = min(z0 + a.zchunk, a.NZ - 4);
     const bool xin = x < a.NXP;
-    const long long so = (long long)shot * a.P;
-    const float *__restrict__ cur = sp.cur + so;
-    const float *prev = sp.prev + so;
-    float *out = sp.out + so;
-    const long long NXP = a.NXP;
+    const int NXP = a.NXP;
+    const long long so = (long long)shot * a.P, row0 = (long long)z0 * NXP;
+    const float *__restrict__ cur = sp.cur + so + row0;
+    const float *prev = sp.prev + so + row0, *c = a.c + row0;
+    float *out0 = sp.out + so + row0, *d20 = D2 ? sp.d2 + so + row0 : nullptr;
 
-    // aux row layout: [prev][c][f0?][f1?][f2?][coef, fc?]
-    const int i_f0 = 2, i_f1 = i_f0 + (a.f0 != nullptr), i_f2 = i_f1 + (a.f1 != nullptr),
-              i_cf = i_f2 + (a.f2 != nullptr);
-    // LOC 1: exactly one local source, f0 (weight a0)
-    const int naux = LOC == 2 ? i_cf + (a.fc != nullptr ? 2 : 0) : (LOC == 1 ? 3 : 2);
-    float *curR = wsm;
-    float *auxR = wsm + CUR_SLOTS * CUR_ROW;
-
-    // copy bounds do not change along the march: hoisted out of the loop
-    const int c0 = x0 - 4 + 4 * lane, c1 = x0 - 4 + 4 * (lane + 32);
-    const bool ok0 = c0 >= 0 && c0 + 4 <= a.NXP;
-    const bool ok1 = lane < CUR_ROW / 4 - 32 && c1 + 4 <= a.NXP;
-    auto issue_cur = [&](int zr) {
-        if (zr > z1 + 3) return;
-        float *dst = curR + ((unsigned)zr % CUR_SLOTS) * CUR_ROW;
-        const float *src = cur + (long long)zr * NXP;
-        cp16(dst + 4 * lane, ok0 ? src + c0 : cur, ok0);
-#if FWIME_PROP_PRED
-        cp16p(dst + 4 * (lane + 32), ok1 ? src + c1 : cur, ok1, lane < CUR_ROW / 4 - 32);
-#else
-        if (lane < CUR_ROW / 4 - 32) cp16(dst + 4 * (lane + 32), ok1 ? src + c1 : cur, ok1);
-#endif
+    // the lane's places in the rings; local sources: [f0?][f1?][f2?][coef, fc?] (LOC 1: exactly one, f0, weight a0)
+    const int i_f1 = a.f0 != nullptr, i_f2 = i_f1 + (a.f1 != nullptr), i_cf = i_f2 + (a.f2 != nullptr);
+    const int nloc = LOC == 2 ? i_cf + (a.fc != nullptr ? 2 : 0) : LOC;
+    constexpr int AR = LOCAL ? LRING : RING;
+    float *curL = wsm + 4 * lane, *prevL = curL + RING * CUR_ROW, *cL = prevL + AR * STRIP, *fL = cL + AR * STRIP;
+    // The lane's columns: of the q^n row with its halo, of the row's end (two lanes), its own; relative to row z0, and
+    // moved down with z.  A column outside reads nothing (zero-filled).
+    const int cA = x0 - 4 + 4 * lane, cB = cA + STRIP;
+    const int nA = cA >= 0 && cA + 4 <= NXP ? 16 : 0, nB = cB + 4 <= NXP ? 16 : 0, nX = xin ? 16 : 0;
+    const bool two = lane < CUR_ROW / 4 - 32;
+    int oA = nA ? cA : 0, oB = nB ? cB : 0, oX = nX ? x : 0;
+    // row z + k into slot s
+    const auto issue_cur = [&](int z, int k, int s) {
+        if (z + k > z1 + 3) return;
+        const float *src = cur + (long long)k * NXP;
+        cp16n(curL + s * CUR_ROW, src + oA, nA);
+        if (two) cp16n(curL + s * CUR_ROW + STRIP, src + oB, nB);
     };
-    const long long o_x = xin ? x : 0;
-    auto issue_aux = [&](int zr) {
-        if (zr >= z1) return;
-        float *dst = auxR + ((unsigned)zr % AUX_SLOTS) * naux * STRIP + 4 * lane;
-        const long long o2 = xin ? (long long)zr * NXP + o_x : 0;
-        cp16(dst, prev + o2, xin);
-        cp16(dst + STRIP, a.c + o2, xin);
-        if (LOCAL) {
-            // local sources vanish outside the source rows: zero-filled there, not read
-            const bool lin = xin && zr >= a.zs_lo && zr < a.zs_hi;
-            if (LOC == 1) {
-                cp16(dst + i_f0 * STRIP, sp.f0 + so + o2, lin);
-            } else {
-                if (a.f0) cp16(dst + i_f0 * STRIP, sp.f0 + so + o2, lin);
-                if (a.f1) cp16(dst + i_f1 * STRIP, a.f1 + so + o2, lin);
-                if (a.f2) cp16(dst + i_f2 * STRIP, a.f2 + so + o2, lin);
-                if (a.fc) {
-                    cp16(dst + i_cf * STRIP, a.coef + o2, lin);
-                    cp16(dst + (i_cf + 1) * STRIP, sp.fc + so + o2, lin);
-                }
+    const auto issue_aux = [&](int z, int k, int s) {
+        if (z + k >= z1) return;
+        cp16n(prevL + s * STRIP, prev + (long long)k * NXP + oX, nX);
+        cp16n(cL + s * STRIP, c + (long long)k * NXP + oX, nX);
+    };
+    const auto issue_f = [&](int z, int k, int s) {
+        if (z + k >= z1) return;
+        // local sources vanish outside the source rows: zero-filled there, not read
+        const bool lin = z + k >= a.zs_lo && z + k < a.zs_hi;
+        const int n = lin ? nX : 0;
+        const long long o = row0 + (lin ? (long long)k * NXP + oX : 0);
+        float *dst = fL + s * nloc * STRIP;
+        if (LOC == 1) {
+            cp16n(dst, sp.f0 + so + o, n);
+        } else {
+            if (a.f0) cp16n(dst, sp.f0 + so + o, n);
+            if (a.f1) cp16n(dst + i_f1 * STRIP, a.f1 + so + o, n);
+            if (a.f2) cp16n(dst + i_f2 * STRIP, a.f2 + so + o, n);
+            if (a.fc) {
+                cp16n(dst + i_cf * STRIP, a.coef + o, n);
+                cp16n(dst + (i_cf + 1) * STRIP, sp.fc + so + o, n);
             }
         }
     };
@@ -350,83 +332,85 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const SP &sp, const
     float4 q[9];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        const float *qp = cur + (long long)(z0 - 4 + k) * NXP + x;
+        const float *qp = cur + (long long)(k - 4) * NXP + oX;
         q[k] = !xin ? f4zero() : COH ? __ldcg(reinterpret_cast<const float4 *>(qp)) : ldg4(qp);
     }
-    // prologue: one group per iteration of look-ahead (rows z0 .. z0+3 feed the first x-taps)
+    // prologue: one group per row of look-ahead (rows z0 .. z0+3 feed the first x-taps)
+    constexpr int DEPTH = LOCAL ? LRING : 4;
 #pragma unroll
-    for (int g = 0; g < AUX_SLOTS; ++g) {
-        if (g < 4) issue_cur(z0 + g);
-        issue_cur(z0 + 4 + g);
-        issue_aux(z0 + g);
-        cp_commit();
+    for (int g = 0; g < 4; ++g) {
+        issue_cur(z0, g, g);
+        if (g < DEPTH) {
+            issue_cur(z0, g + 4, g + 4);
+            issue_aux(z0, g, g);
+            if (LOCAL) issue_f(z0, g, g);
+            if (g < DEPTH - 1 || DEPTH == 4) cp_commit();
+        }
     }
-    for (int g = AUX_SLOTS; g < 4; ++g) issue_cur(z0 + g);   // (only when the depth is below 4)
+    if (DEPTH < 4) cp_commit();
     const float4 gxv = xin ? ldg4(a.gx + x) : f4zero();
 
-    long long soff = -1;
+    int srow = -1, scol = -1;   // the point source's row, and its column within this lane's four
     float amp = 0.f;
     if (SRC) {
-        soff = a.src_off[shot];
+        const int off = a.src_off[shot];
+        srow = off / NXP;
+        scol = off - srow * NXP - x;
+        if (scol < 0 || scol > 3) srow = -1;
         amp = sp.src_amp[(long long)shot * a.src_stride] * a.src_scale;
     }
 
-    // One output row zz; the queue's logical row k (zz-4+k) lives in q[(k + R) % 9], so nine
-    // consecutive rows rotate the queue through the registers without moving any of them.
+    // One output row z; the queue's logical row k (z-4+k) lives in q[(k + R) % 9], so nine consecutive rows rotate
+    // the queue through the registers without moving any of them.
 #define FWIME_PROP_ROW(R)                                                                                    \
     {                                                                                                        \
-        const int zz = z + (R);                                                                              \
-        cp_wait<AUX_SLOTS - 1>();                                                                            \
-        __syncwarp();                                                                                        \
-        const float *crow = curR + ((unsigned)zz % CUR_SLOTS) * CUR_ROW;                                     \
-        q[(8 + (R)) % 9] = lds4(curR + ((unsigned)(zz + 4) % CUR_SLOTS) * CUR_ROW + 4 + 4 * lane);           \
-        const float4 L = lds4(crow + 4 * lane);                                                              \
-        const float4 Rr = lds4(crow + 8 + 4 * lane);                                                         \
-        const float *arow = auxR + ((unsigned)zz % AUX_SLOTS) * naux * STRIP + 4 * lane;                     \
-        const float4 pv = lds4(arow);                                                                        \
-        const float4 cv = lds4(arow + STRIP);                                                                \
+        cp_wait<DEPTH - 1>();                                                                                \
+        __syncwarp(); /* every lane's copies are there, and every lane is done with the row before */        \
+        issue_cur(z, 4 + DEPTH, (4 + DEPTH + (R)) % RING);                                                   \
+        if (!LOCAL) issue_aux(z, DEPTH, (DEPTH + (R)) % AR);                                                 \
+        if (!LOCAL) cp_commit();                                                                             \
+        q[(8 + (R)) % 9] = lds4(curL + ((R) + 4) % RING * CUR_ROW + 4);                                      \
+        const float4 L = lds4(curL + (R) * CUR_ROW), Rr = lds4(curL + (R) * CUR_ROW + 8);                    \
+        const float4 pv = lds4(prevL + (R) % AR * STRIP), cv = lds4(cL + (R) % AR * STRIP);                  \
         float4 lf0 = f4zero(), lf1 = f4zero(), lf2 = f4zero(), lcf = f4zero(), lfc = f4zero();               \
-        if (LOC == 1) {                                                                                      \
-            lf0 = lds4(arow + i_f0 * STRIP);                                                                 \
-        } else if (LOC == 2) {                                                                               \
-            if (a.f0) lf0 = lds4(arow + i_f0 * STRIP);                                                       \
-            if (a.f1) lf1 = lds4(arow + i_f1 * STRIP);                                                       \
-            if (a.f2) lf2 = lds4(arow + i_f2 * STRIP);                                                       \
-            if (a.fc) { lcf = lds4(arow + i_cf * STRIP); lfc = lds4(arow + (i_cf + 1) * STRIP); }            \
+        if (LOCAL) {                                                                                         \
+            const float *arow = fL + ((R) % LRING) * nloc * STRIP;                                           \
+            if (LOC == 1) {                                                                                  \
+                lf0 = lds4(arow);                                                                            \
+            } else {                                                                                         \
+                if (a.f0) lf0 = lds4(arow);                                                                  \
+                if (a.f1) lf1 = lds4(arow + i_f1 * STRIP);                                                   \
+                if (a.f2) lf2 = lds4(arow + i_f2 * STRIP);                                                   \
+                if (a.fc) { lcf = lds4(arow + i_cf * STRIP); lfc = lds4(arow + (i_cf + 1) * STRIP); }        \
+            }                                                                                                \
+            __syncwarp(); /* the slot's next row may come */                                                 \
+            issue_aux(z, DEPTH, (R) % AR);                                                                   \
+            issue_f(z, DEPTH, (R) % LRING);                                                                  \
+            cp_commit();                                                                                     \
         }                                                                                                    \
-        const long long idx = (long long)zz * NXP + x;                                                       \
-        const float gzz = __ldg(a.gz + zz);                                                                  \
-        int sj = -1; /* the point source's column within this lane's four, if it is in them */              \
-        if (SRC) {                                                                                           \
-            const long long sd = soff - idx;                                                                 \
-            sj = (sd >= 0 && sd < 4) ? (int)sd : -1;                                                         \
-        }                                                                                                    \
+        const int sj = SRC && z == srow ? scol : -1;                                                         \
         float4 o, d2;                                                                                        \
         row_math<LOC, D2, SRC>(a, prop_k(a), L, q[(0 + (R)) % 9], q[(1 + (R)) % 9], q[(2 + (R)) % 9], q[(3 + (R)) % 9], \
                                  q[(4 + (R)) % 9], q[(5 + (R)) % 9], q[(6 + (R)) % 9], q[(7 + (R)) % 9],      \
-                                 q[(8 + (R)) % 9], Rr, pv, cv, lf0, lf1, lf2, lcf, lfc, gzz, gxv, sj, amp, o, d2); \
+                                 q[(8 + (R)) % 9], Rr, pv, cv, lf0, lf1, lf2, lcf, lfc, __ldg(a.gz + z), gxv, sj, amp, o, d2); \
         if (xin) {                                                                                           \
-            st4(out + idx, o);                                                                               \
-            if (D2 && zz >= a.zs_lo && zz < a.zs_hi) st4(sp.d2 + so + idx, d2);                               \
+            st4(out0 + oX, o);                                                                               \
+            if (D2 && z >= a.zs_lo && z < a.zs_hi) st4(d20 + oX, d2);                                        \
         }                                                                                                    \
-        __syncwarp(); /* every lane is done with this row's slots before they are refilled */              \
-        issue_cur(zz + 4 + AUX_SLOTS);                                                                       \
-        issue_aux(zz + AUX_SLOTS);                                                                           \
-        cp_commit();                                                                                         \
+        ++z;                                                                                                 \
+        oA += NXP;                                                                                           \
+        oB += NXP;                                                                                           \
+        oX += NXP;                                                                                           \
+        if (z >= z1) break;                                                                                  \
     }
 
-    int z = z0;
-    for (; z + 9 <= z1; z += 9) {
+    for (int z = z0;;) {
         FWIME_PROP_ROW(0) FWIME_PROP_ROW(1) FWIME_PROP_ROW(2) FWIME_PROP_ROW(3) FWIME_PROP_ROW(4)
         FWIME_PROP_ROW(5) FWIME_PROP_ROW(6) FWIME_PROP_ROW(7) FWIME_PROP_ROW(8)
     }
-    for (; z < z1; ++z) {   // the last (z1 - z0) mod 9 rows: shift the queue by one register per row
-        FWIME_PROP_ROW(0)
-#pragma unroll
-        for (int k = 0; k < 8; ++k) q[k] = q[k + 1];
-    }
 #undef FWIME_PROP_ROW
     cp_wait<0>();
+    float *out = sp.out + so;
     if (INJ && xin) {
         // receivers in this warp's rows: each lane adds the injection to the outputs it wrote itself (read
         // back by the writing thread), after the march so the loop above keeps its registers
@@ -495,10 +479,10 @@ __global__ void __launch_bounds__(PROP_WARPS * 32, LOC == 2 ? FWIME_PROP_MIN_BLO
             *dp = a.rec_acc ? *dp + val : val;
         }
     }
-    const int wic = threadIdx.x >> 5;
+    const int wic = warp_in_cta();
     const int wid = blockIdx.x * PROP_WARPS + wic;
     if (wid >= a.nstrip * a.nchunk) return;   // warp-uniform
-    float *wsm = reinterpret_cast<float *>(smem4) + wic * (CUR_SLOTS * CUR_ROW + AUX_SLOTS * a.naux_max * STRIP);
+    float *wsm = reinterpret_cast<float *>(smem4) + wic * prop_smem(a.naux_max);
     prop_body<LOC, D2, SRC, INJ, FS, false>(a, a, wid, blockIdx.y, wsm);
 }
 
@@ -535,7 +519,7 @@ static cudaError_t dispatch_prop(const PropArgs &a0, int nshot, cudaStream_t st)
     const bool d2 = a.d2 != nullptr;
     const bool src = a.src_off != nullptr;
     a.naux_max = 2 + (local ? (a.f0 != nullptr) + (a.f1 != nullptr) + (a.f2 != nullptr) + (a.fc ? 2 : 0) : 0);
-    const size_t smem = (size_t)PROP_WARPS * (CUR_SLOTS * CUR_ROW + AUX_SLOTS * a.naux_max * STRIP) * sizeof(float);
+    const size_t smem = (size_t)PROP_WARPS * prop_smem(a.naux_max) * sizeof(float);
     const int loc = !local ? 0 : (a.f1 || a.f2 || a.fc || !a.f0) ? 2 : 1;
     const int key = loc * 4 + (d2 ? 2 : 0) + (src ? 1 : 0);
     if (a.inj_val) {                           // the caller injects only into plain steps, with or without D2t

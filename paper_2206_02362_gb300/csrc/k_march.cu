@@ -60,9 +60,9 @@ __global__ void __launch_bounds__(march_warps<LOC>() * 32, 1) k_march(const __gr
 {
     extern __shared__ float4 smem4[];
     const PropArgs &a = m.a;
-    const int wic = threadIdx.x >> 5, nw = gridDim.x * (blockDim.x >> 5);
+    const int wic = warp_in_cta(), nw = gridDim.x * (blockDim.x >> 5);
     const int gw = blockIdx.x * (blockDim.x >> 5) + wic;
-    float *wsm = reinterpret_cast<float *>(smem4) + wic * (CUR_SLOTS * CUR_ROW + AUX_SLOTS * a.naux_max * STRIP);
+    float *wsm = reinterpret_cast<float *>(smem4) + wic * prop_smem(a.naux_max);
     for (int k = 0; k < m.nsteps; ++k) {
         StepPtrs sp{a.cur, a.prev, a.out, a.d2, a.f0, a.fc, a.src_amp, a.inj_val};
         if (m.R > 0) {                                          // adjoint ring, m descending
@@ -103,7 +103,7 @@ static cudaError_t launch_march_t(const MarchArgs &m, int nsm, cudaStream_t st)
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_march<LOC, D2, SRC, INJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, MARCH_SMEM);
     if (attr != cudaSuccess) return attr;
-    const int per_warp = (CUR_SLOTS * CUR_ROW + AUX_SLOTS * m.a.naux_max * STRIP) * (int)sizeof(float);
+    const int per_warp = prop_smem(m.a.naux_max) * (int)sizeof(float);
     const int wmax = std::min(m.warps, MARCH_SMEM / per_warp);
     // a small problem in CTAs of four warps: fewer arrivals at the barrier, and still spread over many SMs (45 k points:
     // 3.80 us per step, with one warp per CTA 3.82, with eight 4.13, with sixteen 5.07)

@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_MINB) k_prop_pair(const 
         }
     }
     const int lane = threadIdx.x & 31;
-    const int wic = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);   // (a warp-uniform value)
+    const int wic = warp_in_cta();
     const int wid = blockIdx.x * PAIR_WARPS + wic;
     if (wid >= a.nstrip * a.nchunk) return;   // warp-uniform
     const int NXP = a.NXP;

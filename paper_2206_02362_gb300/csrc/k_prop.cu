@@ -29,10 +29,10 @@ __global__ void __launch_bounds__(PROP_WARPS * 32, 4) k_prop_group(const GroupMe
     const int local = (int)blockIdx.x - m[lo].cta_begin;
     const int cps = m[lo].ctas_per_shot;
     const int shot = local / cps;
-    const int wic = threadIdx.x >> 5;
+    const int wic = warp_in_cta();
     const int wid = (local - shot * cps) * PROP_WARPS + wic;
     if (wid >= sa.nstrip * sa.nchunk) return;   // warp-uniform
-    float *wsm = reinterpret_cast<float *>(smem4) + wic * (CUR_SLOTS * CUR_ROW + AUX_SLOTS * 2 * STRIP);
+    float *wsm = reinterpret_cast<float *>(smem4) + wic * prop_smem(2);
     prop_body<0, false, true, false, false, false>(sa, sa, wid, shot, wsm);
 }
 
@@ -56,7 +56,10 @@ __global__ void k_points_group(const GroupRec *__restrict__ g, int nactive, int 
 cudaError_t launch_prop_group(const GroupMember *m, int nactive, int ctas, const GroupRec *g, int nrec_threads,
                               int step, cudaStream_t st, bool record)
 {
-    const size_t smem = (size_t)PROP_WARPS * (CUR_SLOTS * CUR_ROW + AUX_SLOTS * 2 * STRIP) * sizeof(float);
+    const size_t smem = (size_t)PROP_WARPS * prop_smem(2) * sizeof(float);
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_prop_group, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (attr != cudaSuccess) return attr;
     if (!record) {
         k_prop_group<<<ctas, PROP_WARPS * 32, smem, st>>>(m, nactive, step);
     } else {
@@ -68,7 +71,10 @@ cudaError_t launch_prop_group(const GroupMember *m, int nactive, int ctas, const
 // Resident CTAs per SM of the plain (no local source) variant with the smem it launches with.
 cudaError_t prop_occupancy(int *blocks_per_sm)
 {
-    const size_t smem = (size_t)PROP_WARPS * (CUR_SLOTS * CUR_ROW + AUX_SLOTS * 2 * STRIP) * sizeof(float);
+    const size_t smem = (size_t)PROP_WARPS * prop_smem(2) * sizeof(float);
+    const cudaError_t e = cudaFuncSetAttribute(k_prop<0, false, false, false, false>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+    if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_prop<0, false, false, false, false>, PROP_WARPS * 32,
                                                          smem);
 }
