@@ -18,7 +18,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libfwime.so")
-SOURCES = ["fwime_api.cu", "k_prop.cu", "k_prop_fs.cu", "k_march.cu", "k_pair.cu", "k_scatter.cu", "k_image.cu", "k_misc.cu", "k_spline.cu", "k_tlag.cu", "fwime_static.cu", "fwime_serve.cu"]
+SOURCES = ["fwime_api.cu", "k_prop.cu", "k_prop_fs.cu", "k_pair.cu", "k_scatter.cu", "k_image.cu", "k_misc.cu", "k_spline.cu", "k_tlag.cu", "fwime_static.cu", "fwime_serve.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

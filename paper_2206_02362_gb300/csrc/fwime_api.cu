@@ -14,7 +14,11 @@
 //     scattered) state at every segment start during a forward sweep, then walk
 //     the segments backwards: recompute the segment's D2t fields into rings,
 //     step the adjoint fields down through it, and reduce the imaging
-//     conditions over the segment's K x S pairs in one launch.
+//     conditions over the segment's K x S pairs in one launch.  Where they fit
+//     and pay (hist_pays) the D2t fields of the whole record are kept by the
+//     forward sweep instead, and nothing is recomputed.
+// A run of steps (steps()) is one launch per step, or per two steps for batches
+// beyond the L2 cache.
 // The adjoint wavefield uses mu = c g lambda, which obeys the forward recursion
 // run backwards, so forward and adjoint share the stencil kernel.
 #include <cuda_runtime.h>
@@ -56,8 +60,6 @@ struct fwime_ctx {
     size_t max_ws = 0;
     int device = 0;
     size_t dev_mem = 0;             // total memory of the device
-    int coop_sms = 0;               // SMs for cooperative launches (0: not supported)
-    unsigned *d_bar = nullptr;      // grid barrier of the many-step launches: arrivals, generation
     // options
     int opt_S = 0, opt_K = 0, opt_plain = 0, opt_graph = 0, opt_host_io = 0, opt_zchunk = 0, opt_reuse_bg = 0;
     int opt_tlag = 0;               // > 0: B~ / B~* extend with time lags spaced opt_tlag steps
@@ -128,11 +130,27 @@ Server *ctx_server(const fwime_ctx *x) { return x ? x->srv : nullptr; }
 void ctx_set_shared(fwime_ctx *x) { x->shared = true; }
 
 // No other stream's work is expected beside this context's: it runs on the default stream, where calls follow one
-// another whoever makes them.  Only then is one call's latency bought with the whole chip (many steps per cooperative
-// launch, items of a few rows): on streams of their own, eight threads with one small shot each complete 657 calls/s
-// without either, 463 with the short items and 316 with both.
+// another whoever makes them.  Only then does one call's latency come before the work in all (items of a few rows,
+// which load three times the rows that they write): on streams of their own, eight threads with one small shot each
+// complete 889 calls/s with items of eight rows or more, and made 463 with short ones where long ones made 657.
 static bool alone(const fwime_ctx *x) { return !x->shared && x->st == nullptr; }
 }  // namespace fwk
+
+// Bytes of memory of device `dev`, asked for once (the query takes about a millisecond).
+static size_t device_memory(int dev)
+{
+    static std::mutex mu;
+    static std::map<int, size_t> known;
+    const std::lock_guard<std::mutex> lock(mu);
+    const auto it = known.find(dev);
+    if (it != known.end()) return it->second;
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return known[dev] = tot;
+}
 
 // operator entry points refuse a server context
 #define NOT_SERVER(x)                                                                                  \
@@ -582,7 +600,7 @@ static void init_run(fwime_ctx *x, Run &r, int S)
     if (zc <= 0) {
         // 4 CTAs of 4 warps per SM.  Beside other streams the total work counts, not one launch's latency: items of a
         // few rows load three times the rows that they write.
-        zc = chunk_rows(rows, r.nstrip, std::max(S, 1), 152LL * 16, nullptr);
+        zc = chunk_rows(rows, r.nstrip, std::max(S, 1), 152LL * 16);
         if (!alone(x)) zc = std::max(zc, 8);
     }
     zc = std::min(zc, std::max(1, INT_MAX / x->NXP - 16));   // (offsets within an item are 32-bit)
@@ -681,8 +699,6 @@ struct Steps {
     int rec_acc = 0;
     const float *inj = nullptr;     // data row of the first step (the row before follows)
 };
-constexpr int MARCH_STEPS = 256;    // steps per launch at most: other streams get the SMs in between
-
 static int record(Run &r, int Sb, const float *f1, const float *f2, float *d, int accumulate)
 {
     fwime_ctx *x = r.x;
@@ -710,26 +726,11 @@ static int steps(Run &r, int Sb, int n, Steps &p)
                          InjFrom{inj ? inj - (long long)k * x->nrec : nullptr});
     };
     const auto first = args(0, p.R ? slot(p.m0) : p.prev);
-    // few shots on a small grid: many steps per launch (not in the plain path, nor where every step is timed, nor
-    // beside other streams, whose launches a cooperative one would wait for and hold up)
-    const bool many = n > 2 && x->coop_sms > 0 && alone(x) && !x->opt_plain && !x->opt_profile &&
-                      march_pays(first, Sb, x->coop_sms);
     // large batches: two steps per launch (a first single one where their number is odd)
-    const bool pairs = !many && n >= 2 && !x->opt_plain && (p.R || r.alt[0]) && pair_pays(x->P, Sb) && pair_runs(first);
+    const bool pairs = n >= 2 && !x->opt_plain && (p.R || r.alt[0]) && pair_pays(x->P, Sb) && pair_runs(first);
     int paired = 0;
     for (int k = 0; k < n;) {
-        if (many) {
-            MarchArgs m{};
-            m.a = args(k, p.R ? slot(p.m0 - k) : p.prev);
-            m.nsteps = std::min(n - k, MARCH_STEPS);
-            m.S = Sb;
-            m.ring = p.ring; m.rstride = SP; m.R = p.R; m.m0 = p.m0 - k;
-            m.d2_step = p.d2_step; m.f0_step = p.f0_step; m.fc_step = p.fc_step; m.rec_step = x->nrec; m.inj_step = -x->nrec;
-            m.bar = x->d_bar; m.status = x->d_status;
-            LAUNCH(FWIME_K_PROP, m.nsteps * prop_bytes(x, m.a, Sb), launch_march(m, x->coop_sms, x->st));
-            k += m.nsteps;
-            if (m.nsteps & 1) std::swap(p.cur, p.prev);
-        } else if (pairs && (n - k) % 2 == 0) {
+        if (pairs && (n - k) % 2 == 0) {
             PairArgs m{};
             m.a = args(k, p.R ? slot(p.m0 - k) : r.alt[0]);
             m.out2 = p.R ? slot(p.m0 - k - 1) : r.alt[1];
@@ -1845,15 +1846,7 @@ int fwime_create(fwime_ctx **out, const fwime_grid *g, const fwime_geom *geo, si
     x->st = reinterpret_cast<cudaStream_t>(cuda_stream);
     x->max_ws = max_workspace_bytes;
     cudaGetDevice(&x->device);
-    size_t free_mem = 0;
-    if (cudaMemGetInfo(&free_mem, &x->dev_mem) != cudaSuccess) {
-        cudaGetLastError();
-        x->dev_mem = 0;
-    }
-    int coop = 0, nsm = 0;
-    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, x->device) == cudaSuccess && coop &&
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, x->device) == cudaSuccess)
-        x->coop_sms = nsm;
+    x->dev_mem = device_memory(x->device);
     // offsets: [src_off(nshot)][rec_off(nrec)]
     x->h_off.resize(x->nshot + x->nrec);
     for (int s = 0; s < x->nshot; ++s) x->h_off[s] = (x->src_iz[s] + x->o) * x->NXP + x->src_ix[s] + x->o;
@@ -1878,7 +1871,7 @@ int fwime_create(fwime_ctx **out, const fwime_grid *g, const fwime_geom *geo, si
             last[pos] = r;
         }
     }
-    const size_t off_inj = ((1 + 1024) * sizeof(double) + sizeof(int) * (3 + x->h_off.size()) + 15) / 16 * 16;
+    const size_t off_inj = ((1 + 1024) * sizeof(double) + sizeof(int) * (1 + x->h_off.size()) + 15) / 16 * 16;
     const size_t small_bytes = off_inj + sizeof(int) * x->h_inj.size();
     double *slot = pinned_slot();
     bool ok = slot != nullptr &&
@@ -1889,8 +1882,7 @@ int fwime_create(fwime_ctx **out, const fwime_grid *g, const fwime_geom *geo, si
         x->d_J = reinterpret_cast<double *>(x->small);
         x->d_part = x->d_J + 1;
         x->d_status = reinterpret_cast<int *>(x->d_part + 1024);
-        x->d_bar = reinterpret_cast<unsigned *>(x->d_status + 1);
-        x->d_src_off = x->d_status + 3;
+        x->d_src_off = x->d_status + 1;
         x->d_rec_off = x->d_src_off + x->nshot;
         x->d_inj_map = reinterpret_cast<int *>(reinterpret_cast<char *>(x->small) + off_inj);
         x->d_inj_next = x->d_inj_map + nmap;
@@ -2595,10 +2587,6 @@ int fwime_sync(fwime_ctx *x)
             CK(cudaMemcpy(x->vp_hist_user, x->vp_hist_dev, x->vp_hist_n * sizeof(double), cudaMemcpyDeviceToHost));
         CK(cudaFreeAsync(x->vp_hist_dev, x->st));
         x->vp_hist_dev = x->vp_hist_user = nullptr;
-    }
-    if (st & ST_TIMEOUT) {
-        CK(cudaMemsetAsync(x->d_bar, 0, 2 * sizeof(unsigned), x->st));
-        return fail(x, FWIME_ETIMEOUT, "a many-step launch gave up waiting at its grid barrier");
     }
     if (st & ST_CFL) return fail(x, FWIME_ECFL, "velocity violates the CFL bound or is not positive");
     return FWIME_OK;

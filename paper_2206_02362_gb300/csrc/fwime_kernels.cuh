@@ -24,7 +24,6 @@ constexpr int MAX_NH = 201;     // largest supported number of subsurface offset
 // status bits latched by kernels
 constexpr int ST_CFL = 1;
 constexpr int ST_BADV = 2;
-constexpr int ST_TIMEOUT = 4;   // a bounded device-side wait gave up
 
 // Largest eigenvalue of -h^2 D2 for the 8th-order second-derivative stencil (its symbol at the Nyquist
 // wavenumber: 205/72 + 2 (8/5 + 1/5 + 8/315 + 1/560)).  The leapfrog scheme is stable while
@@ -104,21 +103,6 @@ struct PairArgs {
     float *out2, *d2b;
     const float *f0b, *inj_val2;   // (the second step's source amplitude follows the first's)
     int rec_prev;                  // record prev's receivers too, one row of the data earlier
-};
-
-// several time steps in one cooperative launch (k_march): step k's operands from those of step 0 in `a`
-struct MarchArgs {
-    PropArgs a;
-    int nsteps, S;
-    // R = 0: cur and out (= prev) swap from step to step.  R > 0: the fields are slots of a ring, floats apart
-    // `rstride`: out = slot m, cur = m + 1, prev = m + 2 (mod R), m = m0 - k
-    float *ring;
-    long long rstride;
-    int R, m0;
-    long long d2_step, f0_step, fc_step, rec_step, inj_step;   // floats from one step's operand to the next's
-    unsigned *bar;                 // grid barrier: arrivals, generation (zero at first use)
-    int *status;
-    int nitem, per_shot, warps;    // set by launch_march: items in all and per shot, warps per CTA at most
 };
 
 // grouped forward: one member = one shot batch on its own grid
@@ -204,10 +188,8 @@ struct TlagArgs {
 // launchers (return cudaGetLastError())
 cudaError_t launch_prop(const PropArgs &a, int nshot, cudaStream_t st);
 cudaError_t prop_occupancy(int *blocks_per_sm);
-int chunk_rows(int rows, int nstrip, int S, long long warps, long long *cost_out, int overhead = 6,
-               int start = 0);   // rows per warp
-bool march_pays(const PropArgs &a, int S, int nsm);
-cudaError_t launch_march(const MarchArgs &m, int nsm, cudaStream_t st);
+// rows per warp
+int chunk_rows(int rows, int nstrip, int S, long long warps, int overhead = 6, int start = 0, int crowd = 5);
 cudaError_t launch_pair(const PairArgs &m, int nshot, cudaStream_t st);
 bool pair_runs(const PropArgs &a);
 bool pair_pays(long long P, int S);

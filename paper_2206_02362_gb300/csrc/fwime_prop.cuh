@@ -49,7 +49,7 @@ __device__ __forceinline__ float4 shfl_down4(float4 v)
     return v;
 }
 
-// ---- asynchronous global -> shared copies (LDGSTS); 
+// ---- asynchronous global -> shared copies (LDGSTS)
 __device__ __forceinline__ void cp16n(float *dst, const float *src, int n)   // n: 16, or 0 to zero-fill
 {
     const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
@@ -61,8 +61,11 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0
 __device__ __forceinline__ float4 lds4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 
 // Per-warp pipeline: rings of nine rows of q^n (128 points + 4-point halos, for the x-taps and the register queue),
-// q^{n-1} and c; with local sources rings of three rows of those, of q^{n-1} and of c.  Nine is the period of the unrolled register queue, so every
-// slot is a compile-time constant.  Row z waits for the copy group issued four rows (with local sources three) earlier.
+// q^{n-1} and c; with local sources rings of three rows of those, of q^{n-1} and of c.  Nine is the period of the
+// unrolled register queue, so every slot is a compile-time constant.  Row z waits for the copy group issued four rows
+// (with local sources three) earlier.  With slots and addresses computed per row and lane a row of 128 points took 211
+// instructions and 124 registers, now 102 to 108: 350 x 1700 points, 8 shots, 15.8 / 13.9 us per step; from about 16
+// shots on the kernel is bound by memory and the two are equal.
 constexpr int RING = 9, LRING = 3;
 // Variants k_prop<LOC, D2, SRC>: LOC = 0 no dense local source, 1 exactly one (f0, weight a0), 2 the
 // general sum a0 f0 + a1 f1 + a2 f2 + coef fc; D2 writes D2t; SRC adds the point source.  Register
@@ -265,25 +268,23 @@ __device__ __forceinline__ void inject_row(const PropArgs &a, const float *val, 
 
 // The time step of one warp's work item (strip, chunk) of shot `shot`; wsm is the warp's shared
 // memory (prop_smem(naux_max) floats).  wid is warp-uniform and known to be so (a shuffle's result): the address
-// arithmetic is then done once per warp.  sp: the operands that change from step to step
-// (the same members of PropArgs).  COH: the fields change during the kernel (several steps per launch), so no read of
-// them may come from a non-coherent cache.
-template <int LOC, bool D2, bool SRC, bool INJ, bool FS, bool COH, class SP>
-__device__ __forceinline__ void prop_body(const PropArgs &a, const SP &sp, const int wid, const int shot, float *wsm)
+// arithmetic is then done once per warp.
+template <int LOC, bool D2, bool SRC, bool INJ, bool FS>
+__device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, const int shot, float *wsm)
 {
     constexpr bool LOCAL = LOC > 0;
     const int lane = threadIdx.x & 31;
     const int strip = wid % a.nstrip, chunk = wid / a.nstrip;
     const int x0 = strip * STRIP;
     const int x = x0 + lane * 4;
-    const int z0 = (FS || COH ? a.z_first : 4) + chunk * a.zchunk;
+    const int z0 = (FS ? a.z_first : 4) + chunk * a.zchunk;
     const int z1 = min(z0 + a.zchunk, a.NZ - 4);
     const bool xin = x < a.NXP;
     const int NXP = a.NXP;
     const long long so = (long long)shot * a.P, row0 = (long long)z0 * NXP;
-    const float *__restrict__ cur = sp.cur + so + row0;
-    const float *prev = sp.prev + so + row0, *c = a.c + row0;
-    float *out0 = sp.out + so + row0, *d20 = D2 ? sp.d2 + so + row0 : nullptr;
+    const float *__restrict__ cur = a.cur + so + row0;
+    const float *prev = a.prev + so + row0, *c = a.c + row0;
+    float *out0 = a.out + so + row0, *d20 = D2 ? a.d2 + so + row0 : nullptr;
 
     // the lane's places in the rings; local sources: [f0?][f1?][f2?][coef, fc?] (LOC 1: exactly one, f0, weight a0)
     const int i_f1 = a.f0 != nullptr, i_f2 = i_f1 + (a.f1 != nullptr), i_cf = i_f2 + (a.f2 != nullptr);
@@ -316,14 +317,14 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const SP &sp, const
         const long long o = row0 + (lin ? (long long)k * NXP + oX : 0);
         float *dst = fL + s * nloc * STRIP;
         if (LOC == 1) {
-            cp16n(dst, sp.f0 + so + o, n);
+            cp16n(dst, a.f0 + so + o, n);
         } else {
-            if (a.f0) cp16n(dst, sp.f0 + so + o, n);
+            if (a.f0) cp16n(dst, a.f0 + so + o, n);
             if (a.f1) cp16n(dst + i_f1 * STRIP, a.f1 + so + o, n);
             if (a.f2) cp16n(dst + i_f2 * STRIP, a.f2 + so + o, n);
             if (a.fc) {
                 cp16n(dst + i_cf * STRIP, a.coef + o, n);
-                cp16n(dst + (i_cf + 1) * STRIP, sp.fc + so + o, n);
+                cp16n(dst + (i_cf + 1) * STRIP, a.fc + so + o, n);
             }
         }
     };
@@ -333,7 +334,7 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const SP &sp, const
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const float *qp = cur + (long long)(k - 4) * NXP + oX;
-        q[k] = !xin ? f4zero() : COH ? __ldcg(reinterpret_cast<const float4 *>(qp)) : ldg4(qp);
+        q[k] = xin ? ldg4(qp) : f4zero();
     }
     // prologue: one group per row of look-ahead (rows z0 .. z0+3 feed the first x-taps)
     constexpr int DEPTH = LOCAL ? LRING : 4;
@@ -357,7 +358,7 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const SP &sp, const
         srow = off / NXP;
         scol = off - srow * NXP - x;
         if (scol < 0 || scol > 3) srow = -1;
-        amp = sp.src_amp[(long long)shot * a.src_stride] * a.src_scale;
+        amp = a.src_amp[(long long)shot * a.src_stride] * a.src_scale;
     }
 
     // One output row z; the queue's logical row k (z-4+k) lives in q[(k + R) % 9], so nine consecutive rows rotate
@@ -410,7 +411,7 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const SP &sp, const
     }
 #undef FWIME_PROP_ROW
     cp_wait<0>();
-    float *out = sp.out + so;
+    float *out = a.out + so;
     if (INJ && xin) {
         // receivers in this warp's rows: each lane adds the injection to the outputs it wrote itself (read
         // back by the writing thread), after the march so the loop above keeps its registers
@@ -422,14 +423,14 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const SP &sp, const
             const float4 o0 = *reinterpret_cast<const float4 *>(out + idx);
             float4 o = o0;
             const float4 cv = ldg4(a.c + idx);
-            inject_point(a, sp.inj_val, shot, m4.x, cv.x, o.x);
-            inject_point(a, sp.inj_val, shot, m4.y, cv.y, o.y);
-            inject_point(a, sp.inj_val, shot, m4.z, cv.z, o.z);
-            inject_point(a, sp.inj_val, shot, m4.w, cv.w, o.w);
+            inject_point(a, a.inj_val, shot, m4.x, cv.x, o.x);
+            inject_point(a, a.inj_val, shot, m4.y, cv.y, o.y);
+            inject_point(a, a.inj_val, shot, m4.z, cv.z, o.z);
+            inject_point(a, a.inj_val, shot, m4.w, cv.w, o.w);
             st4(out + idx, o);
             if (D2 && zz >= a.zs_lo && zz < a.zs_hi) {
                 // the D2t output gains the injection too: d2 + (o - o0) / dt^2
-                float *dp = sp.d2 + so + idx;
+                float *dp = a.d2 + so + idx;
                 float4 d = *reinterpret_cast<const float4 *>(dp);
                 d.x = fmaf(o.x - o0.x, a.inv_dt2, d.x);
                 d.y = fmaf(o.y - o0.y, a.inv_dt2, d.y);
@@ -439,7 +440,7 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const SP &sp, const
             }
         }
     }
-    if ((FS || COH) && a.fs_row > 0 && xin) {
+    if (FS && xin) {
         // Free surface (pressure release on row fs_row, where the march starts): q = 0 and D2t = 0 there, and the four
         // rows above hold the odd mirror of the four below, each written by the lane that owns the row below (which
         // it reads back: its own stores, injection included); rows further up stay zero.  As a launch of its own
@@ -449,7 +450,7 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const SP &sp, const
             const long long idx = (long long)zz * NXP + x;
             if (zz == a.fs_row) {
                 st4(out + idx, f4zero());
-                if (D2) st4(sp.d2 + so + idx, f4zero());
+                if (D2) st4(a.d2 + so + idx, f4zero());
             } else {
                 const float4 o = *reinterpret_cast<const float4 *>(out + idx);
                 st4(out + (long long)(2 * a.fs_row - zz) * NXP + x, make_float4(-o.x, -o.y, -o.z, -o.w));
@@ -483,7 +484,7 @@ __global__ void __launch_bounds__(PROP_WARPS * 32, LOC == 2 ? FWIME_PROP_MIN_BLO
     const int wid = blockIdx.x * PROP_WARPS + wic;
     if (wid >= a.nstrip * a.nchunk) return;   // warp-uniform
     float *wsm = reinterpret_cast<float *>(smem4) + wic * prop_smem(a.naux_max);
-    prop_body<LOC, D2, SRC, INJ, FS, false>(a, a, wid, blockIdx.y, wsm);
+    prop_body<LOC, D2, SRC, INJ, FS>(a, wid, blockIdx.y, wsm);
 }
 
 template <bool FS, int LOC, bool D2, bool SRC, bool INJ = false>

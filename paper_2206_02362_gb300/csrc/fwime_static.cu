@@ -155,7 +155,7 @@ extern "C" int fwime_forward_static(const fwime_grid *g, const fwime_geom *geo, 
     a.NZ = NZ; a.NXP = NXP; a.P = P;
     a.nstrip = (NXP + STRIP - 1) / STRIP;
     const int rows = NZ - 8;
-    a.zchunk = chunk_rows(rows, a.nstrip, nshot, 152LL * 16, nullptr);
+    a.zchunk = chunk_rows(rows, a.nstrip, nshot, 152LL * 16);
     a.nchunk = (rows + a.zchunk - 1) / a.zchunk;
     const double A8[5] = {-205.0 / 72.0, 8.0 / 5.0, -1.0 / 5.0, 8.0 / 315.0, -1.0 / 560.0};
     for (int k = 0; k < 5; ++k) {

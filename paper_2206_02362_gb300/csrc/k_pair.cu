@@ -14,8 +14,8 @@ namespace fwk {
 //
 // What it took: every ring slot a compile-time constant (rings of nine rows, the period of the unrolled queues), a
 // warp index that the compiler knows to be uniform, running offsets and one barrier per row (with addresses computed
-// per row 91 ms where this takes 51 and k_prop 67: forward, 100 shots on 458 x 1808 points, 399 steps); two CTAs of
-// four warps per SM (three: 60 ms), four rows in flight (three: 59).
+// per row 91 ms where this takes 51 and k_prop 67: forward, 100 shots on 458 x 1808 points, 399 steps); registers
+// for two CTAs of four warps per SM, of which three fit (bounded to 168: 60 ms), four rows in flight (three: 59).
 constexpr int PAIR_WARPS = 4, PAIR_MINB = 2;
 constexpr int PAIR_STRIP = STRIP - 8;        // columns that a warp writes: the first step's halo costs it two lanes
 constexpr int PAIR_RING = 9;                 // rows per ring
@@ -211,6 +211,13 @@ static cudaError_t launch_pair_t(const PairArgs &m, int nshot, cudaStream_t st)
     static const cudaError_t attr = cudaFuncSetAttribute(k_prop_pair<LOC, D2, SRC, INJ>,
                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
     if (attr != cudaSuccess) return attr;
+    // Shared memory for the three CTAs that the registers allow, the rest to L1, whatever the launch before had: right
+    // behind k_prop, which takes all of it, pairs took 54.3 ms where they take 51.1 (a launch that follows without a
+    // gap keeps the split unless it asks for another).
+    constexpr int cta = sizeof(float) * PAIR_WARPS * pair_smem(LOC) + 1024, carve = (3 * cta * 100 + 233471) / 233472 + 1;
+    static const cudaError_t attr2 = cudaFuncSetAttribute(k_prop_pair<LOC, D2, SRC, INJ>,
+                                                          cudaFuncAttributePreferredSharedMemoryCarveout, carve);
+    if (attr2 != cudaSuccess) return attr2;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((m.a.nstrip * m.a.nchunk + PAIR_WARPS - 1) / PAIR_WARPS, nshot);
     cfg.blockDim = dim3(PAIR_WARPS * 32);
@@ -247,7 +254,7 @@ cudaError_t launch_pair(const PairArgs &m0, int nshot, cudaStream_t st)
     a.nstrip = (a.NXP + PAIR_STRIP - 1) / PAIR_STRIP;
     // an item computes eight rows more than it writes; with half a round for a launch's ends, four shots on 1300 rows
     // take 57 us per step in three rounds instead of 61 in one
-    a.zchunk = chunk_rows(rows, a.nstrip, nshot, 152LL * PAIR_MINB * PAIR_WARPS, nullptr, 12, 1);
+    a.zchunk = chunk_rows(rows, a.nstrip, nshot, 152LL * PAIR_MINB * PAIR_WARPS, 12, 1, 0);
     a.nchunk = (rows + a.zchunk - 1) / a.zchunk;
     const bool d2 = a.d2 != nullptr;
     if (a.inj_val)

@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(PROP_WARPS * 32, 4) k_prop_group(const GroupMe
     const int wid = (local - shot * cps) * PROP_WARPS + wic;
     if (wid >= sa.nstrip * sa.nchunk) return;   // warp-uniform
     float *wsm = reinterpret_cast<float *>(smem4) + wic * prop_smem(2);
-    prop_body<0, false, true, false, false, false>(sa, sa, wid, shot, wsm);
+    prop_body<0, false, true, false, false>(sa, wid, shot, wsm);
 }
 
 // after step n the new field q^{n+1} of a member is in buffer B for even n, A for odd n
@@ -81,20 +81,22 @@ cudaError_t prop_occupancy(int *blocks_per_sm)
 
 // Rows per warp's item: the items (strip, chunk of rows) of S shots go to `warps` resident warps in rounds of equal
 // length; the split of the rows with the least (rounds + start / 2) x (rows + overhead) wins: overhead is about what an
-// item's start costs, start / 2 the part of a round that a launch's ramp and drain take.
+// item's start costs, start / 2 the part of a round that a launch's ramp and drain take, crowd / 2 what it costs that
+// the items fill more than half of the places, so that the next launch's CTAs cannot wait there.
 // Marmousi2-shaped, us per launch with the former aim of 4864 warps and with this: 32 shots 69 / 60, 50 shots 100 / 87,
-// 100 shots 178 / 169.
-int chunk_rows(int rows, int nstrip, int S, long long warps, long long *cost_out, int overhead, int start)
+// 100 shots 178 / 169.  One shot, ms per 1500 steps on 560 x 1260 points: 7.56 in 418 CTAs of 3 rows per warp, 7.15 in
+// 253 of 5; per 1000 steps on 160 x 260 points: 2.71 of 2 rows, 2.55 of 1.
+int chunk_rows(int rows, int nstrip, int S, long long warps, int overhead, int start, int crowd)
 {
     long long best = -1;
     int best_zc = rows;
-    for (int c = 1; c <= (rows + 1) / 2; ++c) {
+    for (int c = 1; c <= rows; ++c) {
         const int zc = (rows + c - 1) / c;
         const long long items = (long long)nstrip * S * ((rows + zc - 1) / zc);
-        const long long cost = (2 * ((items + warps - 1) / warps) + start) * (zc + overhead);
+        const long long cost = (2 * ((items + warps - 1) / warps) + start) * (zc + overhead) +
+                               (2 * items > warps ? crowd : 0);
         if (best < 0 || cost <= best) { best = cost; best_zc = zc; }   // ties: the more, shorter items
     }
-    if (cost_out) *cost_out = std::max(best, 0LL) / 2;
     return std::max(best_zc, 1);
 }
 

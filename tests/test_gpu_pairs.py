@@ -51,7 +51,7 @@ def test_pairs_of_steps(op, nh, opts, nz, nx, sponge, nt):
     nshot = -(-13000000 // points)
     geom, t = inputs(nz, nx, nt, nshot, nh)
     grid = fw.Grid(nz=nz, nx=nx, sponge=sponge, nt=nt, dt=1e-3, dx=10.0, nh=nh)
-    st = torch.cuda.Stream()                 # (on the default stream small grids take many steps per launch)
+    st = torch.cuda.Stream()
     torch.cuda.synchronize()
     with torch.cuda.stream(st):
         with fw.Context(grid, geom, stream=st, shots_per_batch=nshot, **opts) as ctx:
