@@ -144,7 +144,8 @@ int fwime_create(fwime_ctx **out, const fwime_grid *g, const fwime_geom *geo,
                  size_t max_workspace_bytes, void *cuda_stream);
 
 /* Device bytes operator `op` needs for `shots_per_batch` shots advanced
- * together with segment length `segment` (0 = the defaults). */
+ * together with segment length `segment` (0 = the defaults).  A context takes
+ * more where that is faster and fits: kept histories, two further fields. */
 int fwime_workspace_bytes(const fwime_grid *g, const fwime_geom *geo, int op,
                           int shots_per_batch, int segment, size_t *bytes);
 
