@@ -532,7 +532,8 @@ def main():
                                if p["ms"] > 0},
                 "bytes_rule": "12 B per shot-point (q^n, q^n-1 in, q^n+1 out) over the padded NZ x NX points "
                               "+ 4 B per grid point per launch for c (shared by all shots) + 4 B per shot-point "
-                              "per D2t or local-source field over the physical rows (nz x NX points)"}
+                              "per D2t or local-source field over the physical rows (nz x NX points); a launch of "
+                              "two steps 16 B per shot-point instead of 24, and c once"}
     shots_per_s = wl.nshot * world / (ms_step * 1e-3)
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,

@@ -738,7 +738,7 @@ static int steps(Run &r, int Sb, int n, Steps &p)
             m.f0b = p.f0 ? p.f0 + (k + 1) * p.f0_step : nullptr;
             m.inj_val2 = inj ? inj - (long long)(k + 1) * x->nrec : nullptr;
             m.rec_prev = paired;
-            LAUNCH(FWIME_K_PROP, 2.0 * prop_bytes(x, m.a, Sb) - 8.0 * Sb * x->NZ * x->NX, launch_pair(m, Sb, x->st));
+            LAUNCH(FWIME_K_PROP, 2.0 * prop_bytes(x, m.a, Sb) - (8.0 * Sb + 4.0) * x->NZ * x->NX, launch_pair(m, Sb, x->st));
             if (!p.R) {
                 std::swap(p.prev, r.alt[0]);
                 std::swap(p.cur, r.alt[1]);
