@@ -1650,13 +1650,31 @@ static void bg_after(fwime_ctx *x, const Call &c, bool wrote)
     }
 }
 
-static int enqueue(fwime_ctx *x, const Call &c)
+// What a call does with the background cache: decided once, before it is planned, enqueued or captured.
+struct Reuse {
+    bool read = false, write = false;
+};
+
+static Reuse reuse_of(fwime_ctx *x, const Call &c)
+{
+    Reuse u;
+    u.read = bg_usable(x, c);
+    u.write = is_bg_writer(c.op) && bg_applies(x, c.op) && x->opt_reuse_bg && bg_reserve(x, seg_K(x));
+    return u;
+}
+
+static int plan_call(fwime_ctx *x, const Call &c, Reuse &u, WS &w)
+{
+    TRY(plan(x, c.op, w, u.read));
+    if (u.write && !x->bg.hist && w.K < seg_K(x)) u.write = false;   // shorter segments than the cache's
+    return FWIME_OK;
+}
+
+static int enqueue(fwime_ctx *x, const Call &c, Reuse &u)
 {
     Run r;
-    const bool use_bg = bg_usable(x, c);
-    x->bg_used = use_bg;
-    x->bg_written = is_bg_writer(c.op) && bg_applies(x, c.op) && x->opt_reuse_bg && bg_reserve(x, seg_K(x));
-    if (x->bg_written) x->bg.valid = false;   // being overwritten
+    x->bg_used = u.read;
+    x->bg_written = u.write;
     if (c.op == OP_GRAD_FWD || c.op == OP_GRAD_BWD) {
         // the split gradient: checkpoints and residual live in the context's gradient state
         TRY(plan(x, c.op == OP_GRAD_FWD ? FWIME_OP_OBJECTIVE : FWIME_OP_GRADIENT, r.w, true));
@@ -1665,20 +1683,21 @@ static int enqueue(fwime_ctx *x, const Call &c)
         return run_tomo_adj(x, r, 1, c.v, c.w, c.in1, c.in2, c.out, c.accumulate, c.eps,
                             c.op == OP_GRAD_FWD ? PH_FORWARD : PH_BACKWARD);
     }
-    TRY(plan(x, c.op, r.w, use_bg));
-    if (r.w.K < seg_K(x) && !(x->bg_written && x->bg.hist)) x->bg_written = false;   // shorter segments than the cache's
+    TRY(plan_call(x, c, u, r.w));
+    x->bg_written = u.write;
+    if (u.write) x->bg.valid = false;   // being overwritten
     init_run(x, r, r.w.S);
     TRY(prep_model(x, r, c.v));
     switch (c.op) {
     case FWIME_OP_FORWARD: return run_forward(x, r, c.v, c.w, c.out);
     case FWIME_OP_BORN: return run_born(x, r, c.v, c.w, c.in1, c.out);
-    case FWIME_OP_BORN_ADJ: return run_born_adj(x, r, false, c.v, c.w, c.in1, c.out, c.accumulate, use_bg);
+    case FWIME_OP_BORN_ADJ: return run_born_adj(x, r, false, c.v, c.w, c.in1, c.out, c.accumulate, u.read);
     case FWIME_OP_BORN_EXT:
         if (x->opt_tlag > 0) return run_born_tlag(x, r, c.w, c.in1, c.out);
         return run_born_ext(x, r, c.v, c.w, c.in1, c.out);
     case FWIME_OP_BORN_EXT_ADJ:
         if (x->opt_tlag > 0) return run_born_tlag_adj(x, r, c.v, c.w, c.in1, c.out, c.accumulate);
-        return run_born_adj(x, r, true, c.v, c.w, c.in1, c.out, c.accumulate, use_bg);
+        return run_born_adj(x, r, true, c.v, c.w, c.in1, c.out, c.accumulate, u.read);
     case FWIME_OP_TOMO:
         if (x->opt_tlag > 0) return run_tomo_tlag(x, r, c.v, c.w, c.in1, c.in2, c.out);
         return run_tomo(x, r, c.v, c.w, c.in1, c.in2, c.out);
@@ -1698,8 +1717,9 @@ static int enqueue(fwime_ctx *x, const Call &c)
 
 static int enqueue_noted(fwime_ctx *x, const Call &c)
 {
-    const int rc = enqueue(x, c);
-    if (rc == FWIME_OK) bg_after(x, c, x->bg_written);
+    Reuse u = reuse_of(x, c);
+    const int rc = enqueue(x, c, u);
+    if (rc == FWIME_OK) bg_after(x, c, u.write);
     return rc;
 }
 
@@ -1711,23 +1731,22 @@ static int run_call(fwime_ctx *x, const Call &c)
     }
     if (x->st == nullptr) return fail(x, FWIME_EINVAL, "graph mode needs a non-default stream");
     // plan (and reserve the background cache) first so that no allocation happens inside a capture
-    const bool use_bg = bg_usable(x, c);
-    const bool write_bg = is_bg_writer(c.op) && bg_applies(x, c.op) && x->opt_reuse_bg && bg_reserve(x, seg_K(x));
-    {
-        WS w;
-        TRY(plan(x, c.op, w, use_bg));
-    }
+    Reuse u = reuse_of(x, c);
+    WS w;
+    TRY(plan_call(x, c, u, w));
+    // a graph that reads or writes the cache has its place, its form and the segments of its states built in
+    const bool cached = u.read || u.write;
     char key[320];
-    snprintf(key, sizeof(key), "%d|%p|%p|%p|%p|%p|%d|%a|%d|%d|%d|%d%d|%p|%d", c.op, (const void *)c.v, (const void *)c.w,
+    snprintf(key, sizeof(key), "%d|%p|%p|%p|%p|%p|%d|%a|%d|%d|%d|%d%d|%p|%d|%d", c.op, (const void *)c.v, (const void *)c.w,
              (const void *)c.in1, (const void *)c.in2, (void *)c.out, c.accumulate, (double)c.eps, x->opt_S, x->opt_K,
-             x->opt_zchunk, use_bg ? 1 : 0, write_bg ? 1 : 0, (const void *)(use_bg || write_bg ? x->bg.buf : nullptr),
-             x->opt_tlag * 2 + x->opt_fs);
+             x->opt_zchunk, u.read ? 1 : 0, u.write ? 1 : 0, (const void *)(cached ? x->bg.buf : nullptr),
+             !cached ? 0 : x->bg.hist ? -1 : w.K, x->opt_tlag * 2 + x->opt_fs);
     auto it = x->graphs.find(key);
     if (it == x->graphs.end()) {
         CK(cudaStreamBeginCapture(x->st, cudaStreamCaptureModeThreadLocal));
         x->capturing = true;
         x->launches = 0;
-        int rc = enqueue(x, c);
+        int rc = enqueue(x, c, u);
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamEndCapture(x->st, &graph);
         x->capturing = false;
@@ -1745,8 +1764,8 @@ static int run_call(fwime_ctx *x, const Call &c)
     }
     x->launches = it->second.launches;
     CK(cudaGraphLaunch(it->second.exec, x->st));
-    x->bg_used = use_bg;
-    bg_after(x, c, write_bg);
+    x->bg_used = u.read;
+    bg_after(x, c, u.write);
     return FWIME_OK;
 }
 

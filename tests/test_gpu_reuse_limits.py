@@ -1,0 +1,64 @@
+"""Background reuse (FWIME_OPT_REUSE_BACKGROUND) where memory is short: the adjoints give the results of the
+self-contained operators, directly and captured in graphs, whatever the writer could keep.  FP32 reorderings only:
+relative L2 <= 2e-6 (the bound between schedules of test_gpu_history), 1e-4 against the FP64 oracle."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+import paper_2206_02362_gb300 as fw  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+NZ, NX, W, DX, DT = 20, 90, 6, 10.0, 1e-3
+PLANE = 4 * (NZ + 2 * (W + 4)) * (-(-(NX + 2 * (W + 4)) // 32) * 32)       # bytes of a padded field
+
+
+def problem(nt, nh):
+    rng = np.random.default_rng(synth.SEED0 + 1201)
+    v = (1800.0 + 25.0 * np.arange(NZ)[:, None] + 60.0 * np.sin(np.arange(NX)[None, :] / 11.0)).astype(np.float32)
+    w = synth.ricker(nt, DT, 22.0)[None].astype(np.float32)
+    a = dict(nz=NZ, nx=NX, nt=nt, dt=DT, dx=DX, nh=nh)
+    g = dict(src_iz=np.array([1]), src_ix=np.array([40]), rec_iz=np.full(30, 1), rec_ix=3 * np.arange(30))
+    x = dict(v=v, w=w, pt=rng.standard_normal((nh, NZ, NX)).astype(np.float32),
+             d=rng.standard_normal((1, nt, 30)).astype(np.float32),
+             dv=(40.0 * np.sin(1.0 + np.arange(NZ)[:, None] / 5.0 + np.arange(NX)[None, :] / 9.0)).astype(np.float32))
+    f64 = {k: q.astype(np.float64) for k, q in x.items()}
+    og, ogeo = oracle.Grid(W=W, **a), oracle.Geometry(**g)
+    ref = dict(born_adj=oracle.born_adj(og, f64["v"], ogeo, f64["w"], f64["d"]),
+               born_ext_adj=oracle.born_ext_adj(og, f64["v"], ogeo, f64["w"], f64["d"]))
+    return fw.Grid(sponge=W, **a), fw.Geometry(**g), {k: torch.from_numpy(np.ascontiguousarray(q)).cuda() for k, q in x.items()}, ref
+
+
+def adjoint(ctx, name, t):
+    out = torch.full(t["pt"].shape if name == "born_ext_adj" else t["v"].shape, 7.0, device="cuda")
+    torch.cuda.synchronize()
+    getattr(ctx, name)(t["v"], t["w"], t["d"], out)
+    return out.cpu().numpy().astype(np.float64)
+
+
+def write(ctx, name, t):
+    getattr(ctx, name)(t["v"], t["w"], t["pt" if name == "born_ext" else "dv"], torch.zeros_like(t["d"]))
+
+
+def close(a, b, tol):
+    assert np.isfinite(a).all() and np.linalg.norm(a - b) <= tol * np.linalg.norm(b)
+
+
+# 399 steps, 41 offsets: a segment of 64 steps takes B~ 175 fields and B* 135, one of 20 steps 87 and 47 (and states)
+@pytest.mark.parametrize("graph", [0, 1])
+@pytest.mark.parametrize("planes", [100, 150, 190])
+@pytest.mark.parametrize("writer,reader", [("born_ext", "born_adj")])
+def test_adjoint_after_a_writer_under_a_cap(graph, planes, writer, reader):
+    grid, geom, t, ref = problem(400, 41)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with fw.Context(grid, geom, segment=20) as ctx:
+        own = adjoint(ctx, reader, t)
+    close(own, ref[reader], 1e-4)
+    with fw.Context(grid, geom, stream=stream, max_workspace_bytes=planes * PLANE, graph=graph,
+                    reuse_background=1) as ctx:
+        for _ in range(2):                    # the second time replays the graphs
+            write(ctx, writer, t)
+            close(adjoint(ctx, reader, t), own, 2e-6)
