@@ -71,7 +71,7 @@ struct fwime_ctx {
         size_t bytes = 0;
         bool valid = false, hist = false;
         const float *v = nullptr, *w = nullptr;
-        int K = 0;
+        int K = 0, seg = 0;             // segment length of the states; the default one (seg_K) when they were written
     } bg;
     bool bg_written = false;        // set by the last enqueued B / B~ that filled the cache
     // state the forward half of the gradient leaves for its adjoint half (fwime_gradient_forward /
@@ -383,20 +383,41 @@ static bool hist_pays(const fwime_ctx *x, int op, int S_h, int S_c)
     return h < c;
 }
 
-// no_ckpt: the source side's states or history are kept outside the workspace
-static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
+// What a call takes from outside its workspace (or leaves there): the background cache, the split gradient's state.
+// Decided once, before the call is planned, enqueued or captured.
+struct Reuse {
+    bool read = false, write = false;
+    int K = 0;          // the segment length that the states read or written have (0: none)
+    bool must = false;  // cannot do without (the split gradient's halves)
+};
+
+static int clamp_K(const fwime_ctx *x, int K) { return std::max(std::min(K, x->g.nt - 1), 1); }
+
+// Default segment length
+static int seg_K(const fwime_ctx *x)
 {
-    w.K = x->opt_K > 0 ? x->opt_K : x->opt_tlag > 0 ? auto_K(x->g.nt) : seg_len(x->g.nt, x->nshot);
-    // time lags: segments of at least 4 Hs steps keep the lag halo (2 Hs samples per segment, read once per
-    // residue class) at half the segment's own K samples or less
-    if (x->opt_tlag > 0 && x->opt_K == 0) w.K = std::max(w.K, 4 * tlag_Hs(x->g, x->opt_tlag));
-    w.K = std::min(w.K, x->g.nt - 1);
-    w.K = std::max(w.K, 1);
-    w.nseg = (x->g.nt - 1 + w.K - 1) / w.K;
-    w.R = w.K + 2;
-    Sizes sz = op_sizes(x->g, x->nshot, x->nrec, x->P, x->NZ, x->NXP, op, w.K, x->opt_host_io != 0, no_ckpt,
-                        x->opt_tlag);
-    size_t budget = x->max_ws;
+    return clamp_K(x, x->opt_K > 0 ? x->opt_K : x->opt_tlag > 0 ? auto_K(x->g.nt) : seg_len(x->g.nt, x->nshot));
+}
+
+// Bytes that `op` takes at least at segment length K without time lags, of one shot or of the caller's batch
+static size_t least_bytes(const fwime_ctx *x, int op, int K, bool no_ckpt)
+{
+    const Sizes s = op_sizes(x->g, x->nshot, x->nrec, x->P, x->NZ, x->NXP, op, K, x->opt_host_io != 0, no_ckpt);
+    const int S = x->opt_S > 0 && !x->opt_plain ? std::min(x->opt_S, x->nshot) : 1;
+    return (s.model + s.staging + s.per_shot * S) * sizeof(float) + 4096;
+}
+
+// The segment length without time lags: the default one, or sqrt(nt) where that is shorter and the default does not fit
+static int fit_K(const fwime_ctx *x, int op, bool no_ckpt, size_t budget)
+{
+    const int K = seg_K(x), least = clamp_K(x, auto_K(x->g.nt));
+    return x->opt_K == 0 && K > least && least_bytes(x, op, K, no_ckpt) > budget ? least : K;
+}
+
+// Bytes that the workspace may take
+static int plan_budget(fwime_ctx *x, size_t &budget)
+{
+    budget = x->max_ws;
     if (budget == 0 && x->capturing) budget = x->ws_bytes;   // the workspace was planned before capture
     if (budget == 0) {
         size_t fr = 0, tot = 0;
@@ -404,18 +425,29 @@ static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
         budget = x->ws_bytes + fr;
         budget = budget > ((size_t)2 << 30) ? budget - ((size_t)2 << 30) : budget / 2;   // keep 2 GB slack
     }
-    // a default segment longer than sqrt(nt) that does not fit falls back to that (not where stored states tie it)
-    const int S_least = x->opt_S > 0 && !x->opt_plain ? std::min(x->opt_S, x->nshot) : 1;
-    if (x->opt_tlag == 0 && x->opt_K == 0 && !no_ckpt && w.K > auto_K(x->g.nt) &&
-        (sz.model + sz.staging + sz.per_shot * S_least) * sizeof(float) + 4096 > budget) {
-        w.K = std::max(std::min(auto_K(x->g.nt), x->g.nt - 1), 1);
-        w.nseg = (x->g.nt - 1 + w.K - 1) / w.K;
-        w.R = w.K + 2;
-        sz = op_sizes(x->g, x->nshot, x->nrec, x->P, x->NZ, x->NXP, op, w.K, x->opt_host_io != 0, no_ckpt, 0);
-    }
+    return FWIME_OK;
+}
+
+// u.read: the source side's states or history are kept outside the workspace.  States whose segments do not fit are
+// given up (u is changed): the call then runs on its own.
+static int plan(fwime_ctx *x, int op, WS &w, Reuse &u)
+{
+    size_t budget = 0;
+    TRY(plan_budget(x, budget));
+    if (u.K > 0 && !u.must && least_bytes(x, op, u.K, u.read) > budget) u = Reuse{};
+    const bool no_ckpt = u.read;
+    w.K = u.K > 0 ? u.K : x->opt_tlag > 0 ? seg_K(x) : fit_K(x, op, no_ckpt, budget);
+    // time lags: segments of at least 4 Hs steps keep the lag halo (2 Hs samples per segment, read once per
+    // residue class) at half the segment's own K samples or less
+    if (x->opt_tlag > 0 && x->opt_K == 0 && u.K == 0) w.K = std::max(w.K, 4 * tlag_Hs(x->g, x->opt_tlag));
+    w.K = clamp_K(x, w.K);
+    w.nseg = (x->g.nt - 1 + w.K - 1) / w.K;
+    w.R = w.K + 2;
+    Sizes sz = op_sizes(x->g, x->nshot, x->nrec, x->P, x->NZ, x->NXP, op, w.K, x->opt_host_io != 0, no_ckpt,
+                        x->opt_tlag);
     // a default time-lag segment of 4 Hs that does not fit one shot falls back to 2 Hs (the halo then
     // equals the segment's own samples; the kernels stay correct for any K)
-    if (x->opt_tlag > 0 && x->opt_K == 0 && w.K > 2 * tlag_Hs(x->g, x->opt_tlag) &&
+    if (x->opt_tlag > 0 && x->opt_K == 0 && u.K == 0 && w.K > 2 * tlag_Hs(x->g, x->opt_tlag) &&
         (sz.model + sz.staging + sz.per_shot) * sizeof(float) > budget) {
         w.K = std::max(std::min(std::max(auto_K(x->g.nt), 2 * tlag_Hs(x->g, x->opt_tlag)), x->g.nt - 1), 1);
         w.nseg = (x->g.nt - 1 + w.K - 1) / w.K;
@@ -579,6 +611,12 @@ static int plan(fwime_ctx *x, int op, WS &w, bool no_ckpt = false)
         w.pred = take((size_t)w.S * x->g.nt * x->nrec);
     if ((char *)p > x->ws + x->ws_bytes) return fail(x, FWIME_ENOMEM, "workspace layout overflow");
     return FWIME_OK;
+}
+
+static int plan(fwime_ctx *x, int op, WS &w)
+{
+    Reuse u;
+    return plan(x, op, w, u);
 }
 
 // --------------------------------------------------------------- launches
@@ -845,28 +883,36 @@ static int prep_model(fwime_ctx *x, Run &r, const float *v)
 // states instead of running their own checkpointing sweep (one propagation fewer per call; the states are
 // those the sweep would compute).
 
-static int seg_K(const fwime_ctx *x)
-{
-    int K = x->opt_K > 0 ? x->opt_K : x->opt_tlag > 0 ? auto_K(x->g.nt) : seg_len(x->g.nt, x->nshot);
-    return std::max(std::min(K, x->g.nt - 1), 1);
-}
-
 static size_t bg_bytes(const fwime_ctx *x, int K, bool hist)
 {
     const size_t planes = hist ? (size_t)x->g.nt - 1 : 2 * (size_t)((x->g.nt - 1 + K - 1) / K);
     return planes * (size_t)x->nshot * (size_t)x->P * sizeof(float);
 }
 
-// Makes room for the cache; false when it does not fit (the call then runs without it).  The D2t of every step
-// (one propagation fewer than the states: nothing is recomputed) where it fits hist_cap and the segment length is
-// not the caller's, else the states; what a context holds it keeps.
-static bool bg_reserve(fwime_ctx *x, int K)
+// Makes room for the cache before a B or B~ (`op`); false when it does not fit (the call then runs without it).  The
+// D2t of every step (one propagation fewer than the states: nothing is recomputed) where it fits hist_cap and the
+// segment length is not the caller's, else the states, of segments that fit this call and either adjoint after it (K;
+// 0: the history has none, and with time lags B plans its own); what a context holds it keeps.
+static bool bg_reserve(fwime_ctx *x, int op, int &K)
 {
     const bool may_hist = x->opt_K == 0 && !x->opt_plain;
-    const size_t hneed = bg_bytes(x, K, true), need_st = bg_bytes(x, K, false);
-    if (x->bg.buf && (x->capturing || !x->bg.hist || may_hist) && x->bg.bytes >= (x->bg.hist ? hneed : need_st))
-        return true;
-    if (x->capturing) return false;
+    const size_t hneed = bg_bytes(x, 1, true);
+    K = 0;
+    if (x->bg.buf && x->bg.hist && may_hist && x->bg.bytes >= hneed) return true;
+    int Ks = seg_K(x);
+    if (x->opt_tlag == 0) {
+        size_t budget = 0;
+        if (plan_budget(x, budget) != FWIME_OK) return false;
+        if (x->max_ws == 0) {   // (beside the states)
+            const size_t st = bg_bytes(x, Ks, false), held = x->bg.buf ? x->bg.bytes : 0;
+            budget = budget + held > st ? budget + held - st : 0;
+        }
+        for (const int o : {op, (int)FWIME_OP_BORN_ADJ, (int)FWIME_OP_BORN_EXT_ADJ})
+            Ks = std::min(Ks, fit_K(x, o, o != op, budget));
+        K = Ks;
+    }
+    const size_t need_st = bg_bytes(x, Ks, false);
+    if (x->bg.buf && !x->bg.hist && x->bg.bytes >= need_st) return true;
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
         cudaGetLastError();
@@ -888,6 +934,7 @@ static bool bg_reserve(fwime_ctx *x, int K)
     }
     x->bg.bytes = need;
     x->bg.hist = hist;
+    if (hist) K = 0;
     return true;
 }
 
@@ -1636,54 +1683,54 @@ static bool bg_applies(const fwime_ctx *x, int op) { return !(x->opt_tlag > 0 &&
 static bool bg_usable(const fwime_ctx *x, const Call &c)
 {
     return is_bg_reader(c.op) && bg_applies(x, c.op) && x->opt_reuse_bg && x->bg.valid && x->bg.v == c.v &&
-           x->bg.w == c.w && x->bg.K == seg_K(x) && x->bg.buf;
+           x->bg.w == c.w && x->bg.seg == seg_K(x) && x->bg.buf;
 }
 
 // host-side bookkeeping once a call has been enqueued (directly or as a graph replay)
-static void bg_after(fwime_ctx *x, const Call &c, bool wrote)
+static void bg_after(fwime_ctx *x, const Call &c, const Reuse &u)
 {
     if (is_bg_writer(c.op)) {
-        x->bg.valid = wrote && bg_applies(x, c.op);
-        x->bg.v = c.v; x->bg.w = c.w; x->bg.K = seg_K(x);
+        x->bg.valid = u.write && bg_applies(x, c.op);
+        x->bg.v = c.v; x->bg.w = c.w; x->bg.K = u.K; x->bg.seg = seg_K(x);
     } else if (!is_bg_reader(c.op)) {
         x->bg.valid = false;
     }
 }
 
-// What a call does with the background cache: decided once, before it is planned, enqueued or captured.
-struct Reuse {
-    bool read = false, write = false;
-};
-
 static Reuse reuse_of(fwime_ctx *x, const Call &c)
 {
     Reuse u;
     u.read = bg_usable(x, c);
-    u.write = is_bg_writer(c.op) && bg_applies(x, c.op) && x->opt_reuse_bg && bg_reserve(x, seg_K(x));
+    if (u.read && !x->bg.hist) u.K = x->bg.K;
+    if (is_bg_writer(c.op) && bg_applies(x, c.op) && x->opt_reuse_bg) u.write = bg_reserve(x, c.op, u.K);
+    if (!u.read && !u.write) u.K = 0;
     return u;
 }
 
 static int plan_call(fwime_ctx *x, const Call &c, Reuse &u, WS &w)
 {
-    TRY(plan(x, c.op, w, u.read));
-    if (u.write && !x->bg.hist && w.K < seg_K(x)) u.write = false;   // shorter segments than the cache's
+    TRY(plan(x, c.op, w, u));
+    if (u.write && !x->bg.hist) u.K = w.K;
     return FWIME_OK;
 }
 
 static int enqueue(fwime_ctx *x, const Call &c, Reuse &u)
 {
     Run r;
-    x->bg_used = u.read;
-    x->bg_written = u.write;
+    x->bg_used = x->bg_written = false;
     if (c.op == OP_GRAD_FWD || c.op == OP_GRAD_BWD) {
         // the split gradient: checkpoints and residual live in the context's gradient state
-        TRY(plan(x, c.op == OP_GRAD_FWD ? FWIME_OP_OBJECTIVE : FWIME_OP_GRADIENT, r.w, true));
+        Reuse gs;
+        gs.read = gs.must = true;
+        gs.K = seg_K(x);
+        TRY(plan(x, c.op == OP_GRAD_FWD ? FWIME_OP_OBJECTIVE : FWIME_OP_GRADIENT, r.w, gs));
         init_run(x, r, r.w.S);
         TRY(prep_model(x, r, c.v));
         return run_tomo_adj(x, r, 1, c.v, c.w, c.in1, c.in2, c.out, c.accumulate, c.eps,
                             c.op == OP_GRAD_FWD ? PH_FORWARD : PH_BACKWARD);
     }
     TRY(plan_call(x, c, u, r.w));
+    x->bg_used = u.read;
     x->bg_written = u.write;
     if (u.write) x->bg.valid = false;   // being overwritten
     init_run(x, r, r.w.S);
@@ -1719,7 +1766,7 @@ static int enqueue_noted(fwime_ctx *x, const Call &c)
 {
     Reuse u = reuse_of(x, c);
     const int rc = enqueue(x, c, u);
-    if (rc == FWIME_OK) bg_after(x, c, u.write);
+    if (rc == FWIME_OK) bg_after(x, c, u);
     return rc;
 }
 
@@ -1740,7 +1787,7 @@ static int run_call(fwime_ctx *x, const Call &c)
     snprintf(key, sizeof(key), "%d|%p|%p|%p|%p|%p|%d|%a|%d|%d|%d|%d%d|%p|%d|%d", c.op, (const void *)c.v, (const void *)c.w,
              (const void *)c.in1, (const void *)c.in2, (void *)c.out, c.accumulate, (double)c.eps, x->opt_S, x->opt_K,
              x->opt_zchunk, u.read ? 1 : 0, u.write ? 1 : 0, (const void *)(cached ? x->bg.buf : nullptr),
-             !cached ? 0 : x->bg.hist ? -1 : w.K, x->opt_tlag * 2 + x->opt_fs);
+             !cached ? 0 : x->bg.hist ? -1 : u.K, x->opt_tlag * 2 + x->opt_fs);
     auto it = x->graphs.find(key);
     if (it == x->graphs.end()) {
         CK(cudaStreamBeginCapture(x->st, cudaStreamCaptureModeThreadLocal));
@@ -1765,7 +1812,7 @@ static int run_call(fwime_ctx *x, const Call &c)
     x->launches = it->second.launches;
     CK(cudaGraphLaunch(it->second.exec, x->st));
     x->bg_used = u.read;
-    bg_after(x, c, u.write);
+    bg_after(x, c, u);
     return FWIME_OK;
 }
 
@@ -1785,10 +1832,14 @@ static int call_op(fwime_ctx *x, Call c, int kin1, int kin2, int kout)
         s.w = reinterpret_cast<const float *>(x->ws) + al((size_t)x->g.nz * x->g.nx);
         return s;
     };
-    bool use_bg = x->ws && bg_usable(x, staged(c));
+    Reuse u;
+    if (x->ws) u = reuse_of(x, staged(c));
     WS w;
-    TRY(plan(x, c.op, w, use_bg));
-    if (use_bg && !bg_usable(x, staged(c))) TRY(plan(x, c.op, w, false));   // the arena moved
+    TRY(plan_call(x, c, u, w));
+    if (u.read && !bg_usable(x, staged(c))) {   // the arena moved
+        u = Reuse{};
+        TRY(plan(x, c.op, w));
+    }
     const size_t nm = (size_t)x->g.nz * x->g.nx, nd = (size_t)x->nshot * x->g.nt * x->nrec;
     auto count = [&](int k) -> size_t {
         return k == K_DATA ? nd : (k == K_MODEL ? nm : (k == K_EXT ? (size_t)x->g.nh * nm : 0));

@@ -49,7 +49,8 @@ def close(a, b, tol):
 # 399 steps, 41 offsets: a segment of 64 steps takes B~ 175 fields and B* 135, one of 20 steps 87 and 47 (and states)
 @pytest.mark.parametrize("graph", [0, 1])
 @pytest.mark.parametrize("planes", [100, 150, 190])
-@pytest.mark.parametrize("writer,reader", [("born_ext", "born_adj")])
+@pytest.mark.parametrize("writer", ["born_ext", "born"])
+@pytest.mark.parametrize("reader", ["born_adj", "born_ext_adj"])
 def test_adjoint_after_a_writer_under_a_cap(graph, planes, writer, reader):
     grid, geom, t, ref = problem(400, 41)
     stream = torch.cuda.Stream()
@@ -62,3 +63,22 @@ def test_adjoint_after_a_writer_under_a_cap(graph, planes, writer, reader):
         for _ in range(2):                    # the second time replays the graphs
             write(ctx, writer, t)
             close(adjoint(ctx, reader, t), own, 2e-6)
+            assert ctx.get_option("background_reused") == 1
+
+
+# 130 steps: the history is 130 fields; a segment of 64 steps takes B~ and B~* 175, one of 11 steps 69
+@pytest.mark.parametrize("graph", [0, 1])
+@pytest.mark.parametrize("planes", [100, 135, 150, 230])
+def test_adjoint_after_a_kept_history_under_a_cap(graph, planes):
+    grid, geom, t, ref = problem(131, 41)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with fw.Context(grid, geom, stream=stream, max_workspace_bytes=planes * PLANE, graph=graph,
+                    reuse_background=1) as ctx:
+        for _ in range(2):
+            write(ctx, "born_ext", t)
+            close(adjoint(ctx, "born_ext_adj", t), ref["born_ext_adj"], 1e-4)
+            assert ctx.get_option("background_reused") == 1
+            ctx.forward(t["v"], t["w"], torch.zeros_like(t["d"]))    # drops what was kept
+            adjoint(ctx, "born_adj", t)
+            assert ctx.get_option("background_reused") == 0
