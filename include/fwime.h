@@ -136,7 +136,9 @@ enum {
 };
 
 /* Creates a context on the current CUDA device.  `max_workspace_bytes` caps the
- * device memory the context may hold (0 = no cap); `cuda_stream` is a
+ * operators' workspace, kept histories included (0 = no cap); the segment-start
+ * states that FWIME_OPT_REUSE_BACKGROUND or fwime_gradient_forward keep come on
+ * top; `cuda_stream` is a
  * cudaStream_t (NULL = legacy default stream).  Returns FWIME_EINVAL for an
  * invalid grid/geometry (receivers or sources outside the physical grid, nh
  * even, nt < 2, non-positive spacing). */

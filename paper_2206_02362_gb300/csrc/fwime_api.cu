@@ -414,10 +414,19 @@ static int fit_K(const fwime_ctx *x, int op, bool no_ckpt, size_t budget)
     return x->opt_K == 0 && K > least && least_bytes(x, op, K, no_ckpt) > budget ? least : K;
 }
 
-// Bytes that the workspace may take
+// Bytes that `op` takes with all shots (or the caller's batch) advanced together, without histories
+static size_t batch_bytes(const fwime_ctx *x, int op, int K, bool no_ckpt)
+{
+    const Sizes s = op_sizes(x->g, x->nshot, x->nrec, x->P, x->NZ, x->NXP, op, K, x->opt_host_io != 0, no_ckpt);
+    const int S = x->opt_plain ? 1 : x->opt_S > 0 ? std::min(x->opt_S, x->nshot) : x->nshot;
+    return (s.model + s.staging + s.per_shot * S) * sizeof(float) + 4096;
+}
+
+// Bytes that the workspace may take: with a cap, what a kept background history leaves of it
 static int plan_budget(fwime_ctx *x, size_t &budget)
 {
     budget = x->max_ws;
+    if (budget != 0 && x->bg.buf && x->bg.hist) budget -= std::min(budget - 1, x->bg.bytes);
     if (budget == 0 && x->capturing) budget = x->ws_bytes;   // the workspace was planned before capture
     if (budget == 0) {
         size_t fr = 0, tot = 0;
@@ -509,8 +518,8 @@ static int plan(fwime_ctx *x, int op, WS &w, Reuse &u)
     w.S = std::max(S, 1);
     x->last_S = w.S;
     size_t need = fixed + per * (size_t)w.S + 4096;
-    if (x->max_ws && need > x->max_ws)
-        return fail(x, FWIME_ENOMEM, "operator needs %zu bytes for S=%d, K=%d; budget %zu", need, w.S, w.K, x->max_ws);
+    if (x->max_ws && need > budget)
+        return fail(x, FWIME_ENOMEM, "operator needs %zu bytes for S=%d, K=%d; budget %zu", need, w.S, w.K, budget);
     const size_t alt_bytes = 2 * al((size_t)w.S * x->P) * sizeof(float);
     const bool alt = op != FWIME_OP_BORN && !x->opt_plain && !x->opt_fs && pair_pays(x->P, w.S) &&
                      need + alt_bytes <= budget;
@@ -922,7 +931,11 @@ static bool bg_reserve(fwime_ctx *x, int op, int &K)
     const auto fits = [&](size_t n) {
         return !(x->max_ws && x->ws_bytes + n > x->max_ws) && n + ((size_t)4 << 30) <= fr + x->bg.bytes;
     };
-    const bool hist = may_hist && hneed <= hist_cap(x, tot) && fits(hneed);
+    // (a cap holds the history and the workspaces of the pair, at no fewer shots per batch for it)
+    const int adj = op == FWIME_OP_BORN ? FWIME_OP_BORN_ADJ : FWIME_OP_BORN_EXT_ADJ;
+    const int Kp = x->opt_tlag > 0 && x->opt_K == 0 ? clamp_K(x, std::max(Ks, 4 * tlag_Hs(x->g, x->opt_tlag))) : Ks;
+    const size_t pair = std::max(batch_bytes(x, op, Kp, false), batch_bytes(x, adj, Kp, true));
+    const bool hist = may_hist && hneed <= hist_cap(x, tot) && fits(hneed) && !(x->max_ws && hneed + pair > x->max_ws);
     const size_t need = hist ? hneed : need_st;
     if (!fits(need)) return false;
     if (x->bg.buf) cudaFreeAsync(x->bg.buf, x->st);
@@ -936,6 +949,15 @@ static bool bg_reserve(fwime_ctx *x, int op, int &K)
     x->bg.hist = hist;
     if (hist) K = 0;
     return true;
+}
+
+// With a cap, a kept history that the next call does not use goes before that call is planned, so that the cap is the
+// workspace's again.
+static void bg_yield(fwime_ctx *x)
+{
+    if (x->max_ws == 0 || !x->bg.buf || !x->bg.hist || x->capturing) return;
+    cudaFreeAsync(x->bg.buf, x->st);
+    x->bg = fwime_ctx::BgCache{};
 }
 
 // cache slot of state t (0: q^n0, 1: q^n0-1) of segment j for the batch starting at shot s0
@@ -1703,7 +1725,14 @@ static Reuse reuse_of(fwime_ctx *x, const Call &c)
     u.read = bg_usable(x, c);
     if (u.read && !x->bg.hist) u.K = x->bg.K;
     if (is_bg_writer(c.op) && bg_applies(x, c.op) && x->opt_reuse_bg) u.write = bg_reserve(x, c.op, u.K);
-    if (!u.read && !u.write) u.K = 0;
+    if (!u.read && !u.write) {
+        u.K = 0;
+        bg_yield(x);
+    } else if (u.read && x->bg.hist && x->max_ws &&
+               x->bg.bytes + least_bytes(x, c.op, fit_K(x, c.op, true, 1), true) > x->max_ws) {
+        bg_yield(x);   // (an adjoint of another kind than the history was kept for)
+        u = Reuse{};
+    }
     return u;
 }
 
@@ -2129,6 +2158,7 @@ int fwime_gradient_forward(fwime_ctx *x, const float *v, const float *w, const f
     x->launches = 0;
     x->user_J = objective;
     x->gs.valid = false;
+    bg_yield(x);
     const int K = seg_K(x);
     if (x->opt_tlag > 0 || x->opt_plain || !gs_reserve(x, K)) {
         // no room for the state (or a schedule that places its checkpoints otherwise): the objective alone;
@@ -2340,6 +2370,7 @@ int fwime_forward_group(fwime_ctx *const *ctxs, int n, const float *const *v, co
     std::vector<Run> runs(n);
     for (int i = 0; i < n; ++i) {
         fwime_ctx *m = ctxs[i];
+        bg_yield(m);
         TRY(plan(m, FWIME_OP_FORWARD, runs[i].w));
         if (runs[i].w.S < m->nshot)
             return fail(x, FWIME_ENOMEM, "group member %d: %d shots do not fit one batch", i, m->nshot);
@@ -2485,6 +2516,7 @@ int fwime_autotune(fwime_ctx *x, int op, int *zchunk_out, float *us_per_launch_o
     NOT_SERVER(x);
     if (x->capturing) return FWIME_EBUSY;
     Run r;
+    bg_yield(x);
     TRY(plan(x, op, r.w));
     const int S = r.w.S;
     // timing needs no model: zero c, the sponge tables and two batch fields
@@ -2523,6 +2555,7 @@ int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
     const bool lag = x->opt_tlag > 0;   // the time-lag schedules: extension kernels not timed here
     const int saved_K = x->opt_K, saved_S = x->opt_S, saved_zc = x->opt_zchunk, saved_prof = x->opt_profile;
     x->opt_profile = 0;
+    bg_yield(x);
     std::vector<int> Ks;
     if (saved_K > 0) Ks = {saved_K};
     else {

@@ -82,3 +82,39 @@ def test_adjoint_after_a_kept_history_under_a_cap(graph, planes):
             ctx.forward(t["v"], t["w"], torch.zeros_like(t["d"]))    # drops what was kept
             adjoint(ctx, "born_adj", t)
             assert ctx.get_option("background_reused") == 0
+
+
+@pytest.mark.parametrize("planes", [500, 600])
+def test_the_cap_holds_a_kept_history_and_the_workspace(planes):
+    """A history of 399 fields beside 139 fields of workspace: only the larger cap holds both (measured as the device's
+    free memory; 64 MB, 15 fields, are left for the allocator's rounding)."""
+    nz, nx, sponge, nt, nh = 996, 1012, 2, 400, 5
+    field = 4 * (nz + 12) * (nx + 12)
+    grid = fw.Grid(nz=nz, nx=nx, sponge=sponge, nt=nt, dt=DT, dx=DX, nh=nh)
+    geom = fw.Geometry(np.array([1]), np.array([500]), np.full(30, 1), 455 + 3 * np.arange(30))
+    gen = torch.Generator(device="cuda").manual_seed(synth.SEED0)
+    v = torch.full((nz, nx), 2000.0, device="cuda")
+    w = torch.from_numpy(synth.ricker(nt, DT, 22.0)[None].astype(np.float32)).cuda()
+    pt = torch.randn((nh, nz, nx), generator=gen, device="cuda")
+    d = torch.randn((1, nt, 30), generator=gen, device="cuda")
+    dout, img, own = torch.zeros_like(d), torch.zeros_like(pt), torch.zeros_like(pt)
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    with fw.Context(grid, geom, segment=20) as ctx:      # (also loads the kernels)
+        ctx.born_ext(v, w, pt, dout)
+        ctx.born_ext_adj(v, w, d, own)
+        ctx.forward(v, w, dout)
+    before = free()
+    with fw.Context(grid, geom, max_workspace_bytes=planes * field, reuse_background=1) as ctx:
+        for _ in range(2):
+            ctx.born_ext(v, w, pt, dout)
+            ctx.born_ext_adj(v, w, d, img)
+            assert ctx.get_option("background_reused") == 1
+            assert before - free() <= planes * field + (64 << 20)
+            diff = torch.linalg.vector_norm((img - own).double()) / torch.linalg.vector_norm(own.double())
+            assert float(diff) <= 2e-6
+            ctx.gradient(v, w, pt, d, torch.zeros_like(v))
+            assert before - free() <= planes * field + (64 << 20)
