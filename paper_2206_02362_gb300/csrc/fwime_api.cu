@@ -82,7 +82,7 @@ struct fwime_ctx {
         size_t bytes = 0;
         bool valid = false;
         const float *v = nullptr, *w = nullptr, *pt = nullptr;
-        int K = 0;
+        int K = 0, seg = 0;             // segment length of the states; the default one (seg_K) when they were written
     } gs;
     bool bg_used = false;           // the last call started from the cache
     long long launches = 0;
@@ -1751,7 +1751,7 @@ static int enqueue(fwime_ctx *x, const Call &c, Reuse &u)
         // the split gradient: checkpoints and residual live in the context's gradient state
         Reuse gs;
         gs.read = gs.must = true;
-        gs.K = seg_K(x);
+        gs.K = x->gs.K;
         TRY(plan(x, c.op == OP_GRAD_FWD ? FWIME_OP_OBJECTIVE : FWIME_OP_GRADIENT, r.w, gs));
         init_run(x, r, r.w.S);
         TRY(prep_model(x, r, c.v));
@@ -2159,8 +2159,14 @@ int fwime_gradient_forward(fwime_ctx *x, const float *v, const float *w, const f
     x->user_J = objective;
     x->gs.valid = false;
     bg_yield(x);
-    const int K = seg_K(x);
-    if (x->opt_tlag > 0 || x->opt_plain || !gs_reserve(x, K)) {
+    // the default segment length, or sqrt(nt) where only that leaves room
+    int K = seg_K(x);
+    bool room = x->opt_tlag == 0 && !x->opt_plain && gs_reserve(x, K);
+    if (!room && x->opt_tlag == 0 && !x->opt_plain && x->opt_K == 0 && K > clamp_K(x, auto_K(x->g.nt))) {
+        K = clamp_K(x, auto_K(x->g.nt));
+        room = gs_reserve(x, K);
+    }
+    if (!room) {
         // no room for the state (or a schedule that places its checkpoints otherwise): the objective alone;
         // the adjoint half then runs the whole gradient
         gs_release(x);
@@ -2168,6 +2174,8 @@ int fwime_gradient_forward(fwime_ctx *x, const float *v, const float *w, const f
         if (rc != FWIME_OK) x->user_J = nullptr;
         return rc;
     }
+    x->gs.K = K;
+    x->gs.seg = seg_K(x);
     const int rc = enqueue_noted(x, Call{OP_GRAD_FWD, v, w, pt, dobs, nullptr, 0, eps});
     if (rc != FWIME_OK) {
         x->user_J = nullptr;
@@ -2175,7 +2183,7 @@ int fwime_gradient_forward(fwime_ctx *x, const float *v, const float *w, const f
         return rc;
     }
     x->gs.valid = true;
-    x->gs.v = v; x->gs.w = w; x->gs.pt = pt; x->gs.K = K;
+    x->gs.v = v; x->gs.w = w; x->gs.pt = pt;
     return FWIME_OK;
 }
 
@@ -2189,7 +2197,7 @@ int fwime_gradient_backward(fwime_ctx *x, const float *v, const float *w, const 
     if (x->opt_host_io || x->capturing) return fail(x, FWIME_EINVAL, "the split gradient takes device pointers, no capture");
     x->launches = 0;
     const bool from_state = x->gs.valid && x->gs.buf && x->gs.v == v && x->gs.w == w && x->gs.pt == pt &&
-                            x->gs.K == seg_K(x) && x->opt_tlag == 0 && !x->opt_plain;
+                            x->gs.seg == seg_K(x) && x->opt_tlag == 0 && !x->opt_plain;
     int rc;
     if (from_state) {
         rc = enqueue_noted(x, Call{OP_GRAD_BWD, v, w, pt, dobs, grad, accumulate ? 1 : 0, eps});
