@@ -289,8 +289,8 @@ int fwime_autotune(fwime_ctx *ctx, int op, int *zchunk, float *us_per_launch);
  * Layouts as for fwime_forward (v, w, d) and fwime_gradient (pt, dobs, grad).
  *
  * Errors: fwime_submit returns FWIME_EINVAL for a bad request (unknown kind, grid, geometry, missing
- * buffer) and FWIME_ENOMEM when the request alone needs more than the budget (it could never be
- * admitted); a message is then available from fwime_server_last_error (per calling thread).  A request
+ * buffer) and FWIME_ENOMEM when the request alone needs more than the budget, in shorter segments too
+ * (fwime_request_least_bytes: it could never be admitted); a message is then available from fwime_server_last_error (per calling thread).  A request
  * that fails on the GPU side is collected with its error code in fwime_result.status.  fwime_sync on a
  * server context waits until every submitted request has finished; fwime_destroy waits for them too,
  * then stops the server's threads. */
@@ -324,6 +324,9 @@ typedef struct {
 int fwime_server_create(fwime_ctx **out, size_t memory_budget, int max_active, int options);
 /* Device bytes the server admits a request with (workspace + staging). */
 int fwime_request_bytes(const fwime_request *req, size_t *bytes);
+/* The same in the shortest default segments (sqrt(nt) steps), with which a request is admitted and run when
+ * fwime_request_bytes alone exceeds the budget. */
+int fwime_request_least_bytes(const fwime_request *req, size_t *bytes);
 int fwime_submit(fwime_ctx *server, const fwime_request *req, uint64_t *ticket);
 /* Non-blocking: res->done = 0 while the request runs; on 1 the result is collected and the ticket freed.
  * FWIME_EINVAL for an unknown (or already collected) ticket. */

@@ -43,7 +43,7 @@ ABI_FUNCTIONS = ("fwime_create", "fwime_workspace_bytes", "fwime_set_option", "f
                  "fwime_objective", "fwime_vp_solve", "fwime_spline", "fwime_spline_refine",
                  "fwime_autotune", "fwime_autotune_schedule", "fwime_forward_group", "fwime_sync", "fwime_profile_read",
                  "fwime_last_error_detail", "fwime_strerror", "fwime_destroy",
-                 "fwime_server_create", "fwime_request_bytes", "fwime_submit", "fwime_poll", "fwime_wait",
+                 "fwime_server_create", "fwime_request_bytes", "fwime_request_least_bytes", "fwime_submit", "fwime_poll", "fwime_wait",
                  "fwime_server_last_error")
 REQ_FORWARD, REQ_GRADIENT = 0, 1
 SERVE_PLAIN = 1
@@ -137,6 +137,7 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
     lib.fwime_destroy.restype = None
     lib.fwime_server_create.argtypes = [ctypes.POINTER(vp), ctypes.c_size_t, ip, ip]
     lib.fwime_request_bytes.argtypes = [ctypes.POINTER(RequestC), ctypes.POINTER(ctypes.c_size_t)]
+    lib.fwime_request_least_bytes.argtypes = [ctypes.POINTER(RequestC), ctypes.POINTER(ctypes.c_size_t)]
     lib.fwime_submit.argtypes = [vp, ctypes.POINTER(RequestC), ctypes.POINTER(ctypes.c_uint64)]
     lib.fwime_poll.argtypes = [vp, ctypes.c_uint64, ctypes.POINTER(ResultC)]
     lib.fwime_wait.argtypes = [vp, ctypes.c_uint64, ctypes.POINTER(ResultC)]

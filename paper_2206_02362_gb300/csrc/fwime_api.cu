@@ -391,6 +391,8 @@ struct Reuse {
     bool must = false;  // cannot do without (the split gradient's halves)
 };
 
+int fwk::least_segment(int nt) { return auto_K(nt); }
+
 static int clamp_K(const fwime_ctx *x, int K) { return std::max(std::min(K, x->g.nt - 1), 1); }
 
 // Default segment length

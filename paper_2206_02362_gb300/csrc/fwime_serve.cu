@@ -71,6 +71,18 @@ size_t stage_floats(const fwime_request &r)
     return f;
 }
 
+// Workspace of a request, all its shots in one batch, in segments of `segment` steps (0: the default), and the bytes it
+// takes with the context's own small block and the staging of host buffers
+int request_bytes(const fwime_request &r, int segment, size_t &ws, size_t &bytes)
+{
+    if (r.kind != FWIME_REQ_FORWARD && r.kind != FWIME_REQ_GRADIENT) return FWIME_EINVAL;
+    const int op = r.kind == FWIME_REQ_FORWARD ? FWIME_OP_FORWARD : FWIME_OP_GRADIENT;
+    const int rc = fwime_workspace_bytes(&r.grid, &r.geom, op, r.geom.nshot, segment, &ws);
+    if (rc != FWIME_OK) return rc;
+    bytes = ws + ((size_t)1 << 20) + stage_floats(r) * sizeof(float);
+    return FWIME_OK;
+}
+
 }  // namespace
 
 struct Server {
@@ -430,15 +442,14 @@ int fwime_server_create(fwime_ctx **out, size_t memory_budget, int max_active, i
 
 int fwime_request_bytes(const fwime_request *r, size_t *bytes)
 {
-    if (!r || !bytes) return FWIME_EINVAL;
-    if (r->kind != FWIME_REQ_FORWARD && r->kind != FWIME_REQ_GRADIENT) return FWIME_EINVAL;
-    const int op = r->kind == FWIME_REQ_FORWARD ? FWIME_OP_FORWARD : FWIME_OP_GRADIENT;
     size_t ws = 0;
-    const int rc = fwime_workspace_bytes(&r->grid, &r->geom, op, r->geom.nshot, 0, &ws);
-    if (rc != FWIME_OK) return rc;
-    // workspace + the context's own small block + staging of host buffers
-    *bytes = ws + ((size_t)1 << 20) + stage_floats(*r) * sizeof(float);
-    return FWIME_OK;
+    return r && bytes ? request_bytes(*r, 0, ws, *bytes) : FWIME_EINVAL;
+}
+
+int fwime_request_least_bytes(const fwime_request *r, size_t *bytes)
+{
+    size_t ws = 0;
+    return r && bytes ? request_bytes(*r, least_segment(r->grid.nt), ws, *bytes) : FWIME_EINVAL;
 }
 
 int fwime_submit(fwime_ctx *srv, const fwime_request *req, uint64_t *ticket)
@@ -446,8 +457,10 @@ int fwime_submit(fwime_ctx *srv, const fwime_request *req, uint64_t *ticket)
     Server *s = ctx_server(srv);
     if (!s || !req || !ticket) return FWIME_EINVAL;
     g_serr[0] = 0;
-    size_t need = 0;
-    int rc = fwime_request_bytes(req, &need);
+    size_t need = 0, ws = 0;
+    int rc = request_bytes(*req, 0, ws, need);
+    // beyond the budget at the default segment length: run in shorter segments (the context, capped at ws, plans them)
+    if (rc == FWIME_OK && need > s->budget) rc = request_bytes(*req, least_segment(req->grid.nt), ws, need);
     if (rc != FWIME_OK) return fail_srv(g_serr, sizeof(g_serr), rc, "fwime_submit: invalid kind, grid or geometry");
     const bool fwd = req->kind == FWIME_REQ_FORWARD;
     if (!req->v || !req->w || (fwd && !req->d) || (!fwd && (!req->pt || !req->dobs || !req->grad)) ||
@@ -467,8 +480,7 @@ int fwime_submit(fwime_ctx *srv, const fwime_request *req, uint64_t *ticket)
     j->req.geom.src_iz = j->siz.data(); j->req.geom.src_ix = j->six.data();
     j->req.geom.rec_iz = j->riz.data(); j->req.geom.rec_ix = j->rix.data();
     j->need = need;
-    fwime_workspace_bytes(&req->grid, &req->geom, fwd ? FWIME_OP_FORWARD : FWIME_OP_GRADIENT, req->geom.nshot, 0,
-                          &j->ws);
+    j->ws = ws;
     j->t_submit = Clock::now();
     std::lock_guard<std::mutex> lk(s->mu);
     if (s->stop) {

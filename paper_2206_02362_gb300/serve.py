@@ -90,8 +90,9 @@ class _Marshalled:
                              ctypes.c_float(req.eps))
 
 
-def request_bytes(req: ShotRequest) -> int:
-    """Device bytes the server admits a request with: workspace + staging (fwime_request_bytes)."""
+def request_bytes(req: ShotRequest, least: bool = False) -> int:
+    """Device bytes the server admits a request with: workspace + staging (fwime_request_bytes); with `least` those
+    that the shortest default segments take (fwime_request_least_bytes)."""
     import paper_2206_02362_gb300 as fw
     grid = fw.Grid(nz=req.nz, nx=req.nx, sponge=req.sponge, nt=req.nt, dt=req.dt, dx=req.dx, nh=req.nh)
     geom = fw.Geometry(np.array([req.src[0]]), np.array([req.src[1]]), req.rec_iz, req.rec_ix)
@@ -99,9 +100,10 @@ def request_bytes(req: ShotRequest) -> int:
     c = fw.RequestC(fw.REQ_FORWARD if req.kind == "forward" else fw.REQ_GRADIENT, grid.c(), gm, 1,
                     None, None, None, None, None, None, ctypes.c_float(req.eps))
     out = ctypes.c_size_t(0)
-    rc = fw.load().fwime_request_bytes(ctypes.byref(c), ctypes.byref(out))
+    name = "fwime_request_least_bytes" if least else "fwime_request_bytes"
+    rc = getattr(fw.load(), name)(ctypes.byref(c), ctypes.byref(out))
     if rc != fw.FWIME_OK:
-        raise fw.FwimeError(rc, "fwime_request_bytes")
+        raise fw.FwimeError(rc, name)
     return int(out.value)
 
 
@@ -158,7 +160,7 @@ class Server:
         """Submits each request at req.arrival seconds (realtime) or all at once, collects every result;
         returns the results in rid order."""
         for r in requests:
-            need = request_bytes(r)
+            need = request_bytes(r, least=True)
             if need > self.budget:
                 raise ValueError(f"request {r.rid} needs {need} bytes, over the budget {self.budget}")
         marsh = {r.rid: _Marshalled(r) for r in requests}
