@@ -25,6 +25,9 @@ namespace fwk {
 // the warp's index in its CTA, as a value that is known to be the same in all its lanes
 __device__ __forceinline__ int warp_in_cta() { return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0); }
 __device__ __forceinline__ float4 f4zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+// Read-only loads: of what no launch in flight writes (model, tables, receivers).  The wavefields are read by plain
+// loads through plain pointers: a launch comes in while the one before still writes them, and what is read as read-only
+// may be fetched before the wait, or from a cache that holds an older step's rows.
 __device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
 __device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ void st4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
@@ -282,7 +285,7 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, cons
     const bool xin = x < a.NXP;
     const int NXP = a.NXP;
     const long long so = (long long)shot * a.P, row0 = (long long)z0 * NXP;
-    const float *__restrict__ cur = a.cur + so + row0;
+    const float *cur = a.cur + so + row0;
     const float *prev = a.prev + so + row0, *c = a.c + row0;
     float *out0 = a.out + so + row0, *d20 = D2 ? a.d2 + so + row0 : nullptr;
 
@@ -334,7 +337,7 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, cons
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const float *qp = cur + (long long)(k - 4) * NXP + oX;
-        q[k] = xin ? ldg4(qp) : f4zero();
+        q[k] = xin ? ld4(qp) : f4zero();
     }
     // prologue: one group per row of look-ahead (rows z0 .. z0+3 feed the first x-taps)
     constexpr int DEPTH = LOCAL ? LRING : 4;

@@ -75,8 +75,7 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_MINB) k_prop_pair(const 
     const int dz = (chunk & 1) ? -1 : 1, NX = dz * NXP;
     const int y0 = dz > 0 ? z0 - 4 : z1 + 3, ye = dz > 0 ? z1 + 4 : z0 - 5;   // rows of the first step
     int oA = y0 * NXP + (nA ? cA : 0), oB = y0 * NXP + (nB ? cB : 0), oX = y0 * NXP + (nX ? x : 0);
-    const float *__restrict__ cur = a.cur + so;
-    const float *__restrict__ prev = a.prev + so;
+    const float *cur = a.cur + so, *prev = a.prev + so;
     const auto cp = [](float *dst, const float *src, int n) {
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
                      "l"(src), "r"(n)
@@ -109,7 +108,7 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_MINB) k_prop_pair(const 
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const int zr = y0 + (k - 4) * dz;
-        q[k] = xin && zr >= 0 && zr < a.NZ ? ldg4(cur + (k - 4) * NX + oX) : f4zero();
+        q[k] = xin && zr >= 0 && zr < a.NZ ? ld4(cur + (k - 4) * NX + oX) : f4zero();
         p[k] = f4zero();
     }
 #pragma unroll
