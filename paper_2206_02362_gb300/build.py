@@ -56,7 +56,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False, 
             BUILD, LIB = saved
     os.makedirs(BUILD, exist_ok=True)
     headers = [os.path.join(CSRC, "fwime_kernels.cuh"), os.path.join(CSRC, "fwime_internal.h"), os.path.join(CSRC, "fwime_ext.cuh"),
-               os.path.join(CSRC, "fwime_prop.cuh"),
+               os.path.join(CSRC, "fwime_prop.cuh"), os.path.join(CSRC, "fwime_device.h"),
                os.path.join(ROOT, "include", "fwime.h")]
     objs = []
     jobs = []

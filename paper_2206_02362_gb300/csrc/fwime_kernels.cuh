@@ -15,6 +15,8 @@
 
 #include <cmath>
 
+#include "fwime_device.h"
+
 namespace fwk {
 
 constexpr int STRIP = 128;      // x-points per warp in the stencil kernel (32 lanes x float4)

@@ -493,10 +493,11 @@ __global__ void __launch_bounds__(PROP_WARPS * 32, LOC == 2 ? FWIME_PROP_MIN_BLO
 template <bool FS, int LOC, bool D2, bool SRC, bool INJ = false>
 static void launch_prop_t(const PropArgs &a, dim3 grid, dim3 block, size_t smem, cudaStream_t st)
 {
-    // once per instantiation, thread-safe (function-local static)
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_prop<LOC, D2, SRC, INJ, FS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-    (void)attr;
+    // once per instantiation and device
+    static PerDevice<cudaError_t> attr;
+    (void)attr.get([] {
+        return cudaFuncSetAttribute(k_prop<LOC, D2, SRC, INJ, FS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+    });
     // The next step's CTAs come in as soon as this one's are all under way and wait there, so that a step starts
     // without the launch gap: 2 to 3 us per step (100 shots on 408 x 1816 points 170 / 167 us, 30 shots 61 / 59 us).
     cudaLaunchConfig_t cfg{};

@@ -248,10 +248,11 @@ template <class Sh, bool LOCAL>
 static void launch_band_t(const ImgArgs &a, int ha, int h_lo, int h_hi, cudaStream_t st)
 {
     constexpr size_t smem = Sh::template smem_chunks<LOCAL>() * 16;
-    // once per instantiation, before any launch (and any capture), thread-safe (function-local static)
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_image_band<Sh, LOCAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    (void)attr;
+    // once per instantiation and device
+    static PerDevice<cudaError_t> attr;
+    (void)attr.get([] {
+        return cudaFuncSetAttribute(k_image_band<Sh, LOCAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    });
     // u = x - h of the physical columns: lane s of the CTA at ub covers [ub + 2 LB (S-1-s), .. + UC)
     int u_lo = a.x_lo - ha - Sh::LB * (2 * Sh::S - 1) + 1;
     u_lo -= ((u_lo % 32) + 32) % 32;                            // whole 128-byte lines

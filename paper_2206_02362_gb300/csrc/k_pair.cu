@@ -207,16 +207,17 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_MINB) k_prop_pair(const 
 template <int LOC, bool D2, bool SRC, bool INJ>
 static cudaError_t launch_pair_t(const PairArgs &m, int nshot, cudaStream_t st)
 {
-    static const cudaError_t attr = cudaFuncSetAttribute(k_prop_pair<LOC, D2, SRC, INJ>,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-    if (attr != cudaSuccess) return attr;
     // Shared memory for the three CTAs that the registers allow, the rest to L1, whatever the launch before had: right
     // behind k_prop, which takes all of it, pairs took 54.3 ms where they take 51.1 (a launch that follows without a
     // gap keeps the split unless it asks for another).
     constexpr int cta = sizeof(float) * PAIR_WARPS * pair_smem(LOC) + 1024, carve = (3 * cta * 100 + 233471) / 233472 + 1;
-    static const cudaError_t attr2 = cudaFuncSetAttribute(k_prop_pair<LOC, D2, SRC, INJ>,
-                                                          cudaFuncAttributePreferredSharedMemoryCarveout, carve);
-    if (attr2 != cudaSuccess) return attr2;
+    static PerDevice<cudaError_t> attr;
+    const cudaError_t e = attr.get([] {
+        const auto k = k_prop_pair<LOC, D2, SRC, INJ>;
+        const cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+        return r != cudaSuccess ? r : cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
+    });
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((m.a.nstrip * m.a.nchunk + PAIR_WARPS - 1) / PAIR_WARPS, nshot);
     cfg.blockDim = dim3(PAIR_WARPS * 32);

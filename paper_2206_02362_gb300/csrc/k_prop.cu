@@ -57,9 +57,10 @@ cudaError_t launch_prop_group(const GroupMember *m, int nactive, int ctas, const
                               int step, cudaStream_t st, bool record)
 {
     const size_t smem = (size_t)PROP_WARPS * prop_smem(2) * sizeof(float);
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_prop_group, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (attr != cudaSuccess) return attr;
+    static PerDevice<cudaError_t> attr;
+    const cudaError_t e = attr.get(
+        [&] { return cudaFuncSetAttribute(k_prop_group, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
+    if (e != cudaSuccess) return e;
     if (!record) {
         k_prop_group<<<ctas, PROP_WARPS * 32, smem, st>>>(m, nactive, step);
     } else {

@@ -268,16 +268,16 @@ static int launch_band(const ExtArgs &a, int g_lo, int accumulate, cudaStream_t 
 {
     const int ga = g_lo - ((g_lo % Sh::GALIGN) + Sh::GALIGN) % Sh::GALIGN;
     const int g_hi = std::min(ga + Sh::C - 1, a.hm);
-    // once per instantiation, before any launch (and any capture), thread-safe (function-local static): the
-    // attribute, then the CTAs resident on the device
-    static const double wave = [] {
+    // once per instantiation and device: the attribute, then the CTAs resident on the device
+    static PerDevice<double> resident;
+    const double wave = resident.get([] {
         int r = 0, dev = 0, nsm = 0;
         cudaFuncSetAttribute(k_scatter_band<Sh>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::SMEM);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k_scatter_band<Sh>, Sh::TX, Sh::SMEM);
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         return (double)std::max(r, 1) * std::max(nsm, 1);
-    }();
+    });
     const int y_lo = a.x_lo - a.x_lo % 32;                      // whole 128-byte lines
     const int nx = (a.x_hi - y_lo + Sh::YC - 1) / Sh::YC, nz = a.z_hi - a.z_lo;
     // Every CTA streams its pairs for the whole launch, so a partly filled last wave idles SMs for long: the pairs
