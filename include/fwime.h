@@ -341,12 +341,14 @@ int fwime_server_last_error(char *buf, size_t n);
  * chunking as fwime_autotune does, times the operator's extension kernels once over a full segment of K x S
  * (step, shot) pairs with CUDA events, and models the time per shot as
  *   ((nt - 1) props t_stencil + nseg (scatters t_scatter + images t_image)) / S
- * with the operator's launches per step and per segment.  The fastest schedule is set as the context's
- * FWIME_OPT_SEGMENT, FWIME_OPT_SHOTS_PER_BATCH and FWIME_OPT_ZCHUNK and returned.  Synchronous; the
+ * with the operator's launches per step and per segment (t_stencil: a step's, as it runs: two steps share a
+ * launch for batches beyond the L2 cache).  The fastest schedule is set as the context's
+ * FWIME_OPT_SEGMENT, FWIME_OPT_SHOTS_PER_BATCH and FWIME_OPT_ZCHUNK and returned; unlike a segment set by
+ * the caller it keeps the histories that FWIME_OPT_SEGMENT = 0 keeps.  Synchronous; the
  * workspace contents are overwritten (no operator state survives it).  Not with the plain path. */
 typedef struct {
     int segment, shots_per_batch, zchunk;
-    float us_stencil, us_scatter, us_image;   /* per launch at the chosen schedule */
+    float us_stencil, us_scatter, us_image;   /* per step, per launch at the chosen schedule */
     double us_per_shot;                       /* modelled operator time per shot */
 } fwime_schedule;
 int fwime_autotune_schedule(fwime_ctx *ctx, int op, fwime_schedule *res);

@@ -62,6 +62,7 @@ struct fwime_ctx {
     size_t dev_mem = 0;             // total memory of the device
     // options
     int opt_S = 0, opt_K = 0, opt_plain = 0, opt_graph = 0, opt_host_io = 0, opt_zchunk = 0, opt_reuse_bg = 0;
+    bool tuned_K = false;           // opt_K is the schedule tuner's choice, not the caller's: histories may be kept
     int opt_tlag = 0;               // > 0: B~ / B~* extend with time lags spaced opt_tlag steps
     int opt_fs = 0;                 // 1: free surface at the top physical row
     // background wavefield kept by B and B~ for a B* or B~* on the same v, w (FWIME_OPT_REUSE_BACKGROUND): its D2t at
@@ -481,7 +482,7 @@ static int plan(fwime_ctx *x, int op, WS &w, Reuse &u)
                         op == FWIME_OP_GRADIENT;
     w.hist = false;
     int hist_S = 0;
-    if (adj_op && !no_ckpt && x->opt_K == 0 && x->opt_tlag == 0 && !x->opt_plain) {
+    if (adj_op && !no_ckpt && (x->opt_K == 0 || x->tuned_K) && x->opt_tlag == 0 && !x->opt_plain) {
         const size_t cap = hist_cap(x, budget);
         const Sizes sh = op_sizes(x->g, x->nshot, x->nrec, x->P, x->NZ, x->NXP, op, w.K, x->opt_host_io != 0, false, 0, true);
         const size_t hf = (sh.model + sh.staging) * sizeof(float) + 4096, hp = sh.per_shot * sizeof(float);
@@ -906,7 +907,7 @@ static size_t bg_bytes(const fwime_ctx *x, int K, bool hist)
 // 0: the history has none, and with time lags B plans its own); what a context holds it keeps.
 static bool bg_reserve(fwime_ctx *x, int op, int &K)
 {
-    const bool may_hist = x->opt_K == 0 && !x->opt_plain;
+    const bool may_hist = (x->opt_K == 0 || x->tuned_K) && !x->opt_plain;
     const size_t hneed = bg_bytes(x, 1, true);
     K = 0;
     if (x->bg.buf && x->bg.hist && may_hist && x->bg.bytes >= hneed) return true;
@@ -2031,7 +2032,11 @@ int fwime_set_option(fwime_ctx *x, int option, long long value)
     if (x->capturing) return FWIME_EBUSY;
     switch (option) {
     case FWIME_OPT_SHOTS_PER_BATCH: if (value < 0) break; x->opt_S = (int)value; return FWIME_OK;
-    case FWIME_OPT_SEGMENT: if (value < 0) break; x->opt_K = (int)value; return FWIME_OK;
+    case FWIME_OPT_SEGMENT:
+        if (value < 0) break;
+        x->opt_K = (int)value;
+        x->tuned_K = false;
+        return FWIME_OK;
     case FWIME_OPT_PLAIN: x->opt_plain = value != 0; return FWIME_OK;
     case FWIME_OPT_GRAPH: x->opt_graph = value != 0; return FWIME_OK;
     case FWIME_OPT_HOST_IO: x->opt_host_io = value != 0; return FWIME_OK;
@@ -2552,7 +2557,8 @@ int fwime_autotune(fwime_ctx *x, int op, int *zchunk_out, float *us_per_launch_o
 // S_K and half of it are tried.  At each (K, S) the stencil is timed for its chunking candidates and the
 // operator's extension kernels once over a full segment of K x S pairs; the modelled time per shot,
 //   (nt - 1) * props * t_stencil / S + nseg * (scatters * t_scatter + images * t_image) / S,
-// picks the schedule (props, scatters, images: the operator's launches per step and per segment).
+// picks the schedule (props, scatters, images: the operator's launches per step and per segment, fewer where the plan
+// keeps the source side's D2t; t_stencil: half a launch's time where a batch runs two steps per launch).
 int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
 {
     if (!x || !res || op < 0 || op > FWIME_OP_OBJECTIVE) return FWIME_EINVAL;
@@ -2560,15 +2566,19 @@ int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
     if (x->capturing) return FWIME_EBUSY;
     if (x->opt_plain) return fail(x, FWIME_EINVAL, "the plain path has a fixed schedule");
     static const int PROPS[] = {1, 2, 3, 2, 3, 4, 6, 6, 2};
-    static const int SCAT[] = {0, 0, 0, 1, 0, 3, 2, 2, 1};
+    static const int KEPT[] = {1, 2, 2, 2, 2, 4, 4, 4, 2};      // with kept histories
+    static const int PAIRED[] = {1, 0, 9, 2, 9, 2, 9, 9, 2};    // of these at most that many can run two steps per launch
+    static const int SCAT[] = {0, 0, 0, 1, 0, 3, 3, 3, 1};      // (T*, gradient: one fewer with kept histories)
     static const int IMGS[] = {0, 0, 0, 0, 1, 0, 1, 1, 0};
     const bool lag = x->opt_tlag > 0;   // the time-lag schedules: extension kernels not timed here
+    const bool saved_tuned = x->tuned_K;
     const int saved_K = x->opt_K, saved_S = x->opt_S, saved_zc = x->opt_zchunk, saved_prof = x->opt_profile;
     x->opt_profile = 0;
     bg_yield(x);
     std::vector<int> Ks;
     if (saved_K > 0) Ks = {saved_K};
     else {
+        x->tuned_K = true;
         const int K0 = std::max(std::min(auto_K(x->g.nt), x->g.nt - 1), 1);
         Ks = {K0, std::max(K0 / 2, 8), std::min(2 * K0, x->g.nt - 1)};
         std::sort(Ks.begin(), Ks.end());
@@ -2626,6 +2636,26 @@ int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
             x->opt_zchunk = zbest;
             init_run(x, r, S);
             const int kk = std::min(K, x->g.nt - 1);
+            const int props = r.w.hist ? KEPT[op] : PROPS[op];
+            int paired = 0;
+            float t2 = 0.f;                        // a step of a launch of two
+            if (r.w.alt[0] && kk >= 2 && !(lag && op == FWIME_OP_TOMO)) {
+                PairArgs m{};
+                m.a = prop_args(r, r.w.f[0], r.w.f[1], r.w.alt[0], nullptr, nullptr, 0, r.w.f[0], 1.f, nullptr, nullptr,
+                                RecTo{}, InjFrom{});
+                m.out2 = r.w.alt[1];
+                m.f0b = r.w.f[0];
+                if (pair_runs(m.a)) {
+                    rc = timed([&]() -> int {
+                        LAUNCH(FWIME_K_PROP, 0.0, launch_pair(m, S, x->st));
+                        return FWIME_OK;
+                    }, 4, t2);
+                    if (rc != FWIME_OK) break;
+                    t2 *= 0.5f;
+                    paired = std::min(PAIRED[op], props);
+                }
+            }
+            tp = ((props - paired) * tp + paired * t2) / props;
             float tsc = 0.f, tim = 0.f;
             if (!lag && SCAT[op] > 0 && r.w.W && r.w.ring[0] && r.w.ring[1]) {
                 rc = timed([&]() {
@@ -2644,7 +2674,8 @@ int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
                 if (rc != FWIME_OK) break;
             }
             const double nseg = (double)r.w.nseg;
-            const double per_shot = ((double)(x->g.nt - 1) * PROPS[op] * tp + nseg * (SCAT[op] * tsc + IMGS[op] * tim)) / S;
+            const int scat = SCAT[op] - (r.w.hist && SCAT[op] > 0 ? 1 : 0);
+            const double per_shot = ((double)(x->g.nt - 1) * props * tp + nseg * (scat * tsc + IMGS[op] * tim)) / S;
             if (per_shot < best) {
                 best = per_shot;
                 out.shots_per_batch = S;
@@ -2660,7 +2691,7 @@ int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
     }
     cleanup();
     if (rc != FWIME_OK || best >= 1e299) {
-        x->opt_K = saved_K; x->opt_S = saved_S; x->opt_zchunk = saved_zc;
+        x->opt_K = saved_K; x->opt_S = saved_S; x->opt_zchunk = saved_zc; x->tuned_K = saved_tuned;
         return rc != FWIME_OK ? rc : fail(x, FWIME_ENOMEM, "no schedule fits");
     }
     x->opt_K = out.segment;
