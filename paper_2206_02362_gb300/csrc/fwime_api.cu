@@ -109,7 +109,7 @@ struct fwime_ctx {
     bool capturing = false;
     // per-launch CUDA-event profiling (FWIME_OPT_PROFILE)
     int opt_profile = 0;
-    struct Pend { int ev; int kind; double bytes; };
+    struct Pend { int ev; int kind; double bytes; int n; };
     std::vector<cudaEvent_t> ev;
     std::vector<Pend> pend;
     double prof_ms[5] = {0, 0, 0, 0, 0}, prof_bytes[5] = {0, 0, 0, 0, 0};
@@ -220,11 +220,11 @@ static int prof_begin(fwime_ctx *x, int &slot)
     return FWIME_OK;
 }
 
-static int prof_end(fwime_ctx *x, int slot, int kind, double bytes)
+static int prof_end(fwime_ctx *x, int slot, int kind, double bytes, int n)
 {
     if (slot < 0) return FWIME_OK;
     CK(cudaEventRecord(x->ev[slot + 1], x->st));
-    x->pend.push_back({slot, kind, bytes});
+    x->pend.push_back({slot, kind, bytes, n});
     return FWIME_OK;
 }
 
@@ -237,21 +237,22 @@ static int prof_collect(fwime_ctx *x)
         CK(cudaEventElapsedTime(&ms, x->ev[p.ev], x->ev[p.ev + 1]));
         x->prof_ms[p.kind] += ms;
         x->prof_bytes[p.kind] += p.bytes;
-        x->prof_n[p.kind] += 1;
+        x->prof_n[p.kind] += p.n;
     }
     x->pend.clear();
     return FWIME_OK;
 }
 
-// a kernel launch: counts it and, when profiling, brackets it with events
-#define LAUNCH(kind, bytes, call)                                                                  \
+// n kernel launches (evaluated after them): counts them and, when profiling, brackets them with events
+#define LAUNCH_N(kind, bytes, call, n)                                                             \
     do {                                                                                           \
         int slot_;                                                                                 \
         TRY(prof_begin(x, slot_));                                                                 \
-        x->launches++;                                                                             \
         CK(call);                                                                                  \
-        TRY(prof_end(x, slot_, (kind), (bytes)));                                                  \
+        x->launches += (n);                                                                        \
+        TRY(prof_end(x, slot_, (kind), (bytes), (n)));                                             \
     } while (0)
+#define LAUNCH(kind, bytes, call) LAUNCH_N(kind, bytes, call, 1)
 
 static int auto_K(int nt)
 {
@@ -840,8 +841,9 @@ static int scatter(Run &r, int Sb, int n0, int kk, const float *W, RingRef in, R
     ext_cols(x, a.x_lo, a.x_hi);   // the launcher may start a few columns earlier (zero weights there)
     a.sigma = sigma; a.W = W; a.in = in; a.outr = out; a.accumulate = accumulate;
     const double pts = (double)x->g.nz * (a.x_hi - a.x_lo);
-    LAUNCH(FWIME_K_SCATTER, pts * ((double)a.npair * (8.0 + (accumulate ? 4 : 0)) + 4.0 * x->g.nh),
-           launch_scatter(a, x->st));
+    int n = 0;
+    LAUNCH_N(FWIME_K_SCATTER, pts * ((double)a.npair * (8.0 + (accumulate ? 4 : 0)) + 4.0 * x->g.nh),
+             launch_scatter(a, x->st, n), n);
     return FWIME_OK;
 }
 
@@ -857,7 +859,8 @@ static int image(Run &r, int Sb, int n0, int kk, int mode, RingRef D, RingRef L,
     const double pts = (double)x->g.nz * x->g.nx;
     const double per = 8.0 + (M2.base ? 4 : 0) + (Ds.base ? 4 : 0);
     const double once = mode == IMG_EXT ? 8.0 * x->g.nh + (img_local ? 8.0 : 0.0) : 8.0;
-    LAUNCH(FWIME_K_IMAGE, pts * ((double)a.npair * per + once), launch_image(a, mode, x->st));
+    int n = 0;
+    LAUNCH_N(FWIME_K_IMAGE, pts * ((double)a.npair * per + once), launch_image(a, mode, x->st, n), n);
     return FWIME_OK;
 }
 

@@ -198,8 +198,9 @@ bool pair_pays(long long P, int S);
 cudaError_t launch_prop_group(const GroupMember *m, int nactive, int ctas, const GroupRec *g, int nrec_threads,
                               int step, cudaStream_t st, bool record);
 cudaError_t launch_points(const PointsArgs &a, int nshot, cudaStream_t st);
-cudaError_t launch_scatter(const ExtArgs &a, cudaStream_t st);
-cudaError_t launch_image(const ImgArgs &a, int mode, cudaStream_t st);
+// (n: the kernels launched, more than one from 48 offsets on)
+cudaError_t launch_scatter(const ExtArgs &a, cudaStream_t st, int &n);
+cudaError_t launch_image(const ImgArgs &a, int mode, cudaStream_t st, int &n);
 cudaError_t launch_tlag_scatter(const TlagArgs &a, cudaStream_t st);
 cudaError_t launch_tlag_image(const TlagArgs &a, cudaStream_t st);
 int tlag_jc(int K, int lag, int nh);          // chunk length (outputs of one residue class) for segments of K steps

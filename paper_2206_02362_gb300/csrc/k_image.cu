@@ -293,7 +293,7 @@ static int launch_band(const ImgArgs &a, int h_lo, cudaStream_t st)
 #define FWIME_IMG_S48 4, 12, 4, 2, 6, 6, 4, 2
 #endif
 
-static cudaError_t launch_image_ext(const ImgArgs &a, cudaStream_t st)
+static cudaError_t launch_image_ext(const ImgArgs &a, cudaStream_t st, int &launched)
 {
     int h = -a.hm;
     while (h <= a.hm) {
@@ -306,6 +306,7 @@ static cudaError_t launch_image_ext(const ImgArgs &a, cudaStream_t st)
         else if (want + slack(4) <= 32) h = launch_band<ImgShape<FWIME_IMG_S32>>(a, h, st);
         else h = launch_band<ImgShape<FWIME_IMG_S48>>(a, h, st);
         ++h;
+        ++launched;
     }
     return cudaGetLastError();
 }
@@ -373,16 +374,18 @@ __global__ void __launch_bounds__(LOC_TX) k_image_local(const ImgArgs a, int xa,
         if (X + c >= a.x_lo && X + c < a.x_hi) a.img[off + c] += (acc[c][0] + acc[c][1]) + (acc[c][2] + acc[c][3]);
 }
 
-cudaError_t launch_image(const ImgArgs &a, int mode, cudaStream_t st)
+cudaError_t launch_image(const ImgArgs &a, int mode, cudaStream_t st, int &launched)
 {
+    launched = 0;
     if (a.npair <= 0 || a.x_hi <= a.x_lo || a.z_hi <= a.z_lo) return cudaSuccess;
     if (!a.img || !a.D.base || !a.L.base || (a.img_local && (!a.M2.base || !a.Ds.base))) return cudaErrorInvalidValue;
-    if (mode == IMG_EXT) return launch_image_ext(a, st);
+    if (mode == IMG_EXT) return launch_image_ext(a, st, launched);
     const int xa = a.x_lo - a.x_lo % 4;   // 16-byte aligned: rows are NXP (a multiple of 32) floats apart
     const int ncol4 = (a.x_hi - xa + 3) / 4;
     const long long n = (long long)ncol4 * (a.z_hi - a.z_lo);
     if (n > 0x7fffffff - LOC_TX || (a.M2.base == nullptr) != (a.Ds.base == nullptr)) return cudaErrorInvalidValue;
     const unsigned grid = (unsigned)((n + LOC_TX - 1) / LOC_TX);
+    launched = 1;
     if (a.M2.base) k_image_local<true><<<grid, LOC_TX, 0, st>>>(a, xa, ncol4, (int)n);
     else k_image_local<false><<<grid, LOC_TX, 0, st>>>(a, xa, ncol4, (int)n);
     return cudaGetLastError();

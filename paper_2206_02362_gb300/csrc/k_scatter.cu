@@ -320,8 +320,9 @@ static int launch_band(const ExtArgs &a, int g_lo, int accumulate, cudaStream_t 
 #define FWIME_SC_S48 2, 24, 4, 1, 8, 5, 2
 #endif
 
-cudaError_t launch_scatter(const ExtArgs &a, cudaStream_t st)
+cudaError_t launch_scatter(const ExtArgs &a, cudaStream_t st, int &launched)
 {
+    launched = 0;
     if (a.npair <= 0 || a.x_hi <= a.x_lo || a.z_hi <= a.z_lo) return cudaSuccess;
     if (!a.W || !a.in.base || !a.outr.base || a.hm != (a.nh - 1) / 2) return cudaErrorInvalidValue;
     int g = -a.hm, acc = a.accumulate;
@@ -336,6 +337,7 @@ cudaError_t launch_scatter(const ExtArgs &a, cudaStream_t st)
         else if (want <= 32) g = launch_band<ScatShape<FWIME_SC_S32>>(a, g, acc, st);
         else g = launch_band<ScatShape<FWIME_SC_S48>>(a, g, acc, st);
         ++g;
+        ++launched;
         acc = 1;
     }
     return cudaGetLastError();
