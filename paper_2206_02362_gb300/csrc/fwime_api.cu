@@ -391,6 +391,7 @@ struct Reuse {
     bool read = false, write = false;
     int K = 0;          // the segment length that the states read or written have (0: none)
     bool must = false;  // cannot do without (the split gradient's halves)
+    bool pairs = true;  // runs of steps may take two per launch (not in a group's launches)
 };
 
 int fwk::least_segment(int nt) { return auto_K(nt); }
@@ -525,8 +526,9 @@ static int plan(fwime_ctx *x, int op, WS &w, Reuse &u)
     if (x->max_ws && need > budget)
         return fail(x, FWIME_ENOMEM, "operator needs %zu bytes for S=%d, K=%d; budget %zu", need, w.S, w.K, budget);
     const size_t alt_bytes = 2 * al((size_t)w.S * x->P) * sizeof(float);
-    const bool alt = op != FWIME_OP_BORN && !x->opt_plain && !x->opt_fs && pair_pays(x->P, w.S) &&
-                     need + alt_bytes <= budget;
+    // (B and, with time lags, T launch every step singly)
+    const bool alt = u.pairs && op != FWIME_OP_BORN && !(op == FWIME_OP_TOMO && x->opt_tlag > 0) && !x->opt_plain &&
+                     !x->opt_fs && pair_pays(x->P, w.S) && need + alt_bytes <= budget;
     if (alt) need += alt_bytes;
     if (need > x->ws_bytes) {
         if (x->capturing) return fail(x, FWIME_EBUSY, "workspace growth during graph capture");
@@ -2389,7 +2391,9 @@ int fwime_forward_group(fwime_ctx *const *ctxs, int n, const float *const *v, co
     for (int i = 0; i < n; ++i) {
         fwime_ctx *m = ctxs[i];
         bg_yield(m);
-        TRY(plan(m, FWIME_OP_FORWARD, runs[i].w));
+        Reuse u;
+        u.pairs = false;
+        TRY(plan(m, FWIME_OP_FORWARD, runs[i].w, u));
         if (runs[i].w.S < m->nshot)
             return fail(x, FWIME_ENOMEM, "group member %d: %d shots do not fit one batch", i, m->nshot);
         const bool was = m->shared;
@@ -2642,7 +2646,7 @@ int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
             const int props = r.w.hist ? KEPT[op] : PROPS[op];
             int paired = 0;
             float t2 = 0.f;                        // a step of a launch of two
-            if (r.w.alt[0] && kk >= 2 && !(lag && op == FWIME_OP_TOMO)) {
+            if (r.w.alt[0] && kk >= 2) {
                 PairArgs m{};
                 m.a = prop_args(r, r.w.f[0], r.w.f[1], r.w.alt[0], nullptr, nullptr, 0, r.w.f[0], 1.f, nullptr, nullptr,
                                 RecTo{}, InjFrom{});
