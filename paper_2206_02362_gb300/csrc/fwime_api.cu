@@ -734,8 +734,8 @@ static int prop(Run &r, int Sb, const float *cur, const float *prev, float *out,
     return FWIME_OK;
 }
 
-// A run of time steps whose operands move by fixed strides.  Fields: cur and prev (at the end the last two steps), or, with R > 0, slots of the ring `ring` (SP floats apart)
-// for m = m0, m0 - 1, ...: slot m from m + 1 and m + 2.
+// A run of time steps whose operands move by fixed strides.  Fields: cur and prev (at the end the last two steps), or,
+// with R > 0, slots of the ring `ring` (SP floats apart) for m = m0, m0 - 1, ...: slot m from m + 1 and m + 2.
 struct Steps {
     float *cur = nullptr, *prev = nullptr;
     float *ring = nullptr;
@@ -840,7 +840,7 @@ static int scatter(Run &r, int Sb, int n0, int kk, const float *W, RingRef in, R
     ExtArgs a{};
     a.NXP = x->NXP; a.nh = x->g.nh; a.hm = (x->g.nh - 1) / 2; a.S = Sb; a.npair = kk * Sb; a.n0 = n0; a.P = x->P;
     a.z_lo = x->o; a.z_hi = x->o + x->g.nz;
-    ext_cols(x, a.x_lo, a.x_hi);   // the launcher may start a few columns earlier (zero weights there)
+    ext_cols(x, a.x_lo, a.x_hi);
     a.sigma = sigma; a.W = W; a.in = in; a.outr = out; a.accumulate = accumulate;
     const double pts = (double)x->g.nz * (a.x_hi - a.x_lo);
     int n = 0;

@@ -1,5 +1,5 @@
 // Device helpers shared by the extension kernels (scatter, imaging): walking the (step, shot) pairs of a
-// segment, asynchronous copies, 16-byte shared loads as packed pairs.
+// segment, asynchronous copies.
 #pragma once
 #include "fwime_kernels.cuh"
 
@@ -22,16 +22,14 @@ template <int N>
 struct PairRows {
     const float *row[N];
     int slot[N], s;
-    // starting at pair p0
-    __device__ __forceinline__ void init(const RingRef *const (&r)[N], int n0, int S, long long P, long long rowoff,
-                                         int p0 = 0)
+    // starting at the first pair
+    __device__ __forceinline__ void init(const RingRef *const (&r)[N], int n0, long long rowoff)
     {
-        const int step = p0 / S;
-        s = p0 - step * S;
+        s = 0;
 #pragma unroll
         for (int k = 0; k < N; ++k) {
-            slot[k] = r[k]->mod > 0 ? (n0 + r[k]->shift + step) % r[k]->mod : r[k]->shift + step;
-            row[k] = r[k]->base + rowoff + (long long)slot[k] * r[k]->slot_stride + (long long)s * P;
+            slot[k] = r[k]->mod > 0 ? (n0 + r[k]->shift) % r[k]->mod : r[k]->shift;
+            row[k] = r[k]->base + rowoff + (long long)slot[k] * r[k]->slot_stride;
         }
     }
     __device__ __forceinline__ void next(const RingRef *const (&r)[N], int S, long long P, long long rowoff)
@@ -49,13 +47,5 @@ struct PairRows {
         }
     }
 };
-
-// four consecutive floats of shared memory (16-byte aligned) as two packed pairs
-__device__ __forceinline__ void lds_pairs(const float *p, f32x2 &a, f32x2 &b)
-{
-    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(p);
-    a = v.x;
-    b = v.y;
-}
 
 }  // namespace fwk

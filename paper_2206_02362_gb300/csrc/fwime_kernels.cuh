@@ -73,7 +73,7 @@ struct PropArgs {
     long long rec_dstride;
     int nrec, rec_acc;
     // optional receiver injection into the OUTPUT field: out(rec_r) += c(rec_r) inj_val[s * inj_vstride + r]
-    // (the transpose of recording, as k_points injects it).  inj_map[(z - inj_lo) * NXP + x] is the first
+    // (the transpose of recording; g = 1 on the physical grid, where receivers live).  inj_map[(z - inj_lo) * NXP + x] is the first
     // receiver at padded point (z, x) of the rows [inj_lo, inj_hi) or -1, inj_next[r] the next receiver at
     // the same point or -1.
     const int *inj_map, *inj_next;
@@ -130,12 +130,6 @@ struct PointsArgs {
     float *d;
     long long dstride;
     int accumulate;
-    // inject: fld[s*P + off] += c[off] * val[s*vstride + r]   (c g at a receiver; g = 1 on the
-    // physical grid, where receivers live)
-    float *fld;
-    const float *val;
-    long long vstride;
-    const float *c;
 };
 
 // A ring operand of the segment kernels: slot of time step n (pair row j) is

@@ -533,19 +533,16 @@ static cudaError_t dispatch_prop(const PropArgs &a0, int nshot, cudaStream_t st)
         else launch_prop_t<FS, 0, false, false, true>(a, grid, block, smem, st);
         return cudaGetLastError();
     }
-    switch (key) {
+    switch (key) {                             // no operator has a point source and local sources in one step
     case 0: launch_prop_t<FS, 0, false, false>(a, grid, block, smem, st); break;
     case 1: launch_prop_t<FS, 0, false, true>(a, grid, block, smem, st); break;
     case 2: launch_prop_t<FS, 0, true, false>(a, grid, block, smem, st); break;
     case 3: launch_prop_t<FS, 0, true, true>(a, grid, block, smem, st); break;
     case 4: launch_prop_t<FS, 1, false, false>(a, grid, block, smem, st); break;
-    case 5: launch_prop_t<FS, 1, false, true>(a, grid, block, smem, st); break;
     case 6: launch_prop_t<FS, 1, true, false>(a, grid, block, smem, st); break;
-    case 7: launch_prop_t<FS, 1, true, true>(a, grid, block, smem, st); break;
     case 8: launch_prop_t<FS, 2, false, false>(a, grid, block, smem, st); break;
-    case 9: launch_prop_t<FS, 2, false, true>(a, grid, block, smem, st); break;
     case 10: launch_prop_t<FS, 2, true, false>(a, grid, block, smem, st); break;
-    default: launch_prop_t<FS, 2, true, true>(a, grid, block, smem, st); break;
+    default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }

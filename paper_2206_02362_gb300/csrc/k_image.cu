@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(LOC_TX) k_image_local(const ImgArgs a, int xa,
     for (int f = 0; f < NF; ++f) rings_[f] = rings4[f];
     const RingRef *const (&rings)[NF] = rings_;
     PairRows<NF> it;
-    it.init(rings, a.n0, a.S, a.P, off);
+    it.init(rings, a.n0, off);
     float acc[4][4] = {};
     auto add = [&](const float4 (&v)[NF], int u) {
         const float dv[4] = {v[0].x, v[0].y, v[0].z, v[0].w}, lv[4] = {v[1].x, v[1].y, v[1].z, v[1].w};

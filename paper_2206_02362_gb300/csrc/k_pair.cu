@@ -76,31 +76,26 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_MINB) k_prop_pair(const 
     const int y0 = dz > 0 ? z0 - 4 : z1 + 3, ye = dz > 0 ? z1 + 4 : z0 - 5;   // rows of the first step
     int oA = y0 * NXP + (nA ? cA : 0), oB = y0 * NXP + (nB ? cB : 0), oX = y0 * NXP + (nX ? x : 0);
     const float *cur = a.cur + so, *prev = a.prev + so;
-    const auto cp = [](float *dst, const float *src, int n) {
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-                     "l"(src), "r"(n)
-                     : "memory");
-    };
     // Row k of q^n after row y (and the offsets) into slot s.  Rows outside the grid are not read: what the rows that
     // depend on them make of the slot's old contents is replaced by zero.
     const int yend = dz > 0 ? min(a.NZ, z1 + 8) : max(-1, z0 - 9);
     const auto issue_cur = [&](int y, int k, int s) {
         if ((y + k * dz - yend) * dz >= 0) return;
         const float *src = cur + (long long)k * NX;
-        cp(curL + s * CUR_ROW, src + oA, nA);
-        if (two) cp(curL + s * CUR_ROW + STRIP, src + oB, nB);
+        cp16n(curL + s * CUR_ROW, src + oA, nA);
+        if (two) cp16n(curL + s * CUR_ROW + STRIP, src + oB, nB);
     };
     const auto issue_aux = [&](int y, int k, int s) {
         if ((y + k * dz - ye) * dz >= 0) return;
-        cp(cL + s * STRIP, a.c + (long long)k * NX + oX, nX);
-        cp(midL + s * STRIP, prev + (long long)k * NX + oX, nX);
+        cp16n(cL + s * STRIP, a.c + (long long)k * NX + oX, nX);
+        cp16n(midL + s * STRIP, prev + (long long)k * NX + oX, nX);
     };
     const auto issue_f = [&](int y, int k, int s) {
         const int zr = y + k * dz, zr2 = zr - 4 * dz;
         if ((zr - ye) * dz >= 0) return;
         const bool lin = zr >= a.zs_lo && zr < a.zs_hi, lin2 = zr2 >= a.zs_lo && zr2 < a.zs_hi;
-        cp(fL + s * STRIP, a.f0 + so + (lin ? (long long)k * NX + oX : 0), lin ? nX : 0);
-        cp(fL + (PAIR_LRING + s) * STRIP, m.f0b + so + (lin2 ? (long long)(k - 4) * NX + oX : 0), lin2 ? nX : 0);
+        cp16n(fL + s * STRIP, a.f0 + so + (lin ? (long long)k * NX + oX : 0), lin ? nX : 0);
+        cp16n(fL + (PAIR_LRING + s) * STRIP, m.f0b + so + (lin2 ? (long long)(k - 4) * NX + oX : 0), lin2 ? nX : 0);
     };
 
     // queue of q^n: rows y-4 .. y+3 for the first y; queue of q^{n+1}: rows y-8 .. y-1, none yet

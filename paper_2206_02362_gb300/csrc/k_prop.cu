@@ -107,22 +107,17 @@ cudaError_t launch_prop(const PropArgs &a, int nshot, cudaStream_t st)
 }
 
 // ----------------------------------------------------------------- points
-// Receiver recording d[n][r] = q^n(rec_r) and adjoint injection of the data
-// residual at the receivers (the transpose of recording, scaled by c g so it
-// enters the mu-form adjoint recursion inside c (L mu + R^T r)).
+// Receiver recording d[n][r] = q^n(rec_r), of the samples that no stencil launch records.
 __global__ void k_points(const PointsArgs a)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     const int s = blockIdx.y;
     if (r >= a.nrec) return;
     const long long off = (long long)s * a.P + a.rec_off[r];
-    if (a.d) {
-        float val = a.f1[off];
-        if (a.f2) val += a.f2[off];
-        float *dp = a.d + (long long)s * a.dstride + r;
-        *dp = a.accumulate ? *dp + val : val;
-    }
-    if (a.fld) atomicAdd(a.fld + off, a.c[a.rec_off[r]] * a.val[(long long)s * a.vstride + r]);
+    float val = a.f1[off];
+    if (a.f2) val += a.f2[off];
+    float *dp = a.d + (long long)s * a.dstride + r;
+    *dp = a.accumulate ? *dp + val : val;
 }
 
 cudaError_t launch_points(const PointsArgs &a, int nshot, cudaStream_t st)
