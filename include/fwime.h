@@ -86,8 +86,9 @@ enum {
     FWIME_OPT_SHOTS_PER_BATCH = 1, /* shots advanced together per launch; 0 = as many as fit */
     FWIME_OPT_SEGMENT = 2,         /* checkpoint/ring segment length K in time steps; 0 = auto: the adjoint operators
                                       then keep the source side's second time derivatives of the whole record where
-                                      that fits a third of the device memory (or max_workspace_bytes) and is faster,
-                                      instead of recomputing them from checkpoints (the same results) */
+                                      that fits a third of the device memory and half of what is free (or
+                                      max_workspace_bytes) and is faster, instead of recomputing them from
+                                      checkpoints (the same results) */
     FWIME_OPT_PLAIN = 3,           /* 1 = plain path: one shot per launch, host-driven steps */
     FWIME_OPT_GRAPH = 4,           /* 1 = capture each operator call in a CUDA graph and replay */
     FWIME_OPT_HOST_IO = 5,         /* 1 = I/O pointers are host memory */
@@ -96,8 +97,9 @@ enum {
     FWIME_OPT_WORKSPACE = 8,       /* read-only: bytes of device workspace held */
     FWIME_OPT_PROFILE = 9,         /* 1 = bracket every kernel launch with CUDA events (no graphs) */
     FWIME_OPT_REUSE_BACKGROUND = 10, /* 1 = B / B~ keep the background wavefield of every shot (its second time
-                                       derivative at every step where that fits a third of the device memory,
-                                       else its segment-start states when they fit) and a following B* / B~*
+                                       derivative at every step where that fits a third of the device memory and
+                                       half of what is free, else its segment-start states when they fit) and a
+                                       following B* / B~*
                                        with the SAME v and w pointers starts from them instead of its own
                                        forward sweep (one propagation fewer).  The caller guarantees
                                        that v and w are not modified in between; any other operator call

@@ -365,11 +365,13 @@ struct WS {
     float *sv, *sw, *sd1, *sd2, *sm1, *sdv, *smo;
 };
 
-// Device memory the kept D2t histories may take: a third of the card, so that two more contexts of the same kind
-// (and the caller's own arrays) still fit beside this one.
-static size_t hist_cap(const fwime_ctx *x, size_t budget)
+// Device memory the kept D2t histories may take of `avail` bytes: a third of the card, and half of what is there, so
+// that however many contexts run, the next one and the caller's own arrays still find room; `held` bytes of it are the
+// context's already.
+static size_t hist_cap(const fwime_ctx *x, size_t avail, size_t held)
 {
-    return std::min(budget, x->max_ws ? x->max_ws : x->dev_mem / 3);
+    const size_t third = x->dev_mem / 3;
+    return std::min(avail, x->max_ws ? x->max_ws : std::min(third, std::max(avail / 2, held)));
 }
 
 // Does keeping the histories at S_h shots per launch beat recomputing at S_c?  Stencil launches per step with and
@@ -485,7 +487,7 @@ static int plan(fwime_ctx *x, int op, WS &w, Reuse &u)
     w.hist = false;
     int hist_S = 0;
     if (adj_op && !no_ckpt && (x->opt_K == 0 || x->tuned_K) && x->opt_tlag == 0 && !x->opt_plain) {
-        const size_t cap = hist_cap(x, budget);
+        const size_t cap = hist_cap(x, budget, x->ws_bytes);
         const Sizes sh = op_sizes(x->g, x->nshot, x->nrec, x->P, x->NZ, x->NXP, op, w.K, x->opt_host_io != 0, false, 0, true);
         const size_t hf = (sh.model + sh.staging) * sizeof(float) + 4096, hp = sh.per_shot * sizeof(float);
         int S_h = x->opt_S > 0 ? S_max : batch(cap, hf, hp);
@@ -943,7 +945,7 @@ static bool bg_reserve(fwime_ctx *x, int op, int &K)
     const int adj = op == FWIME_OP_BORN ? FWIME_OP_BORN_ADJ : FWIME_OP_BORN_EXT_ADJ;
     const int Kp = x->opt_tlag > 0 && x->opt_K == 0 ? clamp_K(x, std::max(Ks, 4 * tlag_Hs(x->g, x->opt_tlag))) : Ks;
     const size_t pair = std::max(batch_bytes(x, op, Kp, false), batch_bytes(x, adj, Kp, true));
-    const bool hist = may_hist && hneed <= hist_cap(x, tot) && fits(hneed) && !(x->max_ws && hneed + pair > x->max_ws);
+    const bool hist = may_hist && hneed <= hist_cap(x, fr + x->bg.bytes, 0) && fits(hneed) && !(x->max_ws && hneed + pair > x->max_ws);
     const size_t need = hist ? hneed : need_st;
     if (!fits(need)) return false;
     if (x->bg.buf) cudaFreeAsync(x->bg.buf, x->st);
