@@ -406,22 +406,26 @@ def peaks():
 
 
 def ncu_traffic():
-    """Per-launch DRAM bytes of the stencil kernel from the committed ncu summary, if it was
-    taken on the current kernel source (else None)."""
-    src = os.path.join(ROOT, "paper_2206_02362_gb300", "csrc", "k_prop.cu")
-    h = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
+    """Per-launch DRAM bytes of the stencil kernels from the committed ncu summary, if it was
+    taken on the current sources of k_prop and k_prop_pair (else None)."""
     path = os.path.join(ROOT, "profiles", "k_prop_marmousi2_ncu.md")
     if not os.path.exists(path):
         return None
     txt = open(path).read()
-    m = re.search(r"k_prop\.cu sha256\[:16\]:\s*([0-9a-f]{16})", txt)
+    for name in ("k_prop.cu", "fwime_prop.cuh", "k_pair.cu"):
+        src = os.path.join(ROOT, "paper_2206_02362_gb300", "csrc", name)
+        h = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
+        m = re.search(re.escape(name) + r" sha256\[:16\]:\s*([0-9a-f]{16})", txt)
+        if not m or m.group(1) != h:
+            return None
     t = re.search(r"dram bytes per full-size launch:\s*([0-9.eE+]+)", txt)
     a = re.search(r"algorithmic bytes of that variant per full-size launch:\s*([0-9.eE+]+)", txt)
-    if not m or not t or m.group(1) != h:
+    if not t:
         return None
     return {"dram_bytes_per_launch": float(t.group(1)),
             "algorithmic_bytes_per_launch": float(a.group(1)) if a else None,
-            "captured": "every k_prop launch of one timed bench step (full-size launches: 100 shots, nt 40), 1-pass ncu",
+            "captured": "every k_prop and k_prop_pair launch of one timed bench step (full-size launches: 100 shots, "
+                        "nt 40), 1-pass ncu",
             "source": "profiles/k_prop_marmousi2_ncu.md"}
 
 
@@ -520,7 +524,7 @@ def main():
     peak, peak_kind = peaks()
     achieved = pk["bytes"] / (pk["ms"] * 1e-3) / 1e9 if pk["ms"] > 0 else None
     traffic = ncu_traffic()
-    roofline = {"bound": "hbm", "kernel": "k_prop (wave-equation time step, forward and adjoint)",
+    roofline = {"bound": "hbm", "kernel": "k_prop, k_prop_pair (wave-equation time steps, forward and adjoint)",
                 "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak if achieved else None, "peak_source": peak_kind + " (MEASURED_PEAKS.json hbm_gbs)",
                 "traffic": traffic["dram_bytes_per_launch"] if traffic else None,

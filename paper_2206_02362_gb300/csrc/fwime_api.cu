@@ -133,7 +133,8 @@ void ctx_set_shared(fwime_ctx *x) { x->shared = true; }
 // No other stream's work is expected beside this context's: it runs on the default stream, where calls follow one
 // another whoever makes them.  Only then does one call's latency come before the work in all (items of a few rows,
 // which load three times the rows that they write): on streams of their own, eight threads with one small shot each
-// complete 889 calls/s with items of eight rows or more, and made 463 with short ones where long ones made 657.
+// complete 889 calls/s with items of eight rows or more, and made 463 with short ones where long ones made 657.  (One
+// user alone on a stream of their own gets the long items too: a context cannot tell.)
 static bool alone(const fwime_ctx *x) { return !x->shared && x->st == nullptr; }
 }  // namespace fwk
 

@@ -67,8 +67,8 @@ __device__ __forceinline__ float4 lds4(const float *p) { return *reinterpret_cas
 // q^{n-1} and c; with local sources rings of three rows of those, of q^{n-1} and of c.  Nine is the period of the
 // unrolled register queue, so every slot is a compile-time constant.  Row z waits for the copy group issued four rows
 // (with local sources three) earlier.  With slots and addresses computed per row and lane a row of 128 points took 211
-// instructions and 124 registers, now 102 to 108: 350 x 1700 points, 8 shots, 15.8 / 13.9 us per step; from about 16
-// shots on the kernel is bound by memory and the two are equal.
+// instructions in 124 registers, now 139 (one local source) in 103 to 116: 350 x 1700 points, 8 shots, 15.8 / 13.9 us
+// per step; from about 16 shots on the kernel is bound by memory and the two are equal.
 constexpr int RING = 9, LRING = 3;
 // Variants k_prop<LOC, D2, SRC>: LOC = 0 no dense local source, 1 exactly one (f0, weight a0), 2 the
 // general sum a0 f0 + a1 f1 + a2 f2 + coef fc; D2 writes D2t; SRC adds the point source.  Register

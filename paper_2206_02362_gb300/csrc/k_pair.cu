@@ -9,7 +9,7 @@ namespace fwk {
 // launch read q^n and q^{n-1} and write q^{n+1} and q^{n+2}: 16 B instead of 24.  A warp marches down its strip as
 // k_prop does, computes row y of the first step, keeps those rows in a second register queue and computes row y - 4 of
 // the second step from it; four rows above and below its chunk and four columns left and right of its strip are
-// computed twice (250 instructions per row and pair on 120 columns, where k_prop spends 211 per row and step on 128).
+// computed twice (250 instructions per row and pair on 120 columns; k_prop spends 139 per row and step on 128).
 // Same products and sums in the same order as k_prop: the same bits.
 //
 // What it took: every ring slot a compile-time constant (rings of nine rows, the period of the unrolled queues), a
@@ -234,9 +234,11 @@ bool pair_runs(const PropArgs &a)
            a.fs_row == 0 && a.P < (1LL << 31);
 }
 
-// From where a step's three fields no longer stay in L2 (129 MB); below it saves no traffic (us per step, one launch
-// per step and with pairs: 350 x 1700 points, 8 shots 15.8 / 16.4, 16 shots 28.9 / 29.6, 24 shots 45.1 / 37.6, 32 shots
-// 55.6 / 46.8; 1200 x 5000 points, 1 shot 17.5 / 22.5, 2 shots 41.4 / 31.4, 4 shots 67.2 / 53.0).
+// From where a step's three fields no longer stay in this chip's L2 (129 MB); below it saves no traffic (us per step,
+// one launch per step and with pairs: 350 x 1700 points, 8 shots 15.8 / 16.4, 16 shots 28.9 / 29.6, 24 shots 45.1 /
+// 37.6, 32 shots 55.6 / 46.8; 1200 x 5000 points, 1 shot 17.5 / 22.5, 2 shots 41.4 / 31.4, 4 shots 67.2 / 53.0; the
+// line lies between the two sizes' 16 and 24 shots and 1 and 2, and batches of fewer than 8 shots on the smaller grid
+// were not measured).
 bool pair_pays(long long P, int S) { return P * S >= 13000000; }
 
 cudaError_t launch_pair(const PairArgs &m0, int nshot, cudaStream_t st)
