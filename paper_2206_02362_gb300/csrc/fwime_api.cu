@@ -529,9 +529,10 @@ static int plan(fwime_ctx *x, int op, WS &w, Reuse &u)
     if (x->max_ws && need > budget)
         return fail(x, FWIME_ENOMEM, "operator needs %zu bytes for S=%d, K=%d; budget %zu", need, w.S, w.K, budget);
     const size_t alt_bytes = 2 * al((size_t)w.S * x->P) * sizeof(float);
-    // (B and, with time lags, T launch every step singly)
-    const bool alt = u.pairs && op != FWIME_OP_BORN && !(op == FWIME_OP_TOMO && x->opt_tlag > 0) && !x->opt_plain &&
-                     !x->opt_fs && pair_pays(x->P, w.S) && need + alt_bytes <= budget;
+    // (B and, with time lags, T and the objective launch every step singly)
+    const bool single = op == FWIME_OP_BORN || (x->opt_tlag > 0 && (op == FWIME_OP_TOMO || op == FWIME_OP_OBJECTIVE));
+    const bool alt = u.pairs && !single && !x->opt_plain && !x->opt_fs && pair_pays(x->P, w.S) &&
+                     need + alt_bytes <= budget;
     if (alt) need += alt_bytes;
     if (need > x->ws_bytes) {
         if (x->capturing) return fail(x, FWIME_EBUSY, "workspace growth during graph capture");

@@ -1,6 +1,6 @@
-"""The two further fields of two-step launches are reserved only for calls that use them: the workspace of T with time
-lags and of a grouped forward grows by the same bytes per shot below and above the line (13 M points) from which
-batches run two steps per launch; that of a plain forward call by two fields more."""
+"""The two further fields of two-step launches are reserved only for calls that use them: the workspace of T and of the
+objective with time lags and of a grouped forward grows by the same bytes per shot below and above the line (13 M
+points) from which batches run two steps per launch; that of a plain forward call by two fields more."""
 import numpy as np
 import pytest
 
@@ -21,9 +21,11 @@ def workspace(kind, nshot):
     geom = fw.Geometry(np.full(nshot, 2), np.arange(nshot), np.array([3]), np.array([4]))
     d = torch.zeros((nshot, NT, 1), device="cuda")
     grid = fw.Grid(nz=NZ, nx=NX, sponge=W, nt=NT, dt=1e-3, dx=10.0, nh=NH)
-    with fw.Context(grid, geom, time_lag=1 if kind == "tomo_lag" else 0) as ctx:
+    with fw.Context(grid, geom, time_lag=1 if kind.endswith("lag") else 0) as ctx:
         if kind == "tomo_lag":
             ctx.tomo(v, w, pt, dv, d)
+        elif kind == "objective_lag":
+            ctx.objective(v, w, pt, d)
         elif kind == "group":
             fw.forward_group([ctx], [v], [w], [d])
         else:
@@ -31,7 +33,7 @@ def workspace(kind, nshot):
         return ctx.get_option("workspace")
 
 
-@pytest.mark.parametrize("kind,more", [("tomo_lag", 0), ("group", 0), ("forward", 2)])
+@pytest.mark.parametrize("kind,more", [("tomo_lag", 0), ("objective_lag", 0), ("group", 0), ("forward", 2)])
 def test_further_fields_only_where_they_are_used(kind, more):
     size = {s: workspace(kind, s) for s in (2, 4, 6)}
     field = 4 * POINTS
