@@ -68,3 +68,15 @@ def test_tuned_pair_keeps_the_background():
             ctx.set_option("segment", s["segment"])
     close(outs[0], outs[1])
     assert counts[1] - counts[0] >= (NT - 1) * -(-NSHOT // s["shots_per_batch"])
+
+
+def test_tuned_batches_are_not_cut_for_a_history():
+    """20 Marmousi2-sized shots, a history of 7 in the cap, checkpoints of all: the tuner keeps the batch of all shots
+    (or of half of them) instead of the few shots that a history leaves room for."""
+    nz, nx, nt, nshot = 350, 1700, 401, 20
+    field = 4 * 458 * 1824
+    grid = fw.Grid(nz=nz, nx=nx, sponge=50, nt=nt, dt=8e-4, dx=10.0, nh=3)
+    geom = fw.Geometry(np.full(nshot, 2), 80 * np.arange(nshot), np.full(20, 1), np.arange(20))
+    # fields per shot: 424 with the history (K = 20), 84 with checkpoints (104 at K = 40)
+    with fw.Context(grid, geom, max_workspace_bytes=7 * 450 * field) as ctx:
+        assert ctx.autotune_schedule(fw.OP_BORN_EXT_ADJ)["shots_per_batch"] in (nshot, nshot // 2)
