@@ -2617,6 +2617,7 @@ int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
         return FWIME_OK;
     };
     double best = 1e300;
+    std::map<int, float> pair_us;
     fwime_schedule out{};
     int rc = FWIME_OK;
     for (int K : Ks) {
@@ -2653,7 +2654,7 @@ int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
             const int kk = std::min(K, x->g.nt - 1);
             const int props = r.w.hist ? KEPT[op] : PROPS[op];
             int paired = 0;
-            float t2 = 0.f;                        // a step of a launch of two
+            float &t2 = pair_us[S];                // a step of a launch of two: of the batch alone, whatever K
             if (r.w.alt[0] && kk >= 2) {
                 PairArgs m{};
                 m.a = prop_args(r, r.w.f[0], r.w.f[1], r.w.alt[0], nullptr, nullptr, 0, r.w.f[0], 1.f, nullptr, nullptr,
@@ -2661,16 +2662,19 @@ int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
                 m.out2 = r.w.alt[1];
                 m.f0b = r.w.f[0];
                 if (pair_runs(m.a)) {
-                    rc = timed([&]() -> int {
-                        LAUNCH(FWIME_K_PROP, 0.0, launch_pair(m, S, x->st));
-                        return FWIME_OK;
-                    }, 4, t2);
-                    if (rc != FWIME_OK) break;
-                    t2 *= 0.5f;
+                    if (t2 == 0.f) {
+                        rc = timed([&]() -> int {
+                            LAUNCH(FWIME_K_PROP, 0.0, launch_pair(m, S, x->st));
+                            return FWIME_OK;
+                        }, 8, t2);
+                        if (rc != FWIME_OK) break;
+                        t2 *= 0.5f;
+                    }
                     paired = std::min(lag && op >= FWIME_OP_TOMO ? 3 : PAIRED[op], props);
                 }
             }
-            tp = ((props - paired) * tp + paired * t2) / props;
+            const float tr = (kk / 2 * 2 * t2 + kk % 2 * tp) / kk;   // (a run of an odd number starts with a single step)
+            tp = ((props - paired) * tp + paired * tr) / props;
             float tsc = 0.f, tim = 0.f;
             if (!lag && SCAT[op] > 0 && r.w.W && r.w.ring[0] && r.w.ring[1]) {
                 rc = timed([&]() {
@@ -2682,15 +2686,21 @@ int fwime_autotune_schedule(fwime_ctx *x, int op, fwime_schedule *res)
             float *img_acc = op == FWIME_OP_BORN_EXT_ADJ ? r.w.acc1 : r.w.acc2;
             float *lring = op == FWIME_OP_BORN_EXT_ADJ ? r.w.ring[1] : r.w.ring[3];
             if (!lag && IMGS[op] > 0 && img_acc && r.w.ring[0] && lring) {
+                const bool two = op != FWIME_OP_BORN_EXT_ADJ;   // T*, gradient: with the local terms
                 rc = timed([&]() {
                     return image(r, S, 0, kk, IMG_EXT, ringref(r.w.ring[0], SP, 0, 0), ringref(lring, SP, r.w.R, 1),
-                                 ringref(nullptr, 0, 0, 0), ringref(nullptr, 0, 0, 0), 1.f, img_acc);
+                                 ringref(two ? r.w.ring[5] : nullptr, SP, r.w.R, 1),
+                                 ringref(two ? r.w.ring[2] : nullptr, SP, 0, 0), 1.f, img_acc, two ? r.w.acc1 : nullptr);
                 }, 2, tim);
                 if (rc != FWIME_OK) break;
             }
             const double nseg = (double)r.w.nseg;
             const int scat = SCAT[op] - (r.w.hist && SCAT[op] > 0 ? 1 : 0);
-            const double per_shot = ((double)(x->g.nt - 1) * props * tp + nseg * (scat * tsc + IMGS[op] * tim)) / S;
+            // states at the segments' starts, written and read again (at 6.2 TB/s, as hist_pays)
+            const int states = r.w.ckpt && !lag ? (props == 6 ? 8 : 4) : 0;
+            const double copies = states * 8.0 * (double)SP / 6.2e6;
+            const double per_shot =
+                ((double)(x->g.nt - 1) * props * tp + nseg * (scat * tsc + IMGS[op] * tim + copies)) / S;
             if (per_shot < best) {
                 best = per_shot;
                 out.shots_per_batch = S;
