@@ -490,8 +490,8 @@ static int plan(fwime_ctx *x, int op, WS &w, Reuse &u)
     if (adj_op && !no_ckpt && (x->opt_K == 0 || x->tuned_K) && x->opt_tlag == 0 && !x->opt_plain) {
         const size_t cap = hist_cap(x, budget, x->ws_bytes);
         const Sizes sh = op_sizes(x->g, x->nshot, x->nrec, x->P, x->NZ, x->NXP, op, w.K, x->opt_host_io != 0, false, 0, true);
-        const size_t hf = (sh.model + sh.staging) * sizeof(float) + 4096, hp = sh.per_shot * sizeof(float);
-        int S_h = x->opt_S > 0 ? S_max : batch(cap, hf, hp);
+        const size_t hf = (sh.model + sh.staging) * sizeof(float), hp = sh.per_shot * sizeof(float);
+        int S_h = x->opt_S > 0 ? S_max : batch(cap, hf + 4096, hp);
         if (x->opt_S == 0) {
             // The history's memory is mapped once per context, at about 870 GB/s; more batches map less and launch
             // more (6 us per stencil launch).  The number of batches that is best for four calls on a context:
@@ -504,7 +504,7 @@ static int plan(fwime_ctx *x, int op, WS &w, Reuse &u)
             S_h = (x->nshot + batches - 1) / batches;   // of equal size
         }
         const int S_c = x->opt_S > 0 ? S_max : batch(budget, fixed, per);
-        if (hf + hp * (size_t)S_h <= cap && hist_pays(x, op, S_h, S_c)) {
+        if (hf + hp * (size_t)S_h + 4096 <= cap && hist_pays(x, op, S_h, S_c)) {
             w.hist = true;
             hist_S = S_h;
             fixed = hf;
