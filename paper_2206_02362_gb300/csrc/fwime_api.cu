@@ -72,6 +72,7 @@ struct fwime_ctx {
         size_t bytes = 0;
         bool valid = false, hist = false;
         const float *v = nullptr, *w = nullptr;
+        const float *hv = nullptr, *hw = nullptr;   // with host I/O: the caller's own (v and w are the staged copies)
         int K = 0, seg = 0;             // segment length of the states; the default one (seg_K) when they were written
     } bg;
     bool bg_written = false;        // set by the last enqueued B / B~ that filled the cache
@@ -1703,6 +1704,7 @@ struct Call {
     float *out;
     int accumulate;
     float eps;
+    const float *hv = nullptr, *hw = nullptr;   // host I/O: the caller's v and w
 };
 
 // internal operators of the split gradient (never passed through the C ABI)
@@ -1717,7 +1719,7 @@ static bool bg_applies(const fwime_ctx *x, int op) { return !(x->opt_tlag > 0 &&
 static bool bg_usable(const fwime_ctx *x, const Call &c)
 {
     return is_bg_reader(c.op) && bg_applies(x, c.op) && x->opt_reuse_bg && x->bg.valid && x->bg.v == c.v &&
-           x->bg.w == c.w && x->bg.seg == seg_K(x) && x->bg.buf;
+           x->bg.w == c.w && x->bg.hv == c.hv && x->bg.hw == c.hw && x->bg.seg == seg_K(x) && x->bg.buf;
 }
 
 // host-side bookkeeping once a call has been enqueued (directly or as a graph replay)
@@ -1725,7 +1727,7 @@ static void bg_after(fwime_ctx *x, const Call &c, const Reuse &u)
 {
     if (is_bg_writer(c.op)) {
         x->bg.valid = u.write && bg_applies(x, c.op);
-        x->bg.v = c.v; x->bg.w = c.w; x->bg.K = u.K; x->bg.seg = seg_K(x);
+        x->bg.v = c.v; x->bg.w = c.w; x->bg.hv = c.hv; x->bg.hw = c.hw; x->bg.K = u.K; x->bg.seg = seg_K(x);
     } else if (!is_bg_reader(c.op)) {
         x->bg.valid = false;
     }
@@ -1866,6 +1868,8 @@ static int call_op(fwime_ctx *x, Call c, int kin1, int kin2, int kout)
     NOT_SERVER(x);
     if (!c.v || !c.w || (!c.out && c.op != FWIME_OP_OBJECTIVE)) return fail(x, FWIME_EINVAL, "null pointer argument");
     if (!x->opt_host_io) return run_call(x, c);
+    c.hv = c.v;
+    c.hw = c.w;
     // the staged v and w sit at the start of the arena: a B~* can reuse the background of the B~ before it
     // (FWIME_OPT_REUSE_BACKGROUND) when the arena has not moved in between
     auto staged = [&](Call s) {

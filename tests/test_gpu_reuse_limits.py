@@ -118,3 +118,30 @@ def test_the_cap_holds_a_kept_history_and_the_workspace(planes):
             assert float(diff) <= 2e-6
             ctx.gradient(v, w, pt, d, torch.zeros_like(v))
             assert before - free() <= planes * field + (64 << 20)
+
+
+@pytest.mark.parametrize("change", ["v", "w"])
+@pytest.mark.parametrize("reader", ["born_adj", "born_ext_adj"])
+def test_host_pointers_tell_models_and_wavelets_apart(change, reader):
+    """With host I/O every model is staged at one address: the caller's pointers decide whether the background is of
+    the same v and w."""
+    grid, geom, t, _ = problem(131, 5)
+    a = {k: q.cpu().numpy() for k, q in t.items()}
+    b = dict(a)
+    b[change] = (a[change] * np.float32(1.05)).copy()
+
+    def run(ctx, x):
+        out = np.full(a["pt"].shape if reader == "born_ext_adj" else a["v"].shape, 7.0, np.float32)
+        getattr(ctx, reader)(x["v"], x["w"], x["d"], out)
+        return out.astype(np.float64)
+
+    with fw.Context(grid, geom, host_io=1) as ctx:
+        own = [run(ctx, a), run(ctx, b)]
+    with fw.Context(grid, geom, host_io=1, reuse_background=1) as ctx:
+        for _ in range(2):                     # the first writer may find the staging not yet in place
+            ctx.born_ext(a["v"], a["w"], a["pt"], np.zeros_like(a["d"]))
+            close(run(ctx, b), own[1], 2e-6)
+            assert ctx.get_option("background_reused") == 0
+        ctx.born_ext(a["v"], a["w"], a["pt"], np.zeros_like(a["d"]))
+        close(run(ctx, a), own[0], 2e-6)
+        assert ctx.get_option("background_reused") == 1
