@@ -1757,7 +1757,9 @@ static int plan_call(fwime_ctx *x, const Call &c, Reuse &u, WS &w)
     return FWIME_OK;
 }
 
-static int enqueue(fwime_ctx *x, const Call &c, Reuse &u)
+// planned: the call's plan where its caller has made it (captures; host I/O, whose staged inputs sit in the arena): the
+// arena stays as it is.
+static int enqueue(fwime_ctx *x, const Call &c, Reuse &u, const WS *planned = nullptr)
 {
     Run r;
     x->bg_used = x->bg_written = false;
@@ -1772,7 +1774,8 @@ static int enqueue(fwime_ctx *x, const Call &c, Reuse &u)
         return run_tomo_adj(x, r, 1, c.v, c.w, c.in1, c.in2, c.out, c.accumulate, c.eps,
                             c.op == OP_GRAD_FWD ? PH_FORWARD : PH_BACKWARD);
     }
-    TRY(plan_call(x, c, u, r.w));
+    if (planned) r.w = *planned;
+    else TRY(plan_call(x, c, u, r.w));
     x->bg_used = u.read;
     x->bg_written = u.write;
     if (u.write) x->bg.valid = false;   // being overwritten
@@ -1836,7 +1839,7 @@ static int run_call(fwime_ctx *x, const Call &c)
         CK(cudaStreamBeginCapture(x->st, cudaStreamCaptureModeThreadLocal));
         x->capturing = true;
         x->launches = 0;
-        int rc = enqueue(x, c, u);
+        int rc = enqueue(x, c, u, &w);
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamEndCapture(x->st, &graph);
         x->capturing = false;
@@ -1877,13 +1880,13 @@ static int call_op(fwime_ctx *x, Call c, int kin1, int kin2, int kout)
         s.w = reinterpret_cast<const float *>(x->ws) + al((size_t)x->g.nz * x->g.nx);
         return s;
     };
-    Reuse u;
-    if (x->ws) u = reuse_of(x, staged(c));
+    Reuse u = reuse_of(x, x->ws ? staged(c) : c);
     WS w;
     TRY(plan_call(x, c, u, w));
     if (u.read && !bg_usable(x, staged(c))) {   // the arena moved
+        bg_yield(x);
         u = Reuse{};
-        TRY(plan(x, c.op, w));
+        TRY(plan_call(x, c, u, w));
     }
     const size_t nm = (size_t)x->g.nz * x->g.nx, nd = (size_t)x->nshot * x->g.nt * x->nrec;
     auto count = [&](int k) -> size_t {
@@ -1902,7 +1905,8 @@ static int call_op(fwime_ctx *x, Call c, int kin1, int kin2, int kout)
     float *user_out = c.out;
     c.v = w.sv; c.w = w.sw; c.in1 = in1; c.in2 = in2; c.out = out;
     x->launches = 0;
-    TRY(enqueue_noted(x, c));
+    TRY(enqueue(x, c, u, &w));
+    bg_after(x, c, u);
     if (kout != K_NONE) CK(cudaMemcpyAsync(user_out, out, count(kout) * sizeof(float), cudaMemcpyDeviceToHost, x->st));
     return fwime_sync(x);
 }

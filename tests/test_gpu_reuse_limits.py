@@ -145,3 +145,22 @@ def test_host_pointers_tell_models_and_wavelets_apart(change, reader):
         ctx.born_ext(a["v"], a["w"], a["pt"], np.zeros_like(a["d"]))
         close(run(ctx, a), own[0], 2e-6)
         assert ctx.get_option("background_reused") == 1
+
+
+@pytest.mark.parametrize("planes", [150, 300, 420, 600])
+@pytest.mark.parametrize("writer", ["born", "born_ext"])
+@pytest.mark.parametrize("reader", ["born_adj", "born_ext_adj"])
+def test_staged_inputs_stay_in_place_under_a_cap(planes, writer, reader):
+    """Host I/O: the adjoint's plan may move the arena, and what was kept may be given back for it; the call then runs
+    on the inputs that it staged."""
+    grid, geom, t, ref = problem(131, 41)
+    a = {k: q.cpu().numpy() for k, q in t.items()}
+    staging = 4 * (2 * 41 * NZ * NX + 4 * 131 * 30)
+    with fw.Context(grid, geom, host_io=1, max_workspace_bytes=planes * PLANE + staging, reuse_background=1) as ctx:
+        for _ in range(2):
+            dout = np.full_like(a["d"], 7.0)
+            getattr(ctx, writer)(a["v"], a["w"], a["pt" if writer == "born_ext" else "dv"], dout)
+            assert np.isfinite(dout).all() and np.abs(dout).max() > 0
+            out = np.full(a["pt"].shape if reader == "born_ext_adj" else a["v"].shape, 7.0, np.float32)
+            getattr(ctx, reader)(a["v"], a["w"], a["d"], out)
+            close(out.astype(np.float64), ref[reader], 1e-4)
