@@ -25,11 +25,21 @@ namespace fwk {
 // the warp's index in its CTA, as a value that is known to be the same in all its lanes
 __device__ __forceinline__ int warp_in_cta() { return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0); }
 __device__ __forceinline__ float4 f4zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-// Read-only loads: of what no launch in flight writes (model, tables, receivers).  The wavefields are read by plain
+// Read-only loads: of what no launch in flight writes (model, tables, receivers).  The wavefields are read by ordinary
 // loads through plain pointers: a launch comes in while the one before still writes them, and what is read as read-only
 // may be fetched before the wait, or from a cache that holds an older step's rows.
 __device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
-__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+// a wavefield's row: from L2, as the copies, and not before what stands before it (plain loads through L1 took 0.7 to
+// 1.2 % more of a small grid's step)
+__device__ __forceinline__ float4 ldcg4(const float *p)
+{
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
 __device__ __forceinline__ void st4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
 __device__ __forceinline__ float cmp(const float4 &v, int j)
 {
@@ -67,7 +77,7 @@ __device__ __forceinline__ float4 lds4(const float *p) { return *reinterpret_cas
 // q^{n-1} and c; with local sources rings of three rows of those, of q^{n-1} and of c.  Nine is the period of the
 // unrolled register queue, so every slot is a compile-time constant.  Row z waits for the copy group issued four rows
 // (with local sources three) earlier.  With slots and addresses computed per row and lane a row of 128 points took 211
-// instructions in 124 registers, now 139 (one local source) in 103 to 116: 350 x 1700 points, 8 shots, 15.8 / 13.9 us
+// instructions in 124 registers, now 139 (one local source) in 102 to 116: 350 x 1700 points, 8 shots, 15.8 / 13.9 us
 // per step; from about 16 shots on the kernel is bound by memory and the two are equal.
 constexpr int RING = 9, LRING = 3;
 // Variants k_prop<LOC, D2, SRC>: LOC = 0 no dense local source, 1 exactly one (f0, weight a0), 2 the
@@ -337,7 +347,7 @@ __device__ __forceinline__ void prop_body(const PropArgs &a, const int wid, cons
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const float *qp = cur + (long long)(k - 4) * NXP + oX;
-        q[k] = xin ? ld4(qp) : f4zero();
+        q[k] = xin ? ldcg4(qp) : f4zero();
     }
     // prologue: one group per row of look-ahead (rows z0 .. z0+3 feed the first x-taps)
     constexpr int DEPTH = LOCAL ? LRING : 4;

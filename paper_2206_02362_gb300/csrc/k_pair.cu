@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_MINB) k_prop_pair(const 
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const int zr = y0 + (k - 4) * dz;
-        q[k] = xin && zr >= 0 && zr < a.NZ ? ld4(cur + (k - 4) * NX + oX) : f4zero();
+        q[k] = xin && zr >= 0 && zr < a.NZ ? ldcg4(cur + (k - 4) * NX + oX) : f4zero();
         p[k] = f4zero();
     }
 #pragma unroll

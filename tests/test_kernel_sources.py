@@ -1,5 +1,5 @@
 """What holds for kernels that come in while the launch before them still runs (griddepcontrol.wait), checked on their
-source: the wavefields, which that launch writes, are read by plain loads through plain pointers.  A read-only load
+source: the wavefields, which that launch writes, are read by ordinary loads through plain pointers.  A read-only load
 (__ldg, ldg4, a const __restrict__ pointer) may be moved before the wait or be served from a cache that was filled
 before it, and no test of the results could be relied on to show it."""
 import glob
